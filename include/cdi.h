@@ -436,7 +436,10 @@ enum { CDI_KERNEL_FORWARD = 0, CDI_KERNEL_ADJOINT = 1 };
 /* Choose the launch configuration of a kernel of this grid (not part of the
  * paper: a performance control).  Forward tiles: 0..3 one cell per thread
  * (32x8, 32x16, 64x8, 32x4 cells), 4 and 5 sixteen-byte vectors per thread
- * (16x16 and 16x8 threads; need nx % (16/sizeof(element)) == 0); tile < 0
+ * (FP32 64x14 and 64x6 cells, FP64 32x16 and 32x8; need nx %
+ * (16/sizeof(element)) == 0), 6 the same with tensor-map copies (nx % 64 == 0
+ * (FP32) or 32 (FP64), ny % 16 == 0), 7 and 8 vectors per thread for any nx (16
+ * vectors by 14 and 6 rows, copied and stored element by element); tile < 0
  * restores the default.  blocks_per_sm <= 0 fills the GPU.  Forward work
  * split: nchunks >= 1 cuts every tile column into that many z chunks, taken
  * round-robin by the persistent blocks; CDI_NCHUNKS_BALANCED gives every block

@@ -32,7 +32,7 @@ CDI_NCHUNKS_ROTATED = -2    # near-equal shares (column starts weighted), column
                             # neighbouring tiles share their halo rows in L2
 CDI_SHARPEN_CENTRE, CDI_SHARPEN_FACE = 0, 1
 SHARPEN = {"centre": CDI_SHARPEN_CENTRE, "face": CDI_SHARPEN_FACE}
-FWD_TILES = 7
+FWD_TILES = 9
 ADJ_TILES = 4
 BATCH_TILES = 7
 

@@ -202,10 +202,7 @@ static int fwd_cfg_rk(const cdi_grid *g, int tile, LaunchCfg *c) { return fwd_cf
 
 static int default_fwd_tile(const cdi_grid *g)
 {
-    if (g->sharpen == CDI_SHARPEN_FACE) return 0;
-    const int vx = 16 / (int)esize(g);
-    if (g->nx % vx == 0 && g->nx >= 48) return g->ny >= 12 ? 4 : 5;
-    return (g->nx >= 32 && g->ny >= 16) ? 1 : 3;
+    return g->sharpen == CDI_SHARPEN_FACE ? 0 : cdi::fwd_default_tile((int)esize(g), g->nx, g->ny);
 }
 
 // Vector adjoint: z chunking from the forward cost model (rounds of the
@@ -544,7 +541,7 @@ static int step_t(cdi_grid *g, const void *in, void *out, double dt, double eps,
     a.out = (T *)out;
     a.u = (const T *)g->u;
     a.v = (const T *)(g->v ? g->v : g->u);  // ny == nz == 1: v is inert
-    a.w = (const T *)(g->w ? g->w : g->u);  // nz == 1: w is inert
+    a.w = (const T *)(g->nz > 1 ? g->w : g->u);  // nz == 1: w is inert (its two faces are one)
     a.nx = g->nx; a.ny = g->ny; a.nz = g->nz;
     a.z_lo = z_lo;
     a.z_hi = z_hi;
@@ -660,8 +657,8 @@ static int step2_t(cdi_grid *g, const void *in, void *out, double dt, double eps
 
 // One Runge-Kutta stage: evaluates r = dt * RHS(in) and writes
 //   out = (base ? base : in) + alpha r + (q ? delta q : 0),  qout = mu (q ? q : in) + beta r.
-// Uses the RK variant of the configured tile's kernel family (vector 16x16, or
-// the scalar 32x16 / 32x4 tile).
+// Uses the RK variant of the configured tile's kernel family (vectors, aligned rows
+// or any; or the one-cell-per-thread 32x16 / 32x4 tile).
 struct RkStage {
     const void *in, *base, *q;
     void *out, *qout;
@@ -673,7 +670,7 @@ template <typename T>
 static int rk_stage_t(cdi_grid *g, const RkStage &st, double dt, double eps, double gamma, cudaStream_t s)
 {
     if (g->rk.nblocks == 0) {  // first use: RK launch configuration for this grid
-        int tile = cdi::fwd_tile_is_vec(g->fwd.tile) ? 4 : ((g->nx >= 32 && g->ny >= 16) ? 1 : 3);
+        const int tile = g->fwd.tile >= 7 ? 7 : g->fwd.tile >= 4 ? 4 : (g->nx >= 32 && g->ny >= 16) ? 1 : 3;
         if (int rc = fwd_cfg_rk(g, tile, &g->rk)) return rc;
     }
     cdi::FwdArgs<T> a;
@@ -914,11 +911,11 @@ int cdi_mass_and_bounds(cdi_grid *g, const void *phi, cdi_stats *out, void *stre
 }
 
 // Launch configuration of the z-range kernels (the slabs of the pipelined host
-// step, cdi_step_planes): tile 4 where nx allows, else 0; balanced shares.
+// step, cdi_step_planes): tile 4 where nx allows, else 7; balanced shares.
 static int ensure_slab_cfg(cdi_grid *g)
 {
     if (g->slab.nblocks != 0) return CDI_OK;
-    const int tile = g->nx % (16 / (int)esize(g)) == 0 ? 4 : 0;
+    const int tile = g->nx % (16 / (int)esize(g)) == 0 ? 4 : 7;
     return fwd_cfg(g, tile, 0, CDI_NCHUNKS_BALANCED, &g->slab, false, true);
 }
 
@@ -1370,7 +1367,9 @@ int cdi_autotune(cdi_grid *g, void *phi_a, void *phi_b, double dt, double eps, d
     const int chunk_opts[] = {CDI_NCHUNKS_BALANCED, CDI_NCHUNKS_ROTATED, 0, 1, 2, 3, 4, 5, 6, 7, 8, 10, 12, 14,
                               16, 20, 24, 32};
     for (int tile = 0; tile < cdi::fwd_num_tiles() && rc == CDI_OK; ++tile) {
-        if (cdi::fwd_tile_is_vec(tile) && g->nx % (16 / (int)esize(g)) != 0) continue;
+        const bool al = g->nx % (16 / (int)esize(g)) == 0;
+        if (cdi::fwd_tile_is_vec(tile) && !al) continue;
+        if (tile >= 7 && al) continue;  // the same kernels with element copies
         if (g->sharpen == CDI_SHARPEN_FACE && tile != 0) continue;
         for (int oi = 0; oi < (int)(sizeof(chunk_opts) / sizeof(int)); ++oi) {
             if (chunk_opts[oi] > g->nz) continue;

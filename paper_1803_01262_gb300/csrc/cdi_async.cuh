@@ -15,6 +15,16 @@ __device__ __forceinline__ void cp_async(void *smem, const void *gmem)
         asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(s), "l"(gmem), "n"(BYTES));
 }
 
+// The same to shared address base + OFF bytes (OFF an immediate of the instruction).
+template <int BYTES, int OFF>
+__device__ __forceinline__ void cp_async_at(unsigned base, const void *gmem)
+{
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0 + %2], [%1], 16;\n" ::"r"(base), "l"(gmem), "n"(OFF));
+    else
+        asm volatile("cp.async.ca.shared.global [%0 + %3], [%1], %2;\n" ::"r"(base), "l"(gmem), "n"(BYTES), "n"(OFF));
+}
+
 __device__ __forceinline__ void cp_async_commit()
 {
     asm volatile("cp.async.commit_group;\n" ::: "memory");

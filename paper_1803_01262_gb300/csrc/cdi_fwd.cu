@@ -7,9 +7,12 @@
 //   s = phi (1 - phi) g/|g|,  g_d = phi_{c+e_d} - phi_{c-e_d}  (s = 0 where g = 0),
 //   phi'_c = phi_c - c_upd sum_d (F_{c+1/2} - F_{c-1/2}).
 //
-// Two kernels share one structure (a block owns an x-y tile and marches along
+// Three kernels share one structure (a block owns an x-y tile and marches along
 // z over a chunk of planes):
-//   fwd_vec_kernel  -- each thread owns a 16-byte vector of x-cells (4 float
+//   fwd_row_kernel  -- (cdi_fwd_row.cuh) a 16-byte vector of x-cells per thread, phi carried
+//                      in registers from plane to plane; any row length.
+//   fwd_vec_kernel  -- (FP64, whose step the FP64 pipe bounds, not shared memory: 128^3 212.7
+//                      against 235.5 us with the row kernel's shorter tile) each thread owns a 16-byte vector of x-cells (4 float
 //                      or 2 double); phi and the three face-velocity planes
 //                      are staged by 16-byte cp.async two planes ahead of use;
 //                      two extra warps compute the sharpening ring (one cell
@@ -29,6 +32,7 @@
 #include "cdi_reduce.cuh"
 #include "cdi_async.cuh"
 #include "cdi_fwd_common.cuh"
+#include "cdi_fwd_row.cuh"
 #include "cdi_fwd_scalar.cuh"
 
 namespace cdi {
@@ -389,7 +393,7 @@ fwd_vec_kernel(const FwdArgs<T> a, const int nchunks)
 // ===========================================================================
 // Scalar kernel (any extents): the per-unit body is in cdi_fwd_scalar.cuh.
 
-template <typename T, int BX, int BY, bool RK, bool FACE = false, bool ZR = false>
+template <typename T, int BX, int BY, bool RK, bool FACE = false>
 __global__ void __launch_bounds__(BX * BY)
 fwd_kernel(const FwdArgs<T> a, const int nchunks)
 {
@@ -398,30 +402,29 @@ fwd_kernel(const FwdArgs<T> a, const int nchunks)
     const int ntiles = tiles_x * ((a.ny + BY - 1) / BY);
     Acc<T> acc;
     acc.init();
-    const int zlo = ZR ? a.z_lo : 0, zr = ZR ? a.z_hi - a.z_lo : a.nz;
-    UnitIter<BX, BY> units(ntiles, zr, nchunks);
+    UnitIter<BX, BY> units(ntiles, a.nz, nchunks);
     Unit un;
-    while (units.next(un, ntiles, tiles_x, zr, nchunks)) {
-        un.z0 += zlo;
-        un.z1 += zlo;
+    while (units.next(un, ntiles, tiles_x, a.nz, nchunks)) {
         if (!RK && !FACE && a.nz == 1)
             flat_unit<T, BX, BY>(a, un, acc, smem_raw);
         else
             scalar_unit<T, BX, BY, RK, SCALAR_PF, FACE>(a, un, acc, smem_raw);
     }
-    reduce_and_finish<ZR>(acc, a.red);
+    reduce_and_finish(acc, a.red);
 }
 
 // ===========================================================================
 // Kernel table and launch
 //
-// Forward tiles: 0..3 scalar BX x BY = 32x8, 32x16, 64x8, 32x4;
-//                4, 5 vector TX x TY = 16x16, 16x8 (x width 16 * 16/sizeof(T));
-//                6 vector 16x16 with tensor-memory-accelerator staging (cdi_fwd_tma.cu).
+// Forward tiles: 0..3 one cell per thread, BX x BY = 32x8, 32x16, 64x8, 32x4;
+//                4, 5 a vector of cells per thread, rows on 16-byte boundaries: FP32 the row
+//                kernel (64x14, 64x6 cells), FP64 the vector kernel (32x16, 32x8);
+//                6 vector with tensor-memory-accelerator staging (cdi_fwd_tma.cu);
+//                7, 8 the row kernel for any row length (14 and 6 rows of 16 vectors).
 
-int fwd_num_tiles() { return 7; }
+int fwd_num_tiles() { return 9; }
 
-bool fwd_tile_is_vec(int tile) { return tile >= 4; }
+bool fwd_tile_is_vec(int tile) { return tile >= 4 && tile <= 6; }
 
 void fwd_tile_dims(int tile, int esize, int *bw, int *bh)
 {
@@ -429,10 +432,30 @@ void fwd_tile_dims(int tile, int esize, int *bw, int *bh)
     if (tile < 4) {
         *bw = sdim[tile][0];
         *bh = sdim[tile][1];
-    } else {
-        *bw = 16 * (16 / esize);
-        *bh = tile == 5 ? 8 : 16;
+        return;
     }
+    const bool row = tile >= 7 || (esize == 4 && tile != 6);  // the row kernel's heights
+    *bw = 16 * (16 / esize);
+    *bh = tile == 5 || tile == 8 ? (row ? 6 : 8) : (row ? 14 : 16);
+}
+
+// Default tile of an Euler step (centre form): a vector kernel where the box is wide enough to
+// use its 16 vectors per row (FP32 rows of 16 cells and more: one-cell-per-thread tiles cost
+// three times the instructions per lane, and waste half as many lanes at most), the 14-row tile
+// unless the 6-row one covers ny with less work (each tile row of blocks pays two ring rows),
+// else one cell per thread.  FP64, whose time is FP64 instructions, takes the vector kernel on
+// aligned rows of 48 cells and more, and the row kernel on other rows of 64 and more
+// (129^3: 306 us with the 32x16 tile, 289 us).
+int fwd_default_tile(int esize, int nx, int ny)
+{
+    const int vx = 16 / esize;
+    const bool al = nx % vx == 0;
+    if (esize == 4 ? nx >= 16 : (al ? nx >= 48 : nx >= 64)) {
+        if (esize == 8 && al) return ny >= 12 ? 4 : 5;
+        const int w14 = (ny + 13) / 14 * 16, w6 = (ny + 5) / 6 * 8;
+        return (w6 < w14 ? 5 : 4) + (al ? 0 : 3);
+    }
+    return (nx >= 32 && ny >= 16) ? 1 : 3;
 }
 
 long long fwd_tiles_xy(int tile, int esize, int nx, int ny)
@@ -450,18 +473,28 @@ static cudaError_t occ(K kernel, int threads, size_t smem, int *resident)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, kernel, threads, smem);
 }
 
-// Runge-Kutta stage kernels exist for tiles 1, 3 (scalar) and 4 (vector) only.
-bool fwd_tile_has_rk(int tile) { return tile == 1 || tile == 3 || tile == 4; }
+template <typename T, int TY, bool AL, bool RK = false, bool ZR = false>
+static cudaError_t row_occ(int *resident)
+{
+    using C = RowCfg<T, TY, RK>;
+    return occ(fwd_row_kernel<T, TY, RK, ZR, AL>, C::NT, C::bytes, resident);
+}
+
+// Runge-Kutta stage kernels exist for tiles 1, 3 (one cell per thread), 4 and 7 (vectors) only.
+bool fwd_tile_has_rk(int tile) { return tile == 1 || tile == 3 || tile == 4 || tile == 7; }
 
 template <typename T>
 cudaError_t fwd_occupancy(int tile, bool rk, int *resident, bool face, bool slab)
 {
     if (slab) {  // the z-slab kernels of the pipelined host step
         if (rk || face) return cudaErrorInvalidValue;
-        if (tile == 4)
-            return occ(fwd_vec_kernel<T, 16, 16, false, true>, VecCfg<T, 16, 16>::NT, VecCfg<T, 16, 16>::bytes,
-                       resident);
-        if (tile == 0) return occ(fwd_kernel<T, 32, 8, false, false, true>, 256, FwdSmem<T, 32, 8>::bytes, resident);
+        if (tile == 4) {
+            if constexpr (sizeof(T) == 4) return row_occ<T, 14, true, false, true>(resident);
+            else
+                return occ(fwd_vec_kernel<T, 16, 16, false, true>, VecCfg<T, 16, 16>::NT, VecCfg<T, 16, 16>::bytes,
+                           resident);
+        }
+        if (tile == 7) return row_occ<T, 14, false, false, true>(resident);
         return cudaErrorInvalidValue;
     }
     if (face) {
@@ -472,7 +505,10 @@ cudaError_t fwd_occupancy(int tile, bool rk, int *resident, bool face, bool slab
         switch (tile) {
         case 1: return occ(fwd_kernel<T, 32, 16, true>, 512, FwdSmem<T, 32, 16>::bytes, resident);
         case 3: return occ(fwd_kernel<T, 32, 4, true>, 128, FwdSmem<T, 32, 4>::bytes, resident);
-        case 4: return occ(fwd_vec_kernel<T, 16, 16, true>, VecCfg<T, 16, 16>::NT, VecCfg<T, 16, 16>::bytes, resident);
+        case 4:
+            if constexpr (sizeof(T) == 4) return row_occ<T, 14, true, true>(resident);
+            else return occ(fwd_vec_kernel<T, 16, 16, true>, VecCfg<T, 16, 16>::NT, VecCfg<T, 16, 16>::bytes, resident);
+        case 7: return row_occ<T, 14, false, true>(resident);
         default: return cudaErrorInvalidValue;
         }
     }
@@ -481,9 +517,15 @@ cudaError_t fwd_occupancy(int tile, bool rk, int *resident, bool face, bool slab
     case 1: return occ(fwd_kernel<T, 32, 16, false>, 512, FwdSmem<T, 32, 16>::bytes, resident);
     case 2: return occ(fwd_kernel<T, 64, 8, false>, 512, FwdSmem<T, 64, 8>::bytes, resident);
     case 3: return occ(fwd_kernel<T, 32, 4, false>, 128, FwdSmem<T, 32, 4>::bytes, resident);
-    case 4: return occ(fwd_vec_kernel<T, 16, 16, false>, VecCfg<T, 16, 16>::NT, VecCfg<T, 16, 16>::bytes, resident);
-    case 5: return occ(fwd_vec_kernel<T, 16, 8, false>, VecCfg<T, 16, 8>::NT, VecCfg<T, 16, 8>::bytes, resident);
+    case 4:
+        if constexpr (sizeof(T) == 4) return row_occ<T, 14, true>(resident);
+        else return occ(fwd_vec_kernel<T, 16, 16, false>, VecCfg<T, 16, 16>::NT, VecCfg<T, 16, 16>::bytes, resident);
+    case 5:
+        if constexpr (sizeof(T) == 4) return row_occ<T, 6, true>(resident);
+        else return occ(fwd_vec_kernel<T, 16, 8, false>, VecCfg<T, 16, 8>::NT, VecCfg<T, 16, 8>::bytes, resident);
     case 6: return tma_occupancy<T>(resident);
+    case 7: return row_occ<T, 14, false>(resident);
+    case 8: return row_occ<T, 6, false>(resident);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -509,20 +551,27 @@ static cudaError_t launch_dependent(K kernel, int nblocks, int threads, size_t s
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+template <typename T, int TY, bool AL, bool RK = false, bool ZR = false>
+static cudaError_t row_launch(const FwdArgs<T> &a, int nblocks, int nchunks, cudaStream_t s)
+{
+    using C = RowCfg<T, TY, RK>;
+    return launch_dependent(fwd_row_kernel<T, TY, RK, ZR, AL>, nblocks, C::NT, C::bytes, s, a, nchunks);
+}
+
 template <typename T>
 cudaError_t launch_fwd(const FwdArgs<T> &a, int tile, int nblocks, int nchunks, bool rk, cudaStream_t s,
                        bool face)
 {
-    if (a.z_hi > 0) {  // a z slab: tile 4 (vector) or 0 (any extents), centre form, Euler
+    if (a.z_hi > 0) {  // a z slab: tile 4 (aligned rows) or 7 (any), centre form, Euler
         if (rk || face) return cudaErrorInvalidValue;
-        if (tile == 4)
-            fwd_vec_kernel<T, 16, 16, false, true>
-                <<<nblocks, VecCfg<T, 16, 16>::NT, VecCfg<T, 16, 16>::bytes, s>>>(a, nchunks);
-        else if (tile == 0)
-            fwd_kernel<T, 32, 8, false, false, true><<<nblocks, dim3(32, 8), FwdSmem<T, 32, 8>::bytes, s>>>(a, nchunks);
-        else
-            return cudaErrorInvalidValue;
-        return cudaGetLastError();
+        if (tile == 4) {
+            if constexpr (sizeof(T) == 4) return row_launch<T, 14, true, false, true>(a, nblocks, nchunks, s);
+            else
+                return launch_dependent(fwd_vec_kernel<T, 16, 16, false, true>, nblocks, VecCfg<T, 16, 16>::NT,
+                                        VecCfg<T, 16, 16>::bytes, s, a, nchunks);
+        }
+        if (tile == 7) return row_launch<T, 14, false, false, true>(a, nblocks, nchunks, s);
+        return cudaErrorInvalidValue;
     }
     if (face) {  // face-product sharpening: tile 0 only, Euler only
         if (rk || tile != 0) return cudaErrorInvalidValue;
@@ -534,8 +583,11 @@ cudaError_t launch_fwd(const FwdArgs<T> &a, int tile, int nblocks, int nchunks, 
         case 1: fwd_kernel<T, 32, 16, true><<<nblocks, dim3(32, 16), FwdSmem<T, 32, 16>::bytes, s>>>(a, nchunks); break;
         case 3: fwd_kernel<T, 32, 4, true><<<nblocks, dim3(32, 4), FwdSmem<T, 32, 4>::bytes, s>>>(a, nchunks); break;
         case 4:
-            fwd_vec_kernel<T, 16, 16, true><<<nblocks, VecCfg<T, 16, 16>::NT, VecCfg<T, 16, 16>::bytes, s>>>(a, nchunks);
-            break;
+            if constexpr (sizeof(T) == 4) return row_launch<T, 14, true, true>(a, nblocks, nchunks, s);
+            else
+                return launch_dependent(fwd_vec_kernel<T, 16, 16, true>, nblocks, VecCfg<T, 16, 16>::NT,
+                                        VecCfg<T, 16, 16>::bytes, s, a, nchunks);
+        case 7: return row_launch<T, 14, false, true>(a, nblocks, nchunks, s);
         default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
@@ -546,12 +598,18 @@ cudaError_t launch_fwd(const FwdArgs<T> &a, int tile, int nblocks, int nchunks, 
     case 2: fwd_kernel<T, 64, 8, false><<<nblocks, dim3(64, 8), FwdSmem<T, 64, 8>::bytes, s>>>(a, nchunks); break;
     case 3: fwd_kernel<T, 32, 4, false><<<nblocks, dim3(32, 4), FwdSmem<T, 32, 4>::bytes, s>>>(a, nchunks); break;
     case 4:
-        return launch_dependent(fwd_vec_kernel<T, 16, 16, false>, nblocks, VecCfg<T, 16, 16>::NT,
-                                VecCfg<T, 16, 16>::bytes, s, a, nchunks);
+        if constexpr (sizeof(T) == 4) return row_launch<T, 14, true>(a, nblocks, nchunks, s);
+        else
+            return launch_dependent(fwd_vec_kernel<T, 16, 16, false>, nblocks, VecCfg<T, 16, 16>::NT,
+                                    VecCfg<T, 16, 16>::bytes, s, a, nchunks);
     case 5:
-        return launch_dependent(fwd_vec_kernel<T, 16, 8, false>, nblocks, VecCfg<T, 16, 8>::NT,
-                                VecCfg<T, 16, 8>::bytes, s, a, nchunks);
+        if constexpr (sizeof(T) == 4) return row_launch<T, 6, true>(a, nblocks, nchunks, s);
+        else
+            return launch_dependent(fwd_vec_kernel<T, 16, 8, false>, nblocks, VecCfg<T, 16, 8>::NT,
+                                    VecCfg<T, 16, 8>::bytes, s, a, nchunks);
     case 6: return launch_fwd_tma<T>(a, nblocks, nchunks, s);
+    case 7: return row_launch<T, 14, false>(a, nblocks, nchunks, s);
+    case 8: return row_launch<T, 6, false>(a, nblocks, nchunks, s);
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

@@ -79,7 +79,7 @@ struct FwdArgs {
     T *rk_qout;
     T rk_alpha, rk_delta, rk_mu, rk_beta;
     int z_lo = 0, z_hi = 0;  // z_hi > 0: only planes [z_lo, z_hi) are updated (forward
-                             // tiles 0 and 4, the slabs of a pipelined host step)
+                             // tiles 4 and 7, the slabs of a pipelined host step)
 };
 
 template <typename T>
@@ -108,7 +108,8 @@ struct LaunchCfg {
 };
 
 int fwd_num_tiles();
-bool fwd_tile_is_vec(int tile);
+bool fwd_tile_is_vec(int tile);  // tiles that need rows on 16-byte boundaries
+int fwd_default_tile(int esize, int nx, int ny);
 void fwd_tile_dims(int tile, int esize, int *bw, int *bh);
 long long fwd_tiles_xy(int tile, int esize, int nx, int ny);
 

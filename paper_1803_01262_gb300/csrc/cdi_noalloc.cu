@@ -97,10 +97,7 @@ static int noalloc_t(int nx, int ny, int nz, double dx, const void *in, void *ou
                      void *stats_dev, NoAllocScratch *scr, int sms, cudaStream_t s)
 {
     const int es = (int)sizeof(T);
-    const int vx = 16 / es;
-    int tile;
-    if (nx % vx == 0 && nx >= 48) tile = ny >= 12 ? 4 : 5;
-    else tile = (nx >= 32 && ny >= 16) ? 1 : 3;
+    const int tile = cdi::fwd_default_tile(es, nx, ny);
     int resident = 0;
     cudaError_t e = cdi::fwd_occupancy<T>(tile, false, &resident);
     if (e != cudaSuccess) return na_fail(CDI_ERR_CUDA, "occupancy query", e);
@@ -120,7 +117,7 @@ static int noalloc_t(int nx, int ny, int nz, double dx, const void *in, void *ou
     a.out = (T *)out;
     a.u = (const T *)u;
     a.v = (const T *)(v ? v : u);
-    a.w = (const T *)(w ? w : u);
+    a.w = (const T *)(nz > 1 ? w : u);  // nz == 1: w is inert
     a.nx = nx; a.ny = ny; a.nz = nz;
     a.c.c_adv = (T)(0.5 * vs);
     a.c.c_dif = (T)(gamma * eps / dx);
