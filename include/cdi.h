@@ -446,8 +446,9 @@ enum { CDI_KERNEL_FORWARD = 0, CDI_KERNEL_ADJOINT = 1 };
  * an equal contiguous share of the tile-planes (tile-major, cut at column
  * ends), CDI_NCHUNKS_ROTATED the same shares with rotated columns; 0 picks
  * chunks or CDI_NCHUNKS_ROTATED from a cost model.  Adjoint
- * tiles: 0..2 (32x8, 32x16, 32x4 cells) and 3 (vector), nchunks sets the z
- * chunking (CDI_NCHUNKS_BALANCED / CDI_NCHUNKS_ROTATED: balanced shares, tile 3
+ * tiles: 0..2 (32x8, 32x16, 32x4 cells), 3 (vectors, nx % (16/sizeof(element))
+ * == 0) and 4 (vectors, any nx), nchunks sets the z chunking
+ * (CDI_NCHUNKS_BALANCED / CDI_NCHUNKS_ROTATED: balanced shares, tiles 3 and 4
  * only; the vector adjoint's default takes the rotated shares where the cost
  * model favours balanced ones).  Every forward configuration (and the batch
  * and two-steps-per-pass paths) computes the same field bit for bit; the

@@ -33,7 +33,7 @@ CDI_NCHUNKS_ROTATED = -2    # near-equal shares (column starts weighted), column
 CDI_SHARPEN_CENTRE, CDI_SHARPEN_FACE = 0, 1
 SHARPEN = {"centre": CDI_SHARPEN_CENTRE, "face": CDI_SHARPEN_FACE}
 FWD_TILES = 9
-ADJ_TILES = 4
+ADJ_TILES = 5
 BATCH_TILES = 7
 
 _ERRNAMES = {-1: "CDI_ERR_ARG", -2: "CDI_ERR_DIM", -3: "CDI_ERR_CUDA", -4: "CDI_ERR_CONDITION",

@@ -239,14 +239,15 @@ static int adj_vec_zchunk(const cdi_grid *g)
 
 static bool adj_vec_eligible(const cdi_grid *g) { return g->nx % (16 / (int)esize(g)) == 0; }
 
-// Adjoint launch: the vector kernel where nx allows it (and the box is wide enough
-// for its 16-byte tiles); else a one-cell-per-thread tile with a z chunk giving
-// about eight blocks per SM.
+// Adjoint launch: the row kernel (tile 3 where rows start on 16-byte boundaries, else 4) for
+// rows of 16 cells and more, as the forward step (fwd_default_tile; FP64 too: its formulas take
+// fewer FP64 operations); else a one-cell-per-thread tile with a z chunk giving about eight
+// blocks per SM.
 static LaunchCfg adj_default(const cdi_grid *g)
 {
     LaunchCfg c;
-    if (adj_vec_eligible(g) && g->nx >= 48) {
-        c.tile = 3;
+    if (g->nx >= 16) {
+        c.tile = adj_vec_eligible(g) ? 3 : 4;
         c.zchunk = adj_vec_zchunk(g);
         c.nblocks = 0;
         c.nchunks = 0;
@@ -1137,7 +1138,7 @@ int cdi_set_launch(cdi_grid *g, int which, int tile, int blocks_per_sm, int nchu
             return CDI_OK;
         }
         if (tile >= cdi::adj_num_tiles()) return fail(CDI_ERR_ARG, "adjoint tile %d out of range", tile);
-        if (cdi::adj_tile_is_vec(tile) && !adj_vec_eligible(g))
+        if (tile == 3 && !adj_vec_eligible(g))
             return fail(CDI_ERR_ARG, "vector adjoint tile needs nx %% %d == 0", 16 / (int)esize(g));
         LaunchCfg c = adj_default(g);
         if (cdi::adj_tile_is_vec(tile) && !cdi::adj_tile_is_vec(c.tile)) c.zchunk = adj_vec_zchunk(g);

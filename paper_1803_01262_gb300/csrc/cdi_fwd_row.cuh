@@ -28,38 +28,21 @@
 // same bit for bit.
 #pragma once
 
-#include <type_traits>
-
 #include "cdi_async.cuh"
 #include "cdi_fwd_common.cuh"
 #include "cdi_reduce.cuh"
+#include "cdi_row.cuh"
 
 namespace cdi {
 
-template <int V>
-using IC = std::integral_constant<int, V>;
-
 template <typename T, int TY, bool RK = false>
-struct RowCfg {
-    static constexpr int VX = 16 / sizeof(T), TX = 16;
-    static constexpr int W = TX * VX, H = TY;
-    static constexpr int NOWN = TX * TY;
-    static constexpr int NT = NOWN + 32;      // + the ring warp
-    static constexpr int NJ = W / 32;         // a lane's columns of a row
-    static constexpr int PP = W + 2 * VX;     // row pitch of every staged array: x0-VX .. x0+W+VX-1
-    static constexpr int NS = 4;              // ring slots of phi and of the velocities
-    static constexpr int PHI = (H + 4) * PP;  // phi rows y0-2 .. y0+H+1
-    static constexpr int VO = H * PP;         // u rows y0 .. at 0; v rows y0-1 ..; w rows y0 ..
-    static constexpr int WO = VO + (H + 1) * PP;
-    static constexpr int VEL = WO + H * PP;
-    static constexpr int SXS = H * PP;        // s_x, columns -1 .. W
-    static constexpr int SYS = (H + 2) * PP;  // s_y, rows -1 .. H
-    static constexpr int OVEL = NS * PHI, OSX = OVEL + NS * VEL, OSY = OSX + 2 * SXS;
-    static constexpr int RKO = H * W;         // a plane of one Runge-Kutta operand (RK: two operands, two slots)
-    static constexpr int ORK = OSY + 2 * SYS;
+struct RowCfg : RowGeo<T, TY> {
+    using G = RowGeo<T, TY>;
+    static constexpr int OVEL = G::NS * G::PHI, OSX = OVEL + G::NS * G::VEL, OSY = OSX + 2 * G::SXS;
+    static constexpr int RKO = G::H * G::W;   // a plane of one Runge-Kutta operand (RK: two operands, two slots)
+    static constexpr int ORK = OSY + 2 * G::SYS;
     static constexpr size_t bytes = sizeof(T) * (size_t)(ORK + (RK ? 4 * RKO : 0));
-    static_assert(TY % 2 == 0 && TY <= 16, "two rows per own warp, at most 32 ring cells");
-    static_assert(VEL >= PHI, "the prologue's first phi plane borrows a velocity slot");
+    static_assert(G::VEL >= G::PHI, "the prologue's first phi plane borrows a velocity slot");
 };
 
 template <typename T, int TY, bool RK, bool ZR, bool AL>
@@ -68,7 +51,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
 {
     using C = RowCfg<T, TY, RK>;
     using VV = V16<T>;
-    constexpr int VX = C::VX, W = C::W, H = C::H, PP = C::PP, NJ = C::NJ, TX = C::TX, ES = sizeof(T);
+    constexpr int VX = C::VX, W = C::W, H = C::H, PP = C::PP, TX = C::TX;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *const sm = reinterpret_cast<T *>(smem_raw);
 
@@ -85,16 +68,13 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
     const int lane = tid & 31, tx = tid % TX;
     // the row of this thread's group: own 0..H-1; the ring warp's -1 and H
     const int ty = is_own ? tid / TX : (lane < TX ? -1 : H);
-    const int r0 = ty & ~1;                // own warp: its first row
     const bool has_xr = (lane & 15) < TY;  // ring warp: an x-ring cell, row lane & 15, left or right
     // the group's place: phi row ty + d of slot S at bp[S PHI + (1 + d) PP], u / w row ty at
     // bp[.. - PP], v row ty at bp[.. + VO] (row ty - 1 one pitch below), s_x row ty at
     // bp[.. - PP], s_y row ty at bp[..]; xb: the same for the x-ring cell
     T *const bp = sm + (ty + 1) * PP + VX + tx * VX;
     T *const xb = sm + ((lane & 15) + 1) * PP + VX + (lane < 16 ? -1 : W);
-    // base shared address of the copies: own threads, AL: bp; else column `lane` of the warp's
-    // first row (ring warp: of row 0)
-    const unsigned cb = smem_addr(AL ? bp : sm + (is_own ? r0 * PP : 0) + VX + lane);
+    RowStage<T, TY, AL> cp(sm, tid, ty, tx);
 
     // Sharpening of the group's cells c, from its y neighbours, the planes below (zn) and
     // above (zp) and the x neighbours L, R.
@@ -123,8 +103,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
         return p * (T(1) - p) * inv * g0;
     };
 
-    // base shared address of this thread's Runge-Kutta operand copies
-    const unsigned rkb = smem_addr(sm + (AL ? ty * W + tx * VX : r0 * W + lane));
+    const unsigned rkb = cp.own_base(sm, ty, tx);
     (void)rkb;
 
     Acc<T> acc;
@@ -137,168 +116,17 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
     while (units.next(un, ntiles, tiles_x, zr, nchunks)) {
         const int x0 = un.x0, y0 = un.y0, z0 = un.z0 + zlo, z1 = un.z1 + zlo;
 
-        // In-plane offsets of this thread's copies.  Own threads, AL: g[0] the own vector; else
-        // g[r NJ + j] column lane + 32 j of row r0 + r.  Ring warp, AL: g[0..2] vectors of phi
-        // (rows -1 and H with their x halos, rows -2 and H+1, the x halos of rows 0..H-1), g[3]
-        // the x halo of u (lanes < H) and v row -1 (16 lanes); d[] their places.  Else g[r NJ + j]
-        // the phi rows -2, -1, H, H+1, gv[j] v row -1, gh[0..1] / d[0..1] single phi cells
-        // (columns -1 and W of rows -1 and H; columns -2, -1, W, W+1 of rows 0..H-1), gh[2] u
-        // column -1.
-        constexpr int NG = AL ? 4 : 4 * NJ;
-        int g[NG], gh[3], gv[NJ];
-        unsigned d[4];        // shared byte addresses of the ring warp's single places
-        bool hx2 = false;     // ring warp, AL: its third phi vector exists
-        auto at = [&](int y, int x, int len) {  // wrapped in-plane offset (len elements long)
-            return (int)CDI_CHK(wrapi(y, ny) * nx + wrapi(x, nx), plane - len + 1, st);
-        };
-        if (is_own) {
-            if constexpr (AL) {
-                g[0] = at(y0 + ty, x0 + tx * VX, VX);
-            } else {
-#pragma unroll
-                for (int r = 0; r < 2; ++r)
-#pragma unroll
-                    for (int j = 0; j < NJ; ++j) g[r * NJ + j] = at(y0 + r0 + r, x0 + lane + 32 * j, 1);
-            }
-        } else if constexpr (AL) {
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                int e = lane + 32 * i, row, col;  // col: vector column -1 .. 16
-                if (e < 36) {
-                    row = e < 18 ? -1 : H;
-                    col = e % 18 - 1;
-                } else if (e < 68) {
-                    e -= 36;
-                    row = e < 16 ? -2 : H + 1;
-                    col = e & 15;
-                } else {
-                    e -= 68;  // (rows past H - 1, for TY < 14: a row the tile stages anyway, not copied)
-                    row = e >> 1;
-                    col = (e & 1) ? 16 : -1;
-                }
-                g[i] = at(y0 + row, x0 + col * VX, VX);
-                hx2 = lane + 32 * i < 68 || row < H;
-                d[i] = smem_addr(sm + (hx2 ? (row + 2) * PP + VX + col * VX : 0));
-            }
-            const bool isu = lane < H;
-            g[3] = isu ? at(y0 + lane, x0 - VX, VX) : at(y0 - 1, x0 + ((lane - H) & 15) * VX, VX);
-            d[3] = smem_addr(sm + (isu ? lane * PP : C::VO + VX + ((lane - H) & 15) * VX));
-        } else {
-#pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-                for (int j = 0; j < NJ; ++j)
-                    g[r * NJ + j] = at(y0 + (r < 2 ? r - 2 : H + r - 2), x0 + lane + 32 * j, 1);
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) gv[j] = at(y0 - 1, x0 + lane + 32 * j, 1);
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {  // 4 H + 4 <= 64 cells
-                const int e = lane + 32 * i - 4;
-                const int row = e < 0 ? (e & 2 ? H : -1) : e >> 2, q = e & 3;
-                const int col = e < 0 ? (e & 1 ? W : -1) : q < 2 ? q - 2 : W + q - 2;
-                gh[i] = at(y0 + row, x0 + col, 1);
-                d[i] = smem_addr(sm + (e < 4 * H ? (row + 2) * PP + VX + col : 0));
-            }
-            gh[2] = at(y0 + (lane < H ? lane : 0), x0 - 1, 1);
-            d[2] = smem_addr(sm + (lane < H ? lane : 0) * PP + VX - 1);
-        }
-        // phi plane at src (its first element) to the slot at element offset SO
-        auto issue_phi = [&](const T *src, auto SO) {
-            constexpr int so = decltype(SO)::value * ES;
-            if (is_own) {
-                if constexpr (AL) {
-                    cp_async_at<16, so + PP * ES>(cb, src + g[0]);
-                } else {
-                    cp_async_at<ES, so + 2 * PP * ES>(cb, src + g[0]);
-                    cp_async_at<ES, so + 3 * PP * ES>(cb, src + g[NJ]);
-                    if constexpr (NJ == 2) {
-                        cp_async_at<ES, so + (2 * PP + 32) * ES>(cb, src + g[1]);
-                        cp_async_at<ES, so + (3 * PP + 32) * ES>(cb, src + g[NJ + 1]);
-                    }
-                }
-            } else if constexpr (AL) {
-                cp_async_at<16, so>(d[0], src + g[0]);
-                cp_async_at<16, so>(d[1], src + g[1]);
-                if (TY == 14 || hx2) cp_async_at<16, so>(d[2], src + g[2]);
-            } else {
-                cp_async_at<ES, so>(cb, src + g[0]);
-                cp_async_at<ES, so + PP * ES>(cb, src + g[NJ]);
-                cp_async_at<ES, so + (H + 2) * PP * ES>(cb, src + g[2 * NJ]);
-                cp_async_at<ES, so + (H + 3) * PP * ES>(cb, src + g[3 * NJ]);
-                if constexpr (NJ == 2) {
-                    cp_async_at<ES, so + 32 * ES>(cb, src + g[1]);
-                    cp_async_at<ES, so + (PP + 32) * ES>(cb, src + g[NJ + 1]);
-                    cp_async_at<ES, so + ((H + 2) * PP + 32) * ES>(cb, src + g[2 * NJ + 1]);
-                    cp_async_at<ES, so + ((H + 3) * PP + 32) * ES>(cb, src + g[3 * NJ + 1]);
-                }
-                if (lane < 4 * H + 4) cp_async_at<ES, so>(d[0], src + gh[0]);
-                if (lane + 32 < 4 * H + 4) cp_async_at<ES, so>(d[1], src + gh[1]);
-            }
-        };
-        // velocity planes at element offset zo to the slot at element offset SO
+        cp.plan(sm, x0, y0, ty, tx, nx, ny, plane, st);
         auto issue_vel = [&](long long zo, auto SO) {
-            constexpr int so = decltype(SO)::value * ES;
-            if (is_own) {
-                if constexpr (AL) {
-                    const long long o = zo + g[0];
-                    cp_async_at<16, so - PP * ES>(cb, a.u + o);
-                    cp_async_at<16, so + C::VO * ES>(cb, a.v + o);
-                    cp_async_at<16, so + (C::WO - PP) * ES>(cb, a.w + o);
-                } else {
-                    const T *const pu = a.u + zo, *const pv = a.v + zo, *const pw = a.w + zo;
-                    cp_async_at<ES, so>(cb, pu + g[0]);
-                    cp_async_at<ES, so + PP * ES>(cb, pu + g[NJ]);
-                    cp_async_at<ES, so + (C::VO + PP) * ES>(cb, pv + g[0]);
-                    cp_async_at<ES, so + (C::VO + 2 * PP) * ES>(cb, pv + g[NJ]);
-                    cp_async_at<ES, so + C::WO * ES>(cb, pw + g[0]);
-                    cp_async_at<ES, so + (C::WO + PP) * ES>(cb, pw + g[NJ]);
-                    if constexpr (NJ == 2) {
-                        cp_async_at<ES, so + 32 * ES>(cb, pu + g[1]);
-                        cp_async_at<ES, so + (PP + 32) * ES>(cb, pu + g[NJ + 1]);
-                        cp_async_at<ES, so + (C::VO + PP + 32) * ES>(cb, pv + g[1]);
-                        cp_async_at<ES, so + (C::VO + 2 * PP + 32) * ES>(cb, pv + g[NJ + 1]);
-                        cp_async_at<ES, so + (C::WO + 32) * ES>(cb, pw + g[1]);
-                        cp_async_at<ES, so + (C::WO + PP + 32) * ES>(cb, pw + g[NJ + 1]);
-                    }
-                }
-            } else if constexpr (AL) {
-                if (lane < H + 16) cp_async_at<16, so>(d[3], (lane < H ? a.u : a.v) + zo + g[3]);
-            } else {
-                cp_async_at<ES, so + C::VO * ES>(cb, a.v + zo + gv[0]);
-                if constexpr (NJ == 2) cp_async_at<ES, so + (C::VO + 32) * ES>(cb, a.v + zo + gv[1]);
-                if (lane < H) cp_async_at<ES, so>(d[2], a.u + zo + gh[2]);
-            }
+            cp.template vel<decltype(SO)::value>(a.u + zo, a.v + zo, a.w + zo);
         };
-
-        // Runge-Kutta stage operands of plane zo into slot B: own threads, read back by the same
-        // warp only.  Staged a plane ahead rather than held in registers across the sharpening
-        // (which spilled 88 bytes per thread).
+        // Runge-Kutta stage operands of plane zo into slot B: staged a plane ahead rather than
+        // held in registers across the sharpening (which spilled 88 bytes per thread).
         auto issue_rk = [&](long long zo, auto B) {
-            constexpr int so = (C::ORK + decltype(B)::value * 2 * C::RKO) * ES;
+            constexpr int so = C::ORK + decltype(B)::value * 2 * C::RKO;
             if (!is_own) return;
-            const T *const pb = a.rk_base, *const pq = a.rk_q;
-            if constexpr (AL) {
-                if (pb) cp_async_at<16, so>(rkb, pb + zo + g[0]);
-                if (pq) cp_async_at<16, so + C::RKO * ES>(rkb, pq + zo + g[0]);
-            } else {
-                if (pb) {
-                    cp_async_at<ES, so>(rkb, pb + zo + g[0]);
-                    cp_async_at<ES, so + W * ES>(rkb, pb + zo + g[NJ]);
-                    if constexpr (NJ == 2) {
-                        cp_async_at<ES, so + 32 * ES>(rkb, pb + zo + g[1]);
-                        cp_async_at<ES, so + (W + 32) * ES>(rkb, pb + zo + g[NJ + 1]);
-                    }
-                }
-                if (pq) {
-                    constexpr int sq = so + C::RKO * ES;
-                    cp_async_at<ES, sq>(rkb, pq + zo + g[0]);
-                    cp_async_at<ES, sq + W * ES>(rkb, pq + zo + g[NJ]);
-                    if constexpr (NJ == 2) {
-                        cp_async_at<ES, sq + 32 * ES>(rkb, pq + zo + g[1]);
-                        cp_async_at<ES, sq + (W + 32) * ES>(rkb, pq + zo + g[NJ + 1]);
-                    }
-                }
-            }
+            if (a.rk_base) cp.template own<so>(rkb, a.rk_base + zo);
+            if (a.rk_q) cp.template own<so + C::RKO>(rkb, a.rk_q + zo);
         };
 
         // Slot of plane z, phi and velocities: (z - z0) mod 4.
@@ -313,7 +141,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
         if (is_own) {
             const T *src = a.w + (long long)wrapi(z0 - 1, nz) * plane;
             if constexpr (AL) {
-                VV::ld(wlo, src + g[0]);
+                VV::ld(wlo, src + cp.g[0]);
             } else {
                 const int yo = wrapi(own_y, ny) * nx;
 #pragma unroll
@@ -327,7 +155,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
         }
         int zq = wrapi(z0 - 2, nz);  // wrapped index of the next phi plane to stage
         auto next_phi = [&](auto SO) {
-            issue_phi(a.phi + (long long)CDI_CHK(zq, nz, st) * plane, SO);
+            cp.template halo2<decltype(SO)::value>(a.phi + (long long)CDI_CHK(zq, nz, st) * plane);
             zq = zq + 1 == nz ? 0 : zq + 1;
         };
         // planes z0-2 (in the velocity slot of plane z0+3, free until then), z0-1 .. z0+2
@@ -388,7 +216,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
         const int go = nown > 0 ? own_y * nx + own_x : 0;
         // One plane: S = (k - z0) mod 4.
         auto body = [&](auto SC, const int k) {
-            constexpr int S = decltype(SC)::value, S1 = (S + 1) & 3, S2 = (S + 2) & 3, S3 = (S + 3) & 3;
+            constexpr int S = decltype(SC)::value, S1 = (S + 1) & 3, S2 = (S + 2) & 3;
             constexpr int b = S & 1, b1 = b ^ 1;
             // S1: phi plane k+2 and the velocities of plane k have landed, and every thread
             // has left iteration k-1.
@@ -399,7 +227,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
                 cp_async_commit();
             }
             if (k + 4 <= z1 + 1) next_phi(IC<S * C::PHI>{});
-            if (k + 3 < z1) issue_vel(zo + 3 * plane, IC<C::OVEL + S3 * C::VEL>{});
+            if (k + 3 < z1) issue_vel(zo + 3 * plane, IC<C::OVEL + ((S + 3) & 3) * C::VEL>{});
             cp_async_commit();
 
             // B: sharpening at plane k+1 (every warp).
@@ -484,7 +312,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
                 }
                 if constexpr (AL) {
                     if (nown > 0) {
-                        VV::st(op + g[0], o);
+                        VV::st(op + cp.g[0], o);
                         acc.template add_group<VX>(o, a.c.tol);
                     }
                 } else {

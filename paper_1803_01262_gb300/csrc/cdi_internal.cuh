@@ -155,7 +155,7 @@ cudaError_t launch_adj(const AdjArgs<T> &a, int tile, cudaStream_t s);
 
 int adj_num_tiles();
 int adj_blocks(int tile, int zchunk, int nx, int ny, int nz);
-// Tile 3: vector adjoint (nx % (16/sizeof(T)) == 0), tile W x H cells, persistent grid.
+// Tiles 3 (nx % (16/sizeof(T)) == 0) and 4 (any nx): the row kernel, W x H cells, persistent grid.
 bool adj_tile_is_vec(int tile);
 void adj_vec_tile_dims(int esize, int *bw, int *bh);
 template <typename T>

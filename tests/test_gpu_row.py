@@ -4,9 +4,11 @@ and 6 rows with one row more or less, and unit depths around its four ring slots
 one-cell-per-thread tile 0, which computes the same expressions in the same order, so the fields
 must be equal bit for bit (and the extrema and counts equal); NaN and infinity in phi reach the
 same cells."""
+import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_1803_01262_gb300 import cdi
 from paper_1803_01262_gb300 import inputs as I
 
@@ -105,3 +107,35 @@ def test_plane_range_bitwise(dtype, shape, zr):
     g.step_planes(phi, out, zr[0], zr[1], *prm)
     assert torch.equal(out[zr[0]:zr[1]], ref[zr[0]:zr[1]])
     assert (out[:zr[0]] == 7.0).all() and (out[zr[1]:] == 7.0).all()
+
+
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+@pytest.mark.parametrize("shape,split", [((1, 1, 5), 0), ((3, 13, 16), 1), ((5, 15, 63), 2), ((9, 28, 65), 0),
+                                         ((6, 29, 67), cdi.CDI_NCHUNKS_BALANCED), ((21, 16, 130), 3),
+                                         ((4, 43, 33), cdi.CDI_NCHUNKS_ROTATED), ((2, 14, 128), 0)])
+@pytest.mark.parametrize("with_vel", [False, True])
+def test_adjoint_tile_edges(dtype, shape, split, with_vel):
+    """The adjoint row kernel for any row length (tile 4) and for aligned rows (tile 3): the
+    oracle's adjoint step, and velocity gradients added to what the arrays held."""
+    t = np.float64 if dtype == torch.float64 else np.float32
+    nz, ny, nx = shape
+    h = 1.0 / max(shape)
+    rng = np.random.default_rng(7 + nx)
+    phi = np.asarray(I.random_phi(shape, 11 + nx, smooth=True), t).astype(np.float64)
+    u, v, w = (np.asarray(x, t).astype(np.float64) for x in I.random_velocity(shape, h, 8, 3, 5))
+    lam = np.asarray(rng.standard_normal(shape), t).astype(np.float64)
+    dt, eps, gamma, vs = 0.15 * h * h / (1.3 * 1.1 * h), 1.1 * h, 1.3, 0.7
+    ref = oracle.adjoint(phi, u, v, w, lam, h, dt, eps, gamma, vs, want_vel=True, tiny=oracle.adjoint_floor_of(t))
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to("cuda", dtype)
+    g = cdi.Grid(nx, ny, nz, h, dtype)
+    g.set_velocity(*[dev(x) for x in (u, v, w)])
+    base = np.asarray(rng.standard_normal((3,) + shape), t).astype(np.float64)
+    tol = 1e-12 if dtype == torch.float64 else 2e-6  # the bounds of the other adjoint kernels' tests
+    for tile in (4,) + ((3,) if nx % (4 if dtype == torch.float32 else 2) == 0 else ()):
+        g.set_launch(cdi.CDI_KERNEL_ADJOINT, tile, 0, split)
+        out = torch.empty(shape, dtype=dtype, device="cuda")
+        grads = [dev(x) for x in base] if with_vel else None
+        g.step_adjoint(dev(phi), dev(lam), out, dt, eps, gamma, vs, grads=grads)
+        assert np.abs(out.double().cpu().numpy() - ref[0]).max() <= tol * max(1.0, np.abs(ref[0]).max())
+        for a, b, r in zip(grads or (), base, ref[1:]):
+            assert np.abs(a.double().cpu().numpy() - (b + r)).max() <= 4 * tol * max(1.0, np.abs(r).max())
