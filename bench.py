@@ -69,8 +69,8 @@ def measured_peaks():
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("csrc/cdi_fwd.cu", "csrc/cdi_fwd_row.cuh", "csrc/cdi_fwd_common.cuh", "csrc/cdi_reduce.cuh",
-              "csrc/cdi_async.cuh", "csrc/cdi_internal.cuh", "build.py"):
+    for f in ("csrc/cdi_fwd.cu", "csrc/cdi_fwd_row.cuh", "csrc/cdi_row.cuh", "csrc/cdi_fwd_common.cuh",
+              "csrc/cdi_reduce.cuh", "csrc/cdi_async.cuh", "csrc/cdi_internal.cuh", "build.py"):
         h.update(open(os.path.join(ROOT, "paper_1803_01262_gb300", f), "rb").read())
     return h.hexdigest()[:16]
 

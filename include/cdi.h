@@ -146,7 +146,12 @@ CDI_API int cdi_step(cdi_grid *g, const void *phi_in, void *phi_out, double dt, 
  * phi at t0 on entry) and buf_b; vel_scale = cos(pi t / period) at each
  * step's start time t (period <= 0: vel_scale = 1).  The launch loop runs
  * in native code.  On return *final_in_b tells which buffer holds the
- * result.  Stats of the last step are in the device record. */
+ * result.  Stats of the last step are in the device record.
+ * A 2D grid (nz = 1) in its default launch configuration (or the autotuner's)
+ * whose state fits in shared memory is stepped there, up to 512 steps per
+ * cooperative launch, bands of rows exchanging halos; buffers, extrema and
+ * counts as with one launch per step, the sums to rounding.  Its device-side
+ * waits are bounded: CDI_ERR_TIMEOUT from the statistics read-back. */
 CDI_API int cdi_run(cdi_grid *g, void *buf_a, void *buf_b, int nsteps, double t0, double dt,
             double eps, double gamma, double period, int flags, int *final_in_b,
             void *stream);

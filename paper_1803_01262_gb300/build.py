@@ -24,13 +24,13 @@ INCLUDE = os.path.join(ROOT, "include")
 OUT_DIR = os.path.join(PKG, "_lib")
 LIB = os.path.join(OUT_DIR, "libcdi.so")
 LIB_CHECKED = os.path.join(OUT_DIR, "libcdi_checked.so")
-SOURCES = ["cdi_fwd.cu", "cdi_fwd_tma.cu", "cdi_fwd_tb.cu", "cdi_adj.cu", "cdi_batch.cu", "cdi_api.cu",
+SOURCES = ["cdi_fwd.cu", "cdi_fwd_plane.cu", "cdi_fwd_tma.cu", "cdi_fwd_tb.cu", "cdi_adj.cu", "cdi_batch.cu", "cdi_api.cu",
            "cdi_noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # The step kernels (single grid, batch, adjoint) flush FP32 denormals (values
 # below 1.2e-38) to zero; this removes denormal handling around rsqrtf and is far
 # below every tolerance (the adjoint's normal floor is (8 eps)^2 ~ 2e-13).
-PER_FILE = {"cdi_fwd.cu": ["-ftz=true"], "cdi_fwd_tma.cu": ["-ftz=true"], "cdi_fwd_tb.cu": ["-ftz=true"],
+PER_FILE = {"cdi_fwd.cu": ["-ftz=true"], "cdi_fwd_plane.cu": ["-ftz=true"], "cdi_fwd_tma.cu": ["-ftz=true"], "cdi_fwd_tb.cu": ["-ftz=true"],
             "cdi_batch.cu": ["-ftz=true"], "cdi_adj.cu": ["-ftz=true"]}
 # No contraction of a product and a sum into a fused multiply-add beyond the fma()
 # calls the sources write: the compiler's choice differs between the places an

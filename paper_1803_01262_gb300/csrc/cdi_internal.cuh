@@ -134,6 +134,18 @@ cudaError_t tma_occupancy(int *resident);
 template <typename T>
 cudaError_t launch_fwd_tma(const FwdArgs<T> &a, int nblocks, int nchunks, cudaStream_t s);
 
+// Runs of a 2D grid in shared memory (cdi_fwd_plane.cu): at most kPlaneSteps steps per launch,
+// `bands` blocks that wait on one another (plane_bands: 0 where the box does not fit), halo words
+// (plane_word_bytes, zeroed) and a tag counter of the grid (starting at 1).
+constexpr int kPlaneSteps = 512;
+template <typename T>
+cudaError_t plane_bands(int nx, int ny, int sms, int *bands, size_t *smem);
+template <typename T>
+size_t plane_word_bytes(int nx, int bands);
+template <typename T>
+cudaError_t launch_fwd_plane(const FwdArgs<T> &a, T *prev, int n, const T *c_adv, int bands, size_t smem,
+                             unsigned long long *words, unsigned *tag, cudaStream_t s);
+
 // rk selects the Runge-Kutta stage variant (tiles with fwd_tile_has_rk only);
 // face the face-product sharpening (tile 0, Euler only).
 bool fwd_tile_has_rk(int tile);

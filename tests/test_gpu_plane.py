@@ -1,0 +1,83 @@
+"""Runs of 2D grids held in shared memory (bands of rows, one per block, halo words between them):
+the same buffers, extrema and counts as one launch per step on the one-cell-per-thread tile, bit
+for bit (the sums to rounding), for one band (no neighbour), bands of two rows and of uneven
+heights, odd rows, every buffer parity, runs of several launches and time-dependent velocities."""
+import pytest
+import torch
+
+from paper_1803_01262_gb300 import cdi
+
+pytestmark = pytest.mark.gpu
+
+
+def setup(ny, nx, dtype, seed):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    r = lambda: torch.rand((1, ny, nx), generator=gen, device="cuda", dtype=dtype)
+    phi, u, v = 1.1 * r() - 0.05, r() - 0.5, r() - 0.5     # values outside [0, 1]: the counts take part
+    h = 1.0 / max(ny, nx, 2)
+    g = cdi.Grid(nx, ny, 1, h, dtype)
+    g.set_velocity(u, v, torch.zeros_like(u))
+    return g, phi, (0.1 * h, h, 1.0)
+
+
+def ran(g, phi, n, prm, tile):
+    g.set_launch(cdi.CDI_KERNEL_FORWARD, tile, 0, 0)
+    g.reset_run_stats()
+    a, b = phi.clone(), torch.full_like(phi, 3.0)
+    out = g.run(a, b, n, *prm, period=0.7, t0=0.05)
+    return out.clone(), (b if out is a else a).clone(), g.stats()
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("ny,nx", [(1, 1), (1, 37), (3, 5), (4, 300), (5, 301), (37, 1), (33, 129), (128, 128),
+                                   (157, 260), (200, 63)])
+def test_run_equals_one_launch_per_step(dtype, ny, nx):
+    g, phi, prm = setup(ny, nx, dtype, 10 + nx)
+    rel = 1e-12 if dtype == torch.float64 else 1e-6   # order of the sums alone
+    for n in (2, 3, 4, 7):
+        (o0, p0, s0), (o1, p1, s1) = ran(g, phi, n, prm, 0), ran(g, phi, n, prm, -1)
+        assert torch.equal(o0, o1) and torch.equal(p0, p1), n
+        for k in s0:
+            if k in ("mass", "sum"):
+                assert abs(s0[k] - s1[k]) <= rel * max(1.0, abs(s0[k])), (n, k)
+            else:
+                assert s0[k] == s1[k], (n, k)
+
+
+@pytest.mark.parametrize("n", [513, 1030])
+def test_runs_of_several_launches(n):
+    g, phi, prm = setup(20, 70, torch.float32, 5)
+    phi.clamp_(0, 1)
+    (o0, p0, s0), (o1, p1, s1) = ran(g, phi, n, prm, 0), ran(g, phi, n, prm, -1)
+    assert torch.equal(o0, o1) and torch.equal(p0, p1)
+    assert all(s0[k] == s1[k] for k in s0 if k not in ("mass", "sum"))
+
+
+def test_two_grids_on_two_streams_and_a_captured_run():
+    """Halo words and tags belong to a grid: runs of two grids may overlap, and a captured run may
+    be replayed (the tags move on from one replay to the next)."""
+    ga, pa, prm = setup(64, 64, torch.float32, 1)
+    gb, pb, prm_b = setup(96, 50, torch.float32, 2)
+    pa.clamp_(0, 1), pb.clamp_(0, 1)
+    ref_a, ref_b = ran(ga, pa, 30, prm, 0)[0], ran(gb, pb, 30, prm_b, 0)[0]
+    ga.set_launch(cdi.CDI_KERNEL_FORWARD)
+    gb.set_launch(cdi.CDI_KERNEL_FORWARD)
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    a, a2, b, b2 = pa.clone(), torch.empty_like(pa), pb.clone(), torch.empty_like(pb)
+    torch.cuda.synchronize()
+    for _ in range(5):
+        a.copy_(pa), b.copy_(pb)
+        torch.cuda.synchronize()
+        ga.run(a, a2, 30, *prm, period=0.7, t0=0.05, stream=s1)
+        gb.run(b, b2, 30, *prm_b, period=0.7, t0=0.05, stream=s2)
+        torch.cuda.synchronize()
+        assert torch.equal(a, ref_a) and torch.equal(b, ref_b)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ga.run(a, a2, 30, *prm, period=0.7, t0=0.05)
+    for _ in range(3):
+        a.copy_(pa)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(a, ref_a)
+    ga.stats(), gb.stats()      # would raise if a bounded wait had given up
