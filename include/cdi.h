@@ -340,7 +340,10 @@ CDI_API int cdi_batch_get_sharpening(const cdi_batch *b, int *mode);
  * whose largest plane fits in one block's shared memory as 3 nx ny values
  * (about 9600 cells in FP64, 19000 in FP32): the whole plane is staged once
  * and each cell's sharpening evaluated once; the results are those of tiles
- * 0..3 bit for bit (the statistics' sums to rounding).  CDI_ERR_ARG, with the
+ * 0..3 bit for bit (the statistics' sums to rounding).  A run of such a batch
+ * keeps the boxes in shared memory from its first step to its last where they
+ * fit (4 nx ny values), in one launch; its records' sums equal those of single
+ * steps to rounding, everything else exactly.  CDI_ERR_ARG, with the
  * launch unchanged, where it does not apply; zdepth is ignored for it.
  * Tile 5 = bands of whole rows (up to 1024 cells per band, 256 threads, several
  * cells per thread), for batches that hold a 3D box and whose rows are at most

@@ -81,3 +81,54 @@ def test_two_grids_on_two_streams_and_a_captured_run():
         torch.cuda.synchronize()
         assert torch.equal(a, ref_a)
     ga.stats(), gb.stats()      # would raise if a bounded wait had given up
+
+
+def boxes(dtype, sizes, seed):
+    out = []
+    for i, (ny, nx) in enumerate(sizes):
+        gen = torch.Generator(device="cuda").manual_seed(seed + i)
+        r = lambda: torch.rand((1, ny, nx), generator=gen, device="cuda", dtype=dtype)
+        h = 1.0 / max(ny, nx, 2)
+        phi, u, v = 1.1 * r() - 0.05, r() - 0.5, r() - 0.5
+        out.append(dict(dx=h, dt=0.1 * h, eps=h, gamma=1.0, u=u, v=v, w=torch.zeros_like(u), phi_a=phi,
+                        phi_b=torch.full_like(phi, 3.0)))
+    return out
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("sharpen", ["centre", "face"])
+@pytest.mark.parametrize("nbox", [4, 5, 700])
+def test_batch_run_equals_other_tiles(dtype, sharpen, nbox):
+    """Batch tile 4's run (boxes held in shared memory; with more boxes than slots, in units of a
+    few steps handed from block to block): both buffers, extrema and counts of tile 0's run bit
+    for bit, for runs of 1..16 steps in sequence and a run after single steps."""
+    sizes = [(7, 9), (33, 40), (1, 37), (3, 2), (16, 64)] if nbox == 5 else [(5 + i % 7, 4 + i % 11) for i in range(nbox)]
+    b0 = boxes(dtype, sizes, 3)
+    b4 = [dict(x, phi_a=x["phi_a"].clone(), phi_b=x["phi_b"].clone()) for x in b0]
+    bt = [cdi.Batch(x) for x in (b0, b4)]
+    for b, tile in zip(bt, (0, 4)):
+        b.set_sharpening(sharpen)
+        b.set_launch(tile, 0)
+    for n in (2, 5, 1, 16, 3):
+        for b in bt:
+            b.step(1.0)
+            b.run(n)
+        for x, y in zip(b0, b4):
+            assert torch.equal(x["phi_a"], y["phi_a"]) and torch.equal(x["phi_b"], y["phi_b"]), n
+    rel = 1e-12 if dtype == torch.float64 else 1e-6
+    for p, q in zip(bt[0].stats(), bt[1].stats()):
+        for k in p:
+            if k in ("mass", "sum"):
+                assert abs(p[k] - q[k]) <= rel * max(1.0, abs(p[k])), k
+            else:
+                assert p[k] == q[k], k
+
+
+def test_batch_autotune_leaves_state_and_records():
+    """The autotuner's trial runs on chip read the current state and restore the records."""
+    bx = boxes(torch.float64, [(20, 30), (50, 50), (12, 9)], 9)
+    bt = cdi.Batch(bx)
+    bt.step(1.0)
+    ref, st = [bt.current(i).clone() for i in range(3)], bt.stats()
+    bt.autotune(reps=2)
+    assert all(torch.equal(bt.current(i), r) for i, r in enumerate(ref)) and bt.stats() == st
