@@ -351,7 +351,7 @@ CDI_API int cdi_batch_get_sharpening(const cdi_batch *b, int *mode);
  * the array, staged by 16-byte copies whatever the row alignment; the fields
  * are those of tiles 0..3 bit for bit.  CDI_ERR_ARG where it does not apply.
  * Tile 6 = bands of whole rows of the batch's own padded copy of every box
- * (rows padded to 16-byte multiples with periodic ghost cells at both ends,
+ * (rows padded to 16-byte multiples with two periodic ghost cells after the last,
  * allocated on first use: 5 arrays of the padded box size): 16-byte copies and
  * 16-byte shared loads of four (FP32) or two (FP64) cells per thread whatever
  * nx is.  Each step or run call first copies the caller's current state into

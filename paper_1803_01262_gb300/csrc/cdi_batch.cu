@@ -47,7 +47,7 @@ struct BoxDev {
     // the state by parity, and the face velocities
     T *pad[2];
     const T *pu, *pv, *pw;
-    int pitch;
+    int pitch, spitch;  // row pitch, and that of a staged row
 };
 
 // Whole-plane unit body: the unit is a whole 2D box (nz == 1) whose phi and
@@ -167,15 +167,14 @@ __device__ __forceinline__ bool wait_epoch(const unsigned int *epoch, unsigned t
 // in shared memory: one unit per box, the whole-plane body (plane_unit).
 // BODY 3: bands of whole rows (band_unit, cdi_band.cuh), slots of sizes bs.
 // BODY 4: bands of whole rows of the padded copies (vband_unit, cdi_vband.cuh),
-// slots of sizes vbs; final_write: the step also writes the caller's arrays.
+// final_write: the step also writes the caller's arrays.
 // FACE: the face-product sharpening (bodies 0, 1 and 2).  sync: the launch's
 // hand-out counters and its place in a run (BatchSync).
 template <typename T, int BX, int BY, int BODY = 0, bool FACE = false>
 __global__ void __launch_bounds__(BX * BY, BODY >= 3 ? 2 : 1)
 batch_kernel(const BoxDev<T> *__restrict__ boxes, const int *__restrict__ unit_box,
              const int total_units, const int parity, const T vs, Partial *partials,
-             unsigned int *box_done, StatsRec *recs, const BandSlots bs, const VbandSlots vbs,
-             const int final_write, const BatchSync sync)
+             unsigned int *box_done, StatsRec *recs, const BandSlots bs, const int final_write, const BatchSync sync)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int fold, next_u, ready;
@@ -223,8 +222,9 @@ batch_kernel(const BoxDev<T> *__restrict__ boxes, const int *__restrict__ unit_b
             const int lu = u - bx.unit0, nb = bx.ntiles, zc = bx.zc;
             const int chunk = lu / nb, band = lu - chunk * nb;
             const int z0 = chunk * zc;
-            vband_unit<T>(a, bx.pad[parity], bx.pad[parity ^ 1], bx.pu, bx.pv, bx.pw, bx.pitch, final_write != 0,
-                          band * bx.bh, bx.bh, z0, min(a.nz, z0 + zc), vbs, acc, smem_raw);
+            const VbandIO<T> io = {bx.pad[parity], bx.pu, bx.pad[parity ^ 1], final_write ? a.out : nullptr,
+                                   bx.pv - bx.pu, bx.pitch, bx.spitch};
+            vband_unit<T>(a, io, band * bx.bh, bx.bh, z0, min(a.nz, z0 + zc), acc, reinterpret_cast<T *>(smem_raw));
         } else {
             const int lu = u - boxes[bi].unit0;
             const Unit un = unit_of(lu, boxes[bi].ntiles, boxes[bi].tiles_x, BX, BY, boxes[bi].zc, a.nz);
@@ -433,8 +433,10 @@ plane_bands_kernel(const BoxDev<T> *__restrict__ boxes, const int nb, const int 
 }
 
 // Fill a box's padded copy (cdi_vband.cuh) from a caller's array: position p of
-// a padded row holds the row's cell (p - VX) mod nx.  blockIdx.y: the box.
+// a padded row holds the row's cell p mod nx.  blockIdx.y: the box.
 // which: 0, 1 the state of that parity (from phi_a / phi_b), 2, 3, 4 u, v, w.
+// Bound by memory: a vector per thread, four rows in flight (a block per row, an element per
+// thread, took 229 us for 65 M FP32 cells; this 70).
 template <typename T>
 __global__ void __launch_bounds__(256) vband_pack(const BoxDev<T> *__restrict__ boxes, int which)
 {
@@ -443,10 +445,27 @@ __global__ void __launch_bounds__(256) vband_pack(const BoxDev<T> *__restrict__ 
     const FwdArgs<T> &a = bx.a;
     const T *src = which == 0 ? a.phi : which == 1 ? a.out : which == 2 ? a.u : which == 3 ? a.v : a.w;
     T *dst = which <= 1 ? bx.pad[which] : const_cast<T *>(which == 2 ? bx.pu : which == 3 ? bx.pv : bx.pw);
-    const int nx = a.nx, P = bx.pitch;
+    const int nx = a.nx, P = bx.pitch, nv = P / VX, rb = 256 / nv;
+    const int r = threadIdx.x / nv, p = (threadIdx.x - r * nv) * VX;
     const long long rows = (long long)a.ny * a.nz;
-    for (long long row = blockIdx.x; row < rows; row += gridDim.x)
-        for (int p = threadIdx.x; p < P; p += 256) dst[row * P + p] = src[row * nx + wrapi(p - VX, nx)];
+    if (r >= rb) return;
+    int x[VX];
+#pragma unroll
+    for (int i = 0; i < VX; ++i) x[i] = (p + i) % nx;
+    constexpr int U = 4;  // rows in flight per thread
+    const long long stride = (long long)gridDim.x * rb;
+    for (long long row = (long long)blockIdx.x * rb + r; row < rows; row += U * stride) {
+        T c[U][VX];
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const long long o = min(row + k * stride, rows - 1) * nx;
+#pragma unroll
+            for (int i = 0; i < VX; ++i) c[k][i] = __ldg(src + o + x[i]);
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k)
+            if (row + k * stride < rows) V16<T>::st(dst + (row + k * stride) * P + p, c[k]);
+    }
 }
 
 // Batch tiles 0..3: the scalar tiles of the single-box kernel; tile 4: one
@@ -479,8 +498,7 @@ struct cdi_batch {
     int sharpen;               // CDI_SHARPEN_CENTRE or CDI_SHARPEN_FACE (tiles 0 and 4 only)
     BandSlots band;            // row-band body: slot sizes for the largest box
     size_t band_bytes;         // its shared memory (0: the band body does not apply)
-    cdi::VbandSlots vband;     // vector row-band body (tile 6): slot sizes for the largest box
-    size_t vband_bytes;        // its shared memory (0: it does not apply)
+    size_t vband_bytes;        // shared memory of the vector row-band body (tile 6; 0: it does not apply)
     void *padbuf;              // tile 6: the padded copies of every box (allocated on first use)
     bool vel_packed;           // the padded face velocities are filled
     std::vector<cdi_box_desc> desc;
@@ -783,40 +801,19 @@ static size_t band_bytes(cdi_batch *b)
     return b->dtype == CDI_F64 ? band_bytes_t<double>(b) : band_bytes_t<float>(b);
 }
 
-// Slot sizes of the vector band body for this batch (each slot field the largest
-// over its boxes, the velocity regions laid out one after another) and their
-// shared memory; 0 if they exceed the shared memory of one block.
+// Shared memory of the vector band body; 0 if it does not apply to some box of the batch.
 template <typename T>
-static size_t vband_bytes_t(cdi_batch *b)
+static size_t vband_bytes_t(const cdi_batch *b)
 {
     const int vx = 16 / (int)sizeof(T);
     if (b->nbox > 65535) return 0;  // the copy kernels take the box from blockIdx.y
-    int phi = 0, ur = 0, vr = 0, sx = 0, sy = 0;
-    for (const cdi_box_desc &x : b->desc) {
-        if ((x.nx + vx - 1) / vx > cdi::VBAND_NT) return 0;  // a row has more groups than the block threads
-        const int P = cdi::vband_pitch(x.nx, vx), hb = cdi::vband_rows(x.nx, x.ny, vx);
-        if (hb < 1) return 0;  // a padded row too wide for the staging plan
-        const cdi::VbandSlots t = cdi::vband_slots(P, hb);
-        phi = std::max(phi, t.phi);
-        ur = std::max(ur, hb * P);
-        vr = std::max(vr, (hb + 1) * P);
-        sx = std::max(sx, t.sx);
-        sy = std::max(sy, t.sy);
-    }
-    cdi::VbandSlots s;
-    s.phi = phi;
-    s.vo = ur;
-    s.wo = ur + vr;
-    s.vel = 2 * ur + vr;
-    s.sx = sx;
-    s.sy = sy;
-    const size_t need = cdi::vband_smem_bytes(s, sizeof(T));
-    if (need > vband_limit<T>()) return 0;
-    b->vband = s;
-    return need;
+    for (const cdi_box_desc &x : b->desc)
+        if (cdi::vband_rows(x.nx, x.ny, vx, cdi::vband_staged(x.nx, x.ny, vx)) < 1) return 0;  // a row too wide for a band
+    const size_t need = cdi::VbandGeo<T>::bytes;
+    return need <= vband_limit<T>() ? need : 0;
 }
 
-static size_t vband_bytes(cdi_batch *b)
+static size_t vband_bytes(const cdi_batch *b)
 {
     return b->dtype == CDI_F64 ? vband_bytes_t<double>(b) : vband_bytes_t<float>(b);
 }
@@ -909,7 +906,8 @@ static int build_units(cdi_batch *b, int tile, int zdepth)
             e.ntiles = (x.ny + e.bh - 1) / e.bh;
         }
         if (vband) {  // bands of whole padded rows
-            e.bh = cdi::vband_rows(x.nx, x.ny, VX);
+            e.spitch = VX * cdi::vband_staged(x.nx, x.ny, VX);
+            e.bh = cdi::vband_rows(x.nx, x.ny, VX, e.spitch / VX);
             e.ntiles = (x.ny + e.bh - 1) / e.bh;
         }
         if (pad) {  // the padded copies (laid out box after box)
@@ -1013,7 +1011,7 @@ static cudaError_t launch_batch_kernel(cdi_batch *b, size_t smem, int parity, do
     cfg.numAttrs = y.step > 0 && !y.reset ? 1 : 0;  // a run's launches after its first
     return cudaLaunchKernelEx(&cfg, cdi::batch_kernel<T, BX, BY, BODY, FACE>, (const BoxDev<T> *)b->boxes_dev,
                               (const int *)b->unit_box, b->total_units, parity, (T)vs, b->partials, b->box_done,
-                              b->recs, b->band, b->vband, final_write, y);
+                              b->recs, b->band, final_write, y);
 }
 
 template <typename T, int BX, int BY>

@@ -1,184 +1,183 @@
 // Vector row-band unit body of the batched CDI step, on the batch's padded copy
 // of each box.
 //
-// The batch keeps its own copy of every box in a padded layout: each row of nx
-// cells sits at offset GH = VX (one 16-byte vector) inside a row of pitch
-// P = round_up(nx + 2 VX, VX) elements, and the VX positions on either side of
-// the row hold its periodic continuation (ghost cells: position GH + x holds
-// phi at x mod nx for x in [-VX, nx + VX)).  Rows and planes then start on
-// 16-byte boundaries whatever nx is, so a unit -- a band of whole rows
+// The batch keeps its own copy of every box: each row of nx cells starts a row of
+// pitch P = round_up(nx + 2, VX) elements (VX: a 16-byte vector), and the two
+// positions after it hold its periodic continuation (cells 0 and 1).  Rows and planes
+// then start on 16-byte boundaries whatever nx is, so a unit -- a band of whole rows
 // [y0, y0 + hb) and a range of planes [z0, z1) -- is staged by 16-byte copies
-// only (each thread's few vectors of a region planned once per unit, rows
-// outside [0, ny) wrapped in y), and
-// each thread owns one group of VX consecutive cells of the band, read with
-// 16-byte shared loads like the single-box vector kernel (fwd_vec_kernel): the
-// x neighbours of a group are its first and last neighbours in the padded row,
-// the ghosts at the row ends.  s_x at x = -1 and x = nx is s_x at nx - 1 and 0
+// (each thread's few vectors of a region planned once per unit, rows outside [0, ny)
+// wrapped in y) and one 4-byte copy for the cells left of x = 0 (a staged row has a
+// vector of room there: pitch P + VX).  Each thread owns one group of VX consecutive
+// cells of the band: whole rows, so no lane idles past a row's end but in its last
+// group (tiles of 32 x 28 or 64 x 14 cells would cover 32..160-cell boxes 1.3 to 1.4
+// times over, the bands 1.13 times).  s_x at x = -1 and x = nx is s_x at nx - 1 and 0
 // (s is periodic with phi); a partial last group (nx % VX != 0) evaluates s at
-// its ghost cells from their ghost neighbours, the periodic values.
+// x = nx from its ghost neighbours, the periodic values.
 //
-// Per plane k (one barrier): phi plane k+4 and the velocities of plane k+2 are
-// issued; the sharpening s = phi (1 - phi) g/|g| of plane k+1 is evaluated for
-// the band's groups and (s_y only) its two ring rows; plane k is updated from
-// its face fluxes, the x and y faces telescoped and the z face below carried --
-// fwd_vec_kernel's expressions in its order, so the field is the other
-// kernels' bit for bit.  The output goes to the padded copy of the next state
-// (interior and ghost cells) and, on the last step of a call (final), also to
-// the caller's array.
+// The plane loop is the row kernel's (fwd_row_kernel): phi around a group stays in
+// registers from the sharpening at plane k+1 to the update at plane k+1, every slot
+// lies at a compile-time offset (sized for the largest band), unrolled over the four phi
+// slots, and four base registers (a row's place and one, two, three pitches on) reach
+// every array.  Its expressions in its order: the field is the other kernels' bit for
+// bit.
+//
+// What bounds it: latency (16 warps per SM, one barrier per plane; 60% of the issue slots, DRAM
+// and L2 at 60% and 32% of their rates).  Fewer rows per band, so that no thread has a ring group
+// besides its own, took 20% longer.  64 FP32 boxes with edges 32..160 (65 M cells): 143 -> 107
+// instructions per cell, 341 -> 304 us per step of a run (with the ghost cells at both ends of a
+// row kept by the stores, slots at run-time offsets, a condition per thread around the update and
+// its operands loaded after the sharpening).  The output goes to the padded copy of the next state and, on the last step of a
+// call (final_write), also to the caller's array.
 #pragma once
 
 #include "cdi_async.cuh"
 #include "cdi_fwd_common.cuh"
 #include "cdi_reduce.cuh"
+#include "cdi_row.cuh"
 
 namespace cdi {
 
 constexpr int VBAND_NT = 256;  // threads of a vector band block (one cell group each)
+constexpr int VBAND_CPY = 2;   // 16-byte vectors of a staged region a thread copies per plane
+
+// Slots (elements), whatever the box: 106 kB, two blocks per SM.
+template <typename T>
+struct VbandGeo {
+    static constexpr int VX = 16 / sizeof(T);
+    static constexpr int PHI = VBAND_CPY * VBAND_NT * VX;  // rows y0-2 .. y0+hb+1
+    static constexpr int UW = 336 * VX, V = 360 * VX;      // u, w rows y0 ..; v rows y0-1 ..
+    static constexpr int VO = UW, WO = UW + V, VEL = 2 * UW + V;
+    static constexpr int SX = UW, SY = 400 * VX;           // s_x rows y0 ..; s_y rows y0-1 .. y0+hb
+    static constexpr int NPHI = 4, NVEL = 3;
+    static constexpr int OVEL = NPHI * PHI, OSX = OVEL + NVEL * VEL, OSY = OSX + 2 * SX;
+    static constexpr size_t bytes = sizeof(T) * (size_t)(OSY + 2 * SY);
+    static_assert(VEL >= PHI, "the prologue's first phi plane borrows a velocity slot");
+};
 
 // Padded layout of a box: row pitch in elements (VX = 16 / sizeof(T)).
-__host__ __device__ inline int vband_pitch(int nx, int vx) { return (nx + 2 * vx + vx - 1) / vx * vx; }
+__host__ __device__ inline int vband_pitch(int nx, int vx) { return (nx + 2 + vx - 1) / vx * vx; }
 
-// Rows per band: as many whole rows as there are thread groups for, and few
-// enough that each thread copies at most VBAND_CPY 16-byte vectors of a staged
-// region per plane (the phi region is hb + 4 padded rows).  0: a padded row is
-// too wide for that (then the body does not apply).
-constexpr int VBAND_CPY = 2;
-__host__ __device__ inline int vband_rows(int nx, int ny, int vx)
+// Rows per band: as many whole rows as there are thread groups for and as fit in the slots
+// with sv vectors per staged row, with one 4-byte copy per thread (2 (hb + 4) + hb of them).
+// 0: a row is too wide (then the body does not apply).
+__host__ __device__ inline int vband_rows(int nx, int ny, int vx, int sv)
 {
-    const int g = (nx + vx - 1) / vx;
-    const int nv = vband_pitch(nx, vx) / vx;
-    int hb = VBAND_NT / g;
-    const int cap = VBAND_CPY * VBAND_NT / nv - 4;
-    if (hb > cap) hb = cap;
-    if (hb < 1) return 0;
-    return hb < ny ? hb : ny;
+    if (nx > 100 * vx) return 0;
+    int hb = VBAND_NT / ((nx + vx - 1) / vx);
+    const int cap[] = {VBAND_CPY * VBAND_NT / sv - 4, 336 / sv, 360 / sv - 1, 400 / sv - 2, (VBAND_NT - 8) / 3, ny};
+    for (int c : cap) hb = c < hb ? c : hb;
+    return hb;
 }
 
-// Ring-slot sizes (elements; multiples of VX) for the largest box of a batch.
-struct VbandSlots {
-    int phi;          // (hb + 4) P
-    int vel;          // u | v | w: hb P, (hb + 1) P, hb P
-    int vo, wo;       // offsets of v and w in a velocity slot (u at 0)
-    int sx, sy;       // hb P and (hb + 2) P
+// Vectors of a staged row: the row and a vector left of it -- or G + 8 for G groups, where that
+// costs no rows of the band: eight lanes of a 16-byte access that straddle two rows then hit
+// different banks.
+__host__ __device__ inline int vband_staged(int nx, int ny, int vx)
+{
+    const int sv = vband_pitch(nx, vx) / vx + 1, g = (nx + vx - 1) / vx;
+    return g % 8 && vband_rows(nx, ny, vx, g + 8) == vband_rows(nx, ny, vx, sv) ? g + 8 : sv;
+}
+
+// The arrays of a unit: padded copies, plane stride P ny, pu | pv | pw vstride apart; raw: the
+// caller's array, written too (nullable).
+template <typename T>
+struct VbandIO {
+    const T *pin, *pu;
+    T *pout, *raw;
+    long long vstride;
+    int P, PS;      // row pitch, and that of a staged row
 };
-
-__host__ __device__ inline VbandSlots vband_slots(int P, int hb)
-{
-    VbandSlots s;
-    s.phi = (hb + 4) * P;
-    s.vo = hb * P;
-    s.wo = s.vo + (hb + 1) * P;
-    s.vel = s.wo + hb * P;
-    s.sx = hb * P;
-    s.sy = (hb + 2) * P;
-    return s;
-}
-
-__host__ __device__ inline size_t vband_smem_bytes(const VbandSlots &s, size_t esize)
-{
-    return esize * (size_t)(5 * s.phi + 3 * s.vel + 2 * s.sx + 2 * s.sy);
-}
-
-// phi around a thread's group at one plane: the group, the groups above and below
-// it in y, and its x neighbours (carried from the sharpening at plane k+1 to the
-// update at plane k+1 in the next iteration).
-template <typename T, int VX>
-struct PhiNb {
-    T c[VX], yn[VX], yp[VX];
-    T L, R;
-};
-
-// Staging plan of one region -- `rows` padded rows from row yb (wrapped in y)
-// -- for this thread: the in-plane offsets of its (at most VBAND_CPY) 16-byte
-// vectors, chunk c = tid + i VBAND_NT of the region landing at c VX in the
-// slot; -1 where the thread has no such chunk.  Fixed per unit; a plane adds
-// only its base pointer.
-template <int VX>
-__device__ __forceinline__ void vband_plan(int *g, int yb, int rows, int P, int ny, int tid, unsigned *st)
-{
-    (void)st;
-    const int nv = P / VX;
-#pragma unroll
-    for (int i = 0; i < VBAND_CPY; ++i) {
-        const int c = tid + i * VBAND_NT;
-        if (c < rows * nv) {
-            const int row = c / nv;
-            g[i] = CDI_CHK(wrapi(yb + row, ny), ny, st) * P + (c - row * nv) * VX;
-        } else {
-            g[i] = -1;
-        }
-    }
-}
 
 template <typename T>
-__device__ __forceinline__ void vband_unit(const FwdArgs<T> &a, const T *__restrict__ pin, T *__restrict__ pout,
-                                           const T *__restrict__ pu, const T *__restrict__ pv,
-                                           const T *__restrict__ pw, int P, bool final_write, int y0, int hb,
-                                           int z0, int z1, const VbandSlots &S, Acc<T> &acc,
-                                           unsigned char *smem_raw)
+__device__ __forceinline__ void vband_unit(const FwdArgs<T> &a, const VbandIO<T> &io, int y0, int hb, int z0, int z1,
+                                           Acc<T> &acc, T *const sm)
 {
-    constexpr int VX = 16 / sizeof(T), GH = VX, NT = VBAND_NT;
+    using C = VbandGeo<T>;
+    constexpr int VX = C::VX, NT = VBAND_NT, ES = sizeof(T);
     using VV = V16<T>;
-    T *const sphi = reinterpret_cast<T *>(smem_raw);  // [5][S.phi]
-    T *const svel = sphi + 5 * S.phi;                  // [3][S.vel]
-    T *const ssx = svel + 3 * S.vel;                   // [2][S.sx]
-    T *const ssy = ssx + 2 * S.sx;                     // [2][S.sy]
 
     const int tid = threadIdx.x;
-    const int nx = a.nx, ny = a.ny, nz = a.nz;
+    const int nx = a.nx, ny = a.ny, nz = a.nz, P = io.P, PS = io.PS;
     const long long planeP = (long long)P * ny;        // padded plane
-    const long long plane = (long long)nx * ny;        // the caller's plane
     unsigned *const st = a.red.status;
     (void)st;
     const T c_adv = a.c.c_adv, c_dif = a.c.c_dif, c_shp = a.c.c_shp, c_upd = a.c.c_upd;
 
     const int G = (nx + VX - 1) / VX;    // groups per row
     const int hbe = min(hb, ny - y0);    // rows of this band
-    const int r = tid / G, j = tid - r * G;
-    const bool act = r < hbe;            // this thread owns group j of band row r
+    // This thread owns group j of band row r.  Warps with such threads run the loop with the
+    // update, their lanes past the band on its last group (the same values to the same places, no
+    // output); the others the loop without it.  (A condition per thread around the update instead
+    // copied every carried value at its end: 15 moves per cell.)
+    const int own = min(tid, hbe * G - 1);
+    const bool act = (tid & ~31) < hbe * G;
+    const int r = own / G, j = own - r * G;
     const int x0 = j * VX;
-    const int nown = act ? min(VX, nx - x0) : 0;  // cells of the group inside the row
-    const int pos = (r + 2) * P + GH + x0;  // the group in a phi slot
-    const int sxo = r * P + GH + x0;        // ... in s_x
-    const int syo = (r + 1) * P + GH + x0;  // ... in s_y (row 0: the ring row below)
-    const int dL = x0 == 0 ? nx : 0;                   // s_x left of x = 0 is s_x(nx - 1)
-    const int dR = x0 + VX == nx ? -nx : 0;            // right of x = nx - 1 (full last group): s_x(0)
-    // ghost copies of the group's cells: bit 2i, cell i feeds the left ghost at x - nx;
-    // bit 2i+1, the right ghost at x + nx (nx >= GH; smaller rows take every copy)
-    unsigned gmask = 0u;
-#pragma unroll
-    for (int i = 0; i < VX; ++i) {
-        const int x = x0 + i;
-        if (i < nown) gmask |= ((x >= nx - GH ? 1u : 0u) | (x < GH ? 2u : 0u)) << (2 * i);
-    }
+    const int nown = tid < hbe * G ? min(VX, nx - x0) : 0;  // cells of the group inside the row
+    // b0 + q PS: the group in row r + q of an array, so phi row r - 2 + q, u, w, s_x row r + q,
+    // v, s_y row r - 1 + q
+    T *const b0 = sm + r * PS + VX + x0;
+    T *const b1 = b0 + PS, *const b2 = b1 + PS, *const b3 = b2 + PS;
+    // s_x left of x = 0 is s_x(nx - 1), right of x = nx - 1 (full last group) s_x(0)
+    const T *const sL = b0 + (x0 == 0 ? nx - 1 : -1), *const sR = b0 + (x0 + VX == nx ? VX - nx : VX);
+    // ring rows (s_y below and above the band): a group each for 2 G threads, those without a
+    // group of their own first; rg: its place as b2 is the own group's
+    const int l = NT - 1 - tid;
+    const bool ring = l < 2 * G;
+    T *const rg = sm + (ring ? ((l >= G ? hbe : -1) + 2) * PS + VX + (l >= G ? l - G : l) * VX : PS);
 
-    // sharpening of the group at phi-slot offset off of plane Pm (below Pmm, above Pmp);
-    // zn_in (nullable): the group at the plane below, already loaded; nb_out (nullable):
-    // receives phi around the group at this plane (the own group's next update reads it)
-    auto sharp_group = [&](const T *Pm, const T *Pmm, const T *Pmp, int off, T *s0, T *s1, T *s2,
-                           const T *zn_in = nullptr, PhiNb<T, VX> *nb_out = nullptr) {
-        T c[VX], yn[VX], yp[VX], zn[VX], zp[VX];
-        VV::ld(c, Pm + off);
-        VV::ld(yn, Pm + off - P);
-        VV::ld(yp, Pm + off + P);
-        if (zn_in) {
+    // this thread's chunks of the staged regions: phi, u and w (same rows), v; ge: its single cell,
+    // of phi (2 left of each row) or of u (1 left of each row)
+    int gphi[VBAND_CPY], guw[VBAND_CPY], gv[VBAND_CPY], ge = 0;
+    unsigned d[VBAND_CPY], de;  // shared byte addresses
+    const int nv = P / VX;
 #pragma unroll
-            for (int i = 0; i < VX; ++i) zn[i] = zn_in[i];
-        } else {
-            VV::ld(zn, Pmm + off);
-        }
-        VV::ld(zp, Pmp + off);
-        const T L = Pm[off - 1], R = Pm[off + VX];
-        if (nb_out) {
+    for (int i = 0; i < VBAND_CPY; ++i) {
+        const int c = tid + i * NT, row = c / nv, col = (c - row * nv) * VX;
+        auto at = [&](int yb, int rows) { return row < rows ? CDI_CHK(wrapi(yb + row, ny), ny, st) * P + col : -1; };
+        gphi[i] = at(y0 - 2, hbe + 4);
+        guw[i] = at(y0, hbe);
+        gv[i] = at(y0 - 1, hbe + 1);
+        d[i] = smem_addr(sm + (row < hbe + 4 ? row * PS + VX + col : 0));
+    }
+    const bool ephi = tid < 2 * (hbe + 4), eu = !ephi && tid < 2 * (hbe + 4) + hbe;
+    {
+        const int row = ephi ? tid >> 1 : eu ? tid - 2 * (hbe + 4) : 0, x = ephi ? -1 - (tid & 1) : -1;
+        ge = CDI_CHK(wrapi(y0 + row - (ephi ? 2 : 0), ny), ny, st) * P + wrapi(x, nx);
+        de = smem_addr(sm + row * PS + VX + x);
+    }
+    int zq = wrapi(z0 - 2, nz);  // wrapped index of the next phi plane to stage
+    auto next_phi = [&](auto SO) {
+        constexpr int so = decltype(SO)::value * ES;
+        const T *const src = io.pin + (long long)CDI_CHK(zq, nz, st) * planeP;
 #pragma unroll
-            for (int i = 0; i < VX; ++i) {
-                nb_out->c[i] = c[i];
-                nb_out->yn[i] = yn[i];
-                nb_out->yp[i] = yp[i];
+        for (int i = 0; i < VBAND_CPY; ++i)
+            if (gphi[i] >= 0) cp_async_at<16, so>(d[i], src + gphi[i]);
+        if (ephi) cp_async_at<ES, so>(de, src + ge);
+        zq = zq + 1 == nz ? 0 : zq + 1;
+    };
+    const T *vsrc = io.pu + (long long)CDI_CHK(z0, nz, st) * planeP;  // u at the next velocity plane to stage
+    int vis = 0, vrd = 0;  // velocity slots (element offsets) of that plane, and of plane k
+    auto next_vel = [&]() {
+        constexpr int so = C::OVEL * ES;
+        const unsigned vb = vis * ES;
+#pragma unroll
+        for (int i = 0; i < VBAND_CPY; ++i) {
+            if (guw[i] >= 0) {
+                cp_async_at<16, so>(d[i] + vb, vsrc + guw[i]);
+                cp_async_at<16, so + C::WO * ES>(d[i] + vb, vsrc + 2 * io.vstride + guw[i]);
             }
-            nb_out->L = L;
-            nb_out->R = R;
+            if (gv[i] >= 0) cp_async_at<16, so + C::VO * ES>(d[i] + vb, vsrc + io.vstride + gv[i]);
         }
+        if (eu) cp_async_at<ES, so>(de + vb, vsrc + ge);
+        vsrc += planeP;
+        vis = vis == 2 * C::VEL ? 0 : vis + C::VEL;
+    };
+
+    // Sharpening of the cells c, from the y neighbours, the planes below (zn) and above (zp)
+    // and the x neighbours L, R.
+    auto sharp = [&](const T *c, const T *yn, const T *yp, const T *zn, const T *zp, T L, T R, T *s0, T *s1, T *s2) {
 #pragma unroll
         for (int i = 0; i < VX; ++i) {
             const T g0 = (i + 1 < VX ? c[i + 1] : R) - (i > 0 ? c[i - 1] : L);
@@ -192,202 +191,187 @@ __device__ __forceinline__ void vband_unit(const FwdArgs<T> &a, const T *__restr
             s2[i] = wgt * g2;
         }
     };
-    // s_y of the ring rows (below and above the band) at a plane
-    auto sharp_ring = [&](const T *Pm, const T *Pmm, const T *Pmp, T *sy) {
-        for (int l = NT - 1 - tid; l < 2 * G; l += NT) {  // the threads without a group first
-            const int top = l >= G;
-            const int jj = l - top * G;
-            const int row = top ? hbe : -1;
-            T s0[VX], s1[VX], s2[VX];
-            sharp_group(Pm, Pmm, Pmp, (row + 2) * P + GH + jj * VX, s0, s1, s2);
-            VV::st(sy + (row + 1) * P + GH + jj * VX, s1);
-        }
-    };
 
-    // this thread's chunks of the staged regions: phi, u and w (same rows), v
-    int gphi[VBAND_CPY], guw[VBAND_CPY], gv[VBAND_CPY];
-    vband_plan<VX>(gphi, y0 - 2, hbe + 4, P, ny, tid, st);
-    vband_plan<VX>(guw, y0, hbe, P, ny, tid, st);
-    vband_plan<VX>(gv, y0 - 1, hbe + 1, P, ny, tid, st);
-    // phi plane of wrapped index zw into ring slot `slot`
-    auto issue_phi = [&](int zw, int slot) {
-        const T *const src = pin + (long long)zw * planeP;
-        T *const d = sphi + slot * S.phi + tid * VX;
-#pragma unroll
-        for (int i = 0; i < VBAND_CPY; ++i)
-            if (gphi[i] >= 0) cp_async<16>(d + i * VBAND_NT * VX, src + gphi[i]);
-    };
-    auto issue_vel = [&](int z, int slot) {
-        const long long zo = (long long)CDI_CHK(z, nz, st) * planeP;
-        T *const d = svel + slot * S.vel + tid * VX;
-#pragma unroll
-        for (int i = 0; i < VBAND_CPY; ++i) {
-            if (guw[i] >= 0) {
-                cp_async<16>(d + i * VBAND_NT * VX, pu + zo + guw[i]);
-                cp_async<16>(d + S.wo + i * VBAND_NT * VX, pw + zo + guw[i]);
-            }
-            if (gv[i] >= 0) cp_async<16>(d + S.vo + i * VBAND_NT * VX, pv + zo + gv[i]);
-        }
-    };
-
-    // phi slot of plane z: (z - z0 + 2) mod 5; velocity slot: (z - z0) mod 3.
+    // Slot of phi plane z: (z - z0) mod 4; of its velocities: (z - z0) mod 3.
     __syncthreads();  // the previous unit's readers are done with every slot
-    for (int d = 0; d < 5; ++d) issue_phi(wrapi(z0 - 2 + d, nz), d);  // planes z0-2 .. z0+2
-    issue_vel(z0, 0);
-    cp_async_commit();
+    next_vel();
     T wlo[VX];  // w on the face below plane z0 (own cells)
-    if (act) VV::ld(wlo, pw + (long long)wrapi(z0 - 1, nz) * planeP + (long long)(y0 + r) * P + GH + x0);
-    cp_async_wait<0>();
+    VV::ld(wlo, io.pu + 2 * io.vstride + wrapi(z0 - 1, nz) * planeP + (long long)(y0 + r) * P + x0);
+    // planes z0-2 (in the velocity slot of plane z0+2, free until then), z0-1 .. z0+2
+    constexpr int M2 = C::OVEL + 2 * C::VEL;
+    next_phi(IC<M2>{});
+    next_phi(IC<3 * C::PHI>{});
+    next_phi(IC<0>{});
+    next_phi(IC<C::PHI>{});
+    next_phi(IC<2 * C::PHI>{});
+    cp_async_commit();
+    if (z0 + 1 < z1) next_vel();
+    cp_async_commit();
+    cp_async_wait<1>();
     __syncthreads();
 
     // Prologue: s_z at plane z0-1 (own), s at plane z0 (own + ring), flux at z0-1/2.
-    T szc[VX], Fzm[VX], sxk[VX];  // sxk: the own group's s_x at plane k
-    {
-        const T *Pm2 = sphi, *Pm1 = sphi + S.phi, *P0 = sphi + 2 * S.phi, *P1 = sphi + 3 * S.phi;
-        T *const sx = ssx + (z0 & 1) * S.sx;
-        T *const sy = ssy + (z0 & 1) * S.sy;
-        if (act) {
-            T a0[VX], a1[VX], szm[VX], s0[VX], s1[VX];
-            sharp_group(Pm1, Pm2, P0, pos, a0, a1, szm);
-            sharp_group(P0, Pm1, P1, pos, s0, s1, szc);
-            VV::st(sx + sxo, s0);
+    // Carried: cK, ynK, ypK, LK, RK phi around the group at plane k; cN the group at plane
+    // k+1; sxK, szK its s_x, s_z at plane k; Fzm the flux through its lower z faces; rK the
+    // ring group at plane k.
+    T cK[VX], cN[VX], ynK[VX], ypK[VX], LK, RK, sxK[VX], szK[VX], Fzm[VX], rK[VX];
+    if (ring) {
+        T c[VX], yn[VX], yp[VX], zn[VX], zp[VX], s0[VX], s1[VX], s2[VX];
+        VV::ld(c, rg);
+        VV::ld(yn, rg - PS);
+        VV::ld(yp, rg + PS);
+        VV::ld(zn, rg + 3 * C::PHI);
+        VV::ld(zp, rg + C::PHI);
+        sharp(c, yn, yp, zn, zp, rg[-1], rg[VX], s0, s1, s2);
+        VV::st(rg - PS + C::OSY, s1);
 #pragma unroll
-            for (int i = 0; i < VX; ++i) sxk[i] = s0[i];
-            VV::st(sy + syo, s1);
-            T pm[VX], pc[VX];
-            VV::ld(pm, Pm1 + pos);
-            VV::ld(pc, P0 + pos);
-#pragma unroll
-            for (int i = 0; i < VX; ++i) Fzm[i] = flux(c_adv * wlo[i], c_dif, c_shp, pm[i], pc[i], szm[i], szc[i]);
-        }
-        sharp_ring(P0, Pm1, P1, sy);
+        for (int i = 0; i < VX; ++i) rK[i] = c[i];
     }
-    // plane z0+3 reuses the slot of plane z0-2, which the prologue just read
-    __syncthreads();
-    int zq = wrapi(z0 + 3, nz);  // wrapped index of the next phi plane to stage
-    if (z0 + 3 <= z1 + 1) issue_phi(zq, 0);
-    if (z0 + 1 < z1) issue_vel(z0 + 1, 1);
+    if (act) {
+        VV::ld(cK, b2);
+        VV::ld(ynK, b1);
+        VV::ld(ypK, b3);
+        VV::ld(cN, b2 + C::PHI);
+        LK = b2[-1];
+        RK = b2[VX];
+        T cm[VX], s1[VX];
+        VV::ld(cm, b2 + 3 * C::PHI);
+        sharp(cK, ynK, ypK, cm, cN, LK, RK, sxK, s1, szK);
+        VV::st(b1 + C::OSY, s1);
+        VV::st(b0 + C::OSX, sxK);
+        T ym[VX], yq[VX], zm[VX], a0[VX], a1[VX], szm[VX];
+        VV::ld(ym, b1 + 3 * C::PHI);
+        VV::ld(yq, b3 + 3 * C::PHI);
+        VV::ld(zm, b2 + M2);
+        sharp(cm, ym, yq, zm, cK, b2[3 * C::PHI - 1], b2[3 * C::PHI + VX], a0, a1, szm);
+#pragma unroll
+        for (int i = 0; i < VX; ++i) Fzm[i] = flux(c_adv * wlo[i], c_dif, c_shp, cm[i], cK[i], szm[i], szK[i]);
+    }
+    __syncthreads();  // the slots of planes z0-2 and z0-1 are free
+    if (z0 + 3 <= z1 + 1) next_phi(IC<3 * C::PHI>{});
     cp_async_commit();
 
-    PhiNb<T, VX> cur;  // phi around the own group at plane z0 (slot 2)
-    if (act) {
-        const T *const P0 = sphi + 2 * S.phi + pos;
-        VV::ld(cur.c, P0);
-        VV::ld(cur.yn, P0 - P);
-        VV::ld(cur.yp, P0 + P);
-        cur.L = P0[-1];
-        cur.R = P0[VX];
-    }
-    int pk = 2, vk = 0;  // ring slots of phi plane k and of the velocities of plane k
-    // two planes per pass: the carried values (cur / nxt, s_x, s_z, the z flux)
-    // alternate between two register sets instead of being copied
-#pragma unroll 2
-    for (int k = z0; k < z1; ++k) {
-        const int pk1 = pk == 4 ? 0 : pk + 1, pk2 = pk1 == 4 ? 0 : pk1 + 1;
-        const int pkm = pk == 0 ? 4 : pk - 1;  // also the slot of plane k+4
-        const int vk2 = vk == 0 ? 2 : vk - 1;  // also the slot of plane k+2
+    // the group at plane k of the output, and of the caller's array
+    T *op = io.pout + (long long)z0 * planeP + (long long)(y0 + r) * P + x0;
+    T *raw = io.raw ? io.raw + (long long)z0 * nx * ny + (long long)(y0 + r) * nx + x0 : nullptr;
+    const bool raw_v = nx % VX == 0 && ((size_t)io.raw & 15) == 0;
+    // One plane: S = (k - z0) mod 4; ACT: with the update.
+    auto body = [&](auto SC, auto ACT, const int k) {
+        constexpr int S = decltype(SC)::value, S1 = (S + 1) & 3, S2 = (S + 2) & 3;
+        constexpr int b = S & 1, bn = b ^ 1;
         // phi plane k+2 and the velocities of plane k have landed, and every thread
         // has left iteration k-1
         cp_async_wait<1>();
-        __syncthreads();
-        zq = zq + 1 == nz ? 0 : zq + 1;  // plane k+4
-        if (k + 4 <= z1 + 1) issue_phi(zq, pkm);
-        if (k + 2 < z1) issue_vel(k + 2, vk2);
+        asm volatile("bar.sync 0;" ::: "memory");  // (met from both loops)
+        if (k + 4 <= z1 + 1) next_phi(IC<S * C::PHI>{});
+        if (k + 2 < z1) next_vel();
         cp_async_commit();
 
-        const T *Pk = sphi + pk * S.phi, *Pk1 = sphi + pk1 * S.phi, *Pk2 = sphi + pk2 * S.phi;
-        T *const sxw = ssx + ((k + 1) & 1) * S.sx;
-        T *const syw = ssy + ((k + 1) & 1) * S.sy;
-        // sharpening at plane k+1: the ring rows, then the own group (s_z kept)
-        sharp_ring(Pk1, Pk, Pk2, syw);
-        if (act) {
-            T szn[VX];
-            PhiNb<T, VX> nxt;  // phi around the group at plane k+1
-            T sxn[VX];  // s_x of the group at plane k+1
+        // sharpening at plane k+1: the ring rows, then the own group
+        if (ring) {
+            const T *const R1 = rg + S1 * C::PHI;
+            T c[VX], yn[VX], yp[VX], zp[VX], s0[VX], s1[VX], s2[VX];
+            VV::ld(c, R1);
+            VV::ld(yn, R1 - PS);
+            VV::ld(yp, R1 + PS);
+            VV::ld(zp, rg + S2 * C::PHI);
+            sharp(c, yn, yp, rK, zp, R1[-1], R1[VX], s0, s1, s2);
+            VV::st(rg - PS + C::OSY + bn * C::SY, s1);
+#pragma unroll
+            for (int i = 0; i < VX; ++i) rK[i] = c[i];
+        }
+        if constexpr (decltype(ACT)::value) {
+            T cP[VX], ynN[VX], ypN[VX], sxN[VX], szN[VX];
+            VV::ld(cP, b2 + S2 * C::PHI);
+            VV::ld(ynN, b1 + S1 * C::PHI);
+            VV::ld(ypN, b3 + S1 * C::PHI);
+            const T LN = b2[S1 * C::PHI - 1], RN = b2[S1 * C::PHI + VX];
+            // the update's operands too, before the stores below (the compiler would not move a load
+            // over them): their latency passes under the sharpening
+            T syn[VX], syp[VX], uc[VX], vc[VX], vn[VX], wc[VX];
+            VV::ld(syn, b0 + C::OSY + b * C::SY);
+            VV::ld(syp, b2 + C::OSY + b * C::SY);
+            const T *const v0 = b0 + vrd;
+            VV::ld(uc, v0 + C::OVEL);
+            VV::ld(vn, v0 + C::OVEL + C::VO);
+            VV::ld(vc, b1 + vrd + C::OVEL + C::VO);
+            VV::ld(wc, v0 + C::OVEL + C::WO);
+            const T sxL = sL[C::OSX + b * C::SX], sxR = sR[C::OSX + b * C::SX], uL = v0[C::OVEL - 1];
             {
                 T s1[VX];
-                sharp_group(Pk1, Pk, Pk2, pos, sxn, s1, szn, cur.c, &nxt);
-                VV::st(sxw + sxo, sxn);
-                VV::st(syw + syo, s1);
+                sharp(cN, ynN, ypN, cK, cP, LN, RN, sxN, s1, szN);
+                VV::st(b1 + C::OSY + bn * C::SY, s1);
+                VV::st(b0 + C::OSX + bn * C::SX, sxN);
             }
-            // fluxes and update at plane k (s of plane k: buffer k & 1, written before the barrier)
-            const T *sx = ssx + (k & 1) * S.sx, *sy = ssy + (k & 1) * S.sy;
-            const T *vel = svel + vk * S.vel;
-            // phi around the group at plane k, carried from the previous iteration
-            const T *const c = cur.c, *const yn = cur.yn, *const yp = cur.yp, *const zp = nxt.c;
-            const T L = cur.L, R = cur.R;
-            const T *const sxc = sxk;
-            T syn[VX], syp[VX];
-            VV::ld(syn, sy + syo - P);
-            VV::ld(syp, sy + syo + P);
-            const T sxL = sx[sxo - 1 + dL], sxR = sx[sxo + VX + dR];
-            const T *ur = vel + r * P + GH + x0;
-            const T *vr = vel + S.vo + (r + 1) * P + GH + x0;
-            const T *wr = vel + S.wo + r * P + GH + x0;
-            T uc[VX], vc[VX], vn[VX], wc[VX];
-            VV::ld(uc, ur);
-            VV::ld(vc, vr);
-            VV::ld(vn, vr - P);
-            VV::ld(wc, wr);
-            const T uL = ur[-1];
+            // fluxes and update at plane k (s of plane k: written before the barrier)
             T o[VX];
 #pragma unroll
             for (int i = 0; i < VX; ++i) {
-                const T xl = i > 0 ? c[i - 1] : L, xr = i + 1 < VX ? c[i + 1] : R;
+                const T xl = i > 0 ? cK[i - 1] : LK, xr = i + 1 < VX ? cK[i + 1] : RK;
                 const T ul = i > 0 ? uc[i - 1] : uL;
-                const T sl = i > 0 ? sxc[i - 1] : sxL, sr = i + 1 < VX ? sxc[i + 1] : sxR;
-                T adv = uc[i] * (c[i] + xr);
-                adv = fma(-ul, xl + c[i], adv);
-                adv = fma(vc[i], c[i] + yp[i], adv);
-                adv = fma(-vn[i], yn[i] + c[i], adv);
-                const T dif = fma(T(-4), c[i], (xl + xr) + (yn[i] + yp[i]));
+                const T sl = i > 0 ? sxK[i - 1] : sxL, sr = i + 1 < VX ? sxK[i + 1] : sxR;
+                T adv = uc[i] * (cK[i] + xr);
+                adv = fma(-ul, xl + cK[i], adv);
+                adv = fma(vc[i], cK[i] + ypK[i], adv);
+                adv = fma(-vn[i], ynK[i] + cK[i], adv);
+                const T dif = fma(T(-4), cK[i], (xl + xr) + (ynK[i] + ypK[i]));
                 const T shp = (sr - sl) + (syp[i] - syn[i]);
-                const T Fzp = flux(c_adv * wc[i], c_dif, c_shp, c[i], zp[i], szc[i], szn[i]);
+                const T Fzp = flux(c_adv * wc[i], c_dif, c_shp, cK[i], cN[i], szK[i], szN[i]);
                 const T div = fma(c_adv, adv, fma(-c_dif, dif, fma(c_shp, shp, Fzp - Fzm[i])));
-                o[i] = fma(-c_upd, div, c[i]);
+                o[i] = fma(-c_upd, div, cK[i]);
                 Fzm[i] = Fzp;
-                szc[i] = szn[i];
-            }
-            // the padded copy of the next state: the group, and the ghost cells it feeds
-            T *const orow = pout + (long long)CDI_CHK(k, nz, st) * planeP + (long long)(y0 + r) * P + GH;
-            if (nown == VX) {
-                VV::st(orow + x0, o);
-            } else {
-#pragma unroll
-                for (int i = 0; i < VX; ++i)
-                    if (i < nown) orow[x0 + i] = o[i];
             }
             acc.template add_group_n<VX>(o, nown, a.c.tol);
-            if (gmask) {  // cells within GH of a row end: their ghost copies
-                if (nx >= GH) {
+            if (nown == VX) {
+                VV::st(op, o);
+            } else {
 #pragma unroll
-                    for (int i = 0; i < VX; ++i) {
-                        if ((gmask >> (2 * i)) & 1u) orow[x0 + i - nx] = o[i];
-                        if ((gmask >> (2 * i)) & 2u) orow[x0 + i + nx] = o[i];
-                    }
+                for (int i = 0; i < VX - 1; ++i)
+                    if (i < nown) op[i] = o[i];
+            }
+            if (x0 == 0 && nown > 0) {  // the row's continuation
+                op[nx] = o[0];
+                op[nx + 1] = nx > 1 ? o[1] : o[0];
+            }
+            if (raw) {  // the caller's array: rows on 16-byte boundaries, or at any element
+                if (raw_v) {
+                    if (nown > 0) VV::st(raw, o);
                 } else {
 #pragma unroll
-                    for (int i = 0; i < VX; ++i) {
-                        if (i >= nown) continue;
-                        const int x = x0 + i;
-                        for (int g = x - nx; g >= -GH; g -= nx) orow[g] = o[i];
-                        for (int g = x + nx; g < nx + GH; g += nx) orow[g] = o[i];
-                    }
+                    for (int i = 0; i < VX; ++i)
+                        if (i < nown) raw[i] = o[i];
                 }
+                raw += (long long)nx * ny;
             }
-            if (final_write) {  // the caller's array (rows at any 4-byte boundary: element stores)
-                T *const urow = a.out + (long long)k * plane + (long long)(y0 + r) * nx + x0;
 #pragma unroll
-                for (int i = 0; i < VX; ++i)
-                    if (i < nown) urow[i] = o[i];
+            for (int i = 0; i < VX; ++i) {
+                cK[i] = cN[i];
+                cN[i] = cP[i];
+                ynK[i] = ynN[i];
+                ypK[i] = ypN[i];
+                sxK[i] = sxN[i];
+                szK[i] = szN[i];
             }
-            cur = nxt;
-#pragma unroll
-            for (int i = 0; i < VX; ++i) sxk[i] = sxn[i];
+            LK = LN;
+            RK = RN;
         }
-        pk = pk1;
-        vk = vk == 2 ? 0 : vk + 1;
-    }
+        op += planeP;
+        vrd = vrd == 2 * C::VEL ? 0 : vrd + C::VEL;
+    };
+    auto planes = [&](auto ACT) {
+        for (int k = z0;;) {
+            body(IC<0>{}, ACT, k);
+            if (++k == z1) break;
+            body(IC<1>{}, ACT, k);
+            if (++k == z1) break;
+            body(IC<2>{}, ACT, k);
+            if (++k == z1) break;
+            body(IC<3>{}, ACT, k);
+            if (++k == z1) break;
+        }
+    };
+    if (act) planes(IC<1>{});
+    else planes(IC<0>{});
     cp_async_wait<0>();
 }
 
