@@ -241,6 +241,19 @@ CDI_API int cdi_step_adjoint(cdi_grid *g, const void *phi_k, const void *lam_nex
                      void *gu, void *gv, void *gw, double dt, double eps, double gamma,
                      double vel_scale, void *stream);
 
+/* A checkpoint segment's steps in one call each.  cdi_step_path: phi[i + 1] = one step of phi[i]
+ * with vel_scale[i], i = 0 .. nsteps - 1 (phi: nsteps + 1 arrays, neighbours not overlapping); the
+ * statistics record is the last step's, as after cdi_run.  cdi_adjoint_path: for i = nsteps - 1
+ * .. 0 the adjoint step at phi[i] with vel_scale[i], from lam_a to lam_b and back; *final_in_b is
+ * 1 if the result is in lam_b.  Arguments are otherwise those of cdi_step and cdi_step_adjoint;
+ * the arrays of pointers and scales are host memory, read during the call.  On an error, steps
+ * before the failing one may have been enqueued. */
+CDI_API int cdi_step_path(cdi_grid *g, void *const *phi, int nsteps, double dt, double eps, double gamma,
+                          const double *vel_scale, void *stream);
+CDI_API int cdi_adjoint_path(cdi_grid *g, void *const *phi, int nsteps, void *lam_a, void *lam_b, void *gu,
+                             void *gv, void *gw, double dt, double eps, double gamma,
+                             const double *vel_scale, int *final_in_b, void *stream);
+
 /* Boundedness condition (Eq. 17/24 with U the face maximum) and the Euler
  * diffusive limit A <= 1/(2 D_f) (Eq. 25).  Returns 1 if both hold, 0 if
  * not, CDI_ERR_ARG on bad input.  gamma_over_U = +inf is allowed.  A

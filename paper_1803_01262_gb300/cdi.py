@@ -80,6 +80,8 @@ SIGNATURES = {
     "cdi_mass_and_bounds": [_V, _V, _P(Stats), _V],
     "cdi_step_host": [_V, _V, _V, _Dbl, _Dbl, _Dbl, _Dbl, _I, _P(Stats), _V],
     "cdi_step_adjoint": [_V, _V, _V, _V, _V, _V, _V, _Dbl, _Dbl, _Dbl, _Dbl, _V],
+    "cdi_step_path": [_V, _P(_V), _I, _Dbl, _Dbl, _Dbl, _P(_Dbl), _V],
+    "cdi_adjoint_path": [_V, _P(_V), _I, _V, _V, _V, _V, _V, _Dbl, _Dbl, _Dbl, _P(_Dbl), _P(_I), _V],
     "cdi_check_condition": [_Dbl, _Dbl, _Dbl, _I],
     "cdi_max_dt": [_Dbl, _Dbl, _Dbl, _I, _I, _P(_Dbl)],
     "cdi_max_dt_mixed": [_Dbl, _Dbl, _Dbl, _P(_Dbl), _I, _I, _P(_Dbl)],
@@ -411,6 +413,31 @@ class Grid:
                                    self._arr(g[2], "gw"), dt, eps, gamma, vel_scale,
                                    _stream(stream)))
         return lam_k
+
+    def _path(self, states, scales):
+        return ((ctypes.c_void_p * len(states))(*[self._arr(t, "state") for t in states]),
+                (ctypes.c_double * len(scales))(*scales))
+
+    def step_path(self, states, dt, eps, gamma, scales, stream=None):
+        """states[i + 1] = one Euler step of states[i] with velocity scale scales[i] (native loop)."""
+        if len(states) != len(scales) + 1:
+            raise ValueError("a path of n steps has n + 1 states and n scales")
+        p, vs = self._path(states, scales)
+        _ck(lib().cdi_step_path(self._h, p, len(scales), dt, eps, gamma, vs, _stream(stream)))
+        return states[-1]
+
+    def adjoint_path(self, states, lam_a, lam_b, dt, eps, gamma, scales, grads=None, stream=None):
+        """The adjoint steps at states[-1] .. states[0] of lam_a, ping-ponging with lam_b (native
+        loop); returns (result, the other)."""
+        if len(states) != len(scales):
+            raise ValueError("n adjoint steps have n states and n scales")
+        g = grads if grads is not None else (None, None, None)
+        fb = ctypes.c_int()
+        p, vs = self._path(states, scales)
+        _ck(lib().cdi_adjoint_path(self._h, p, len(scales), self._arr(lam_a, "lam_a"), self._arr(lam_b, "lam_b"),
+                                   self._arr(g[0], "gu"), self._arr(g[1], "gv"), self._arr(g[2], "gw"), dt, eps,
+                                   gamma, vs, ctypes.byref(fb), _stream(stream)))
+        return (lam_b, lam_a) if fb.value else (lam_a, lam_b)
 
 
 class BoxDesc(ctypes.Structure):

@@ -357,18 +357,22 @@ cudaError_t adj_vec_resident(int *resident) { return adj_row_occ<T, false, true>
 template cudaError_t adj_vec_resident<float>(int *);
 template cudaError_t adj_vec_resident<double>(int *);
 
-// Persistent grid of the row kernel: every resident block, at most one per unit.
+// Persistent grid of the row kernel: every resident block (*blocks, of the grid's), at most one
+// per unit.
 template <typename T, bool VEL, bool AL>
-static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s)
+static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s, int *blocks)
 {
     using C = AdjRowCfg<T, kAdjRows>;
-    int resident = 0, dev = 0, sms = 0;
-    cudaError_t e;
-    if ((e = adj_row_occ<T, VEL, AL>(&resident)) != cudaSuccess) return e;
-    if (resident < 1) return cudaErrorInvalidConfiguration;
-    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-        return e;
+    if (*blocks == 0) {  // first launch of this grid: kept, for the queries take longer than the launch
+        int resident = 0, dev = 0, sms = 0;
+        cudaError_t e;
+        if ((e = adj_row_occ<T, VEL, AL>(&resident)) != cudaSuccess) return e;
+        if (resident < 1) return cudaErrorInvalidConfiguration;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+            (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+            return e;
+        *blocks = resident * sms;
+    }
     // zchunk < 0: balanced shares of the tile-planes (UnitIter; -2 rotated); else z chunks
     const long long tiles = (long long)((a.nx + C::W - 1) / C::W) * ((a.ny + C::H - 1) / C::H);
     int nchunks;
@@ -381,7 +385,7 @@ static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s)
         const int zc = (a.nz + nchunks - 1) / nchunks;
         units = tiles * ((a.nz + zc - 1) / zc);
     }
-    long long nb = (long long)resident * sms;
+    long long nb = *blocks;
     if (nb > units) nb = units;
     // programmatic stream serialisation: the launch may overlap the previous grid's
     // end (the kernel waits for it before touching anything it may write)
@@ -416,19 +420,21 @@ static cudaError_t launch_adj_t(const AdjArgs<T> &a, cudaStream_t s)
 }
 
 template <typename T>
-cudaError_t launch_adj(const AdjArgs<T> &a, int tile, cudaStream_t s)
+cudaError_t launch_adj(const AdjArgs<T> &a, int tile, cudaStream_t s, int *row_blocks)
 {
     switch (tile) {
     case 0: return launch_adj_t<T, 32, 8>(a, s);
     case 1: return launch_adj_t<T, 32, 16>(a, s);
     case 2: return launch_adj_t<T, 32, 4>(a, s);
-    case 3: return a.gu ? launch_adj_row<T, true, true>(a, s) : launch_adj_row<T, false, true>(a, s);
-    case 4: return a.gu ? launch_adj_row<T, true, false>(a, s) : launch_adj_row<T, false, false>(a, s);
+    case 3: return a.gu ? launch_adj_row<T, true, true>(a, s, row_blocks)
+                        : launch_adj_row<T, false, true>(a, s, row_blocks + 1);
+    case 4: return a.gu ? launch_adj_row<T, true, false>(a, s, row_blocks + 2)
+                        : launch_adj_row<T, false, false>(a, s, row_blocks + 3);
     default: return cudaErrorInvalidValue;
     }
 }
 
-template cudaError_t launch_adj<float>(const AdjArgs<float> &, int, cudaStream_t);
-template cudaError_t launch_adj<double>(const AdjArgs<double> &, int, cudaStream_t);
+template cudaError_t launch_adj<float>(const AdjArgs<float> &, int, cudaStream_t, int *);
+template cudaError_t launch_adj<double>(const AdjArgs<double> &, int, cudaStream_t, int *);
 
 }  // namespace cdi

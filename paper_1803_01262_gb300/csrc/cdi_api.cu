@@ -67,6 +67,7 @@ struct cdi_grid {
     int capacity;
     // launch configuration of the forward and adjoint kernels
     LaunchCfg fwd, adj;
+    int adj_blocks[4];         // launch_adj's resident blocks (0: not asked yet)
     LaunchCfg rk;  // Runge-Kutta stage kernels (set on first use; nblocks 0 = unset)
     LaunchCfg slab;  // z slabs of the pipelined host step (set on first use; nblocks 0 = unset)
     LaunchCfg tb;    // two steps per pass (cdi_run with depth 2; nblocks 0 = unset)
@@ -1196,7 +1197,7 @@ static int adjoint_t(cdi_grid *g, const void *phi, const void *lam, void *out, v
     a.status = g->status;
     if (cdi::adj_blocks(g->adj.tile, a.zchunk, g->nx, g->ny, g->nz) > g->capacity)
         return fail(CDI_ERR_STATE, "adjoint launch configuration out of range");
-    cudaError_t e = cdi::launch_adj<T>(a, g->adj.tile, s);
+    cudaError_t e = cdi::launch_adj<T>(a, g->adj.tile, s, g->adj_blocks);
     if (e != cudaSuccess) return cuda_fail(e, "adjoint step launch");
     return CDI_OK;
 }
@@ -1223,6 +1224,39 @@ int cdi_step_adjoint(cdi_grid *g, const void *phi_k, const void *lam_next, void 
         : adjoint_t<float>(g, phi_k, lam_next, lam_k, gu, gv, gw, dt, eps, gamma, vel_scale, s);
 }
 
+int cdi_step_path(cdi_grid *g, void *const *phi, int nsteps, double dt, double eps, double gamma,
+                  const double *vel_scale, void *stream)
+{
+    cdi::NvtxRange nvtx_("cdi_step_path");
+    if (nsteps < 0 || (nsteps > 0 && (!phi || !vel_scale))) return fail(CDI_ERR_ARG, "bad step path");
+    cudaStream_t s = (cudaStream_t)stream;
+    const bool defer = nsteps > 1 && 2 * (g ? g->fwd.nblocks : 0) <= (g ? g->capacity : 0);  // as in cdi_run
+    for (int i = 0; i < nsteps; ++i) {
+        if (int rc = check_step_args(g, phi[i], phi[i + 1], dt, eps, gamma, vel_scale[i])) return rc;
+        const DeferCfg d = {i & 1, i + 1 < nsteps, i > 0};
+        const DeferCfg *dp = defer ? &d : nullptr;
+        const int rc = g->dtype == CDI_F64
+            ? step_t<double>(g, phi[i], phi[i + 1], dt, eps, gamma, vel_scale[i], s, 0, 0, 0, 1, dp)
+            : step_t<float>(g, phi[i], phi[i + 1], dt, eps, gamma, vel_scale[i], s, 0, 0, 0, 1, dp);
+        if (rc) return rc;
+    }
+    return CDI_OK;
+}
+
+int cdi_adjoint_path(cdi_grid *g, void *const *phi, int nsteps, void *lam_a, void *lam_b, void *gu, void *gv,
+                     void *gw, double dt, double eps, double gamma, const double *vel_scale, int *final_in_b,
+                     void *stream)
+{
+    if (nsteps < 0 || (nsteps > 0 && (!phi || !vel_scale))) return fail(CDI_ERR_ARG, "bad adjoint path");
+    void *src = lam_a, *dst = lam_b;
+    for (int i = nsteps - 1; i >= 0; --i) {
+        if (int rc = cdi_step_adjoint(g, phi[i], src, dst, gu, gv, gw, dt, eps, gamma, vel_scale[i], stream))
+            return rc;
+        std::swap(src, dst);
+    }
+    if (final_in_b) *final_in_b = src != lam_a;
+    return CDI_OK;
+}
 
 int cdi_set_launch(cdi_grid *g, int which, int tile, int blocks_per_sm, int nchunks)
 {

@@ -162,8 +162,9 @@ template <typename T>
 cudaError_t launch_absmax(const T *u, const T *v, const T *w, long long n, RedScratch red,
                           int nblocks, cudaStream_t s);
 
+// row_blocks[4]: resident blocks of the row kernel's instantiations (0: not asked yet), kept by the grid.
 template <typename T>
-cudaError_t launch_adj(const AdjArgs<T> &a, int tile, cudaStream_t s);
+cudaError_t launch_adj(const AdjArgs<T> &a, int tile, cudaStream_t s, int *row_blocks);
 
 int adj_num_tiles();
 int adj_blocks(int tile, int zchunk, int nx, int ny, int nz);
