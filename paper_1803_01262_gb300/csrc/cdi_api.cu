@@ -252,16 +252,9 @@ static bool adj_vec_eligible(const cdi_grid *g) { return g->nx % (16 / (int)esiz
 // rows of 16 cells and more, as the forward step (fwd_default_tile; FP64 too: its formulas take
 // fewer FP64 operations); else a one-cell-per-thread tile with a z chunk giving about eight
 // blocks per SM.
-static LaunchCfg adj_default(const cdi_grid *g)
+static LaunchCfg adj_scalar_default(const cdi_grid *g)
 {
     LaunchCfg c;
-    if (g->nx >= 16) {
-        c.tile = adj_vec_eligible(g) ? 3 : 4;
-        c.zchunk = adj_vec_zchunk(g);
-        c.nblocks = 0;
-        c.nchunks = 0;
-        return c;
-    }
     c.tile = (g->nx >= 32 && g->ny >= 16) ? 1 : 2;
     const int bx = 32, by = c.tile == 1 ? 16 : 4;
     long long tiles = (long long)((g->nx + bx - 1) / bx) * ((g->ny + by - 1) / by);
@@ -270,6 +263,17 @@ static LaunchCfg adj_default(const cdi_grid *g)
     if (zc < kZMin) zc = kZMin;
     if (zc > g->nz) zc = g->nz;
     c.zchunk = (int)zc;
+    c.nblocks = 0;
+    c.nchunks = 0;
+    return c;
+}
+
+static LaunchCfg adj_default(const cdi_grid *g)
+{
+    if (g->nx < 16) return adj_scalar_default(g);
+    LaunchCfg c;
+    c.tile = adj_vec_eligible(g) ? 3 : 4;
+    c.zchunk = adj_vec_zchunk(g);
     c.nblocks = 0;
     c.nchunks = 0;
     return c;
@@ -1279,8 +1283,8 @@ int cdi_set_launch(cdi_grid *g, int which, int tile, int blocks_per_sm, int nchu
         if (tile >= cdi::adj_num_tiles()) return fail(CDI_ERR_ARG, "adjoint tile %d out of range", tile);
         if (tile == 3 && !adj_vec_eligible(g))
             return fail(CDI_ERR_ARG, "vector adjoint tile needs nx %% %d == 0", 16 / (int)esize(g));
-        LaunchCfg c = adj_default(g);
-        if (cdi::adj_tile_is_vec(tile) && !cdi::adj_tile_is_vec(c.tile)) c.zchunk = adj_vec_zchunk(g);
+        LaunchCfg c = adj_scalar_default(g);  // a row kernel's split may be one these tiles do not have
+        if (cdi::adj_tile_is_vec(tile)) c.zchunk = adj_vec_zchunk(g);
         c.tile = tile;
         if (nchunks > 0) c.zchunk = (g->nz + nchunks - 1) / nchunks;
         if (nchunks == CDI_NCHUNKS_BALANCED || nchunks == CDI_NCHUNKS_ROTATED) {
@@ -1294,7 +1298,6 @@ int cdi_set_launch(cdi_grid *g, int which, int tile, int blocks_per_sm, int nchu
         } else if (nchunks < 0) {
             return fail(CDI_ERR_ARG, "nchunks %d", nchunks);
         }
-        if (c.zchunk < 0 && !cdi::adj_tile_is_vec(c.tile)) c.zchunk = adj_default(g).zchunk;
         if (c.zchunk > 0 && cdi::adj_blocks(c.tile, c.zchunk, g->nx, g->ny, g->nz) > g->capacity)
             return fail(CDI_ERR_ARG, "adjoint configuration needs more blocks than the scratch holds");
         g->adj = c;
