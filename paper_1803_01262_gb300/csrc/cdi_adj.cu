@@ -345,7 +345,7 @@ void adj_vec_tile_dims(int esize, int *bw, int *bh)
 template <typename T, bool VEL, bool AL>
 static cudaError_t adj_row_occ(int *resident)
 {
-    using C = AdjRowCfg<T, kAdjRows>;
+    using C = AdjRowCfg<T, kAdjRows, AL>;
     auto kernel = adj_row_kernel<T, kAdjRows, VEL, AL>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::bytes);
     if (e != cudaSuccess) return e;
@@ -362,7 +362,7 @@ template cudaError_t adj_vec_resident<double>(int *);
 template <typename T, bool VEL, bool AL>
 static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s, int *blocks)
 {
-    using C = AdjRowCfg<T, kAdjRows>;
+    using C = AdjRowCfg<T, kAdjRows, AL>;
     if (*blocks == 0) {  // first launch of this grid: kept, for the queries take longer than the launch
         int resident = 0, dev = 0, sms = 0;
         cudaError_t e;

@@ -10,19 +10,22 @@
 //
 // FP32, aligned rows: 148 -> 105 instructions per cell; 256^3 100.5 -> 83.5 us per step (4.0 -> 4.8
 // TB/s), with velocity gradients 156 -> 142 us (5.7 TB/s); FP64 128^3 348 -> 316 us (fewer FP64
-// operations).  Other rows, against one cell per thread: 255^3 FP32 172.5 -> 130 us, with
-// gradients 322 -> 214 us; FP64 129^3 609 -> 389 us.
+// operations).  Other rows, against one cell per thread: 255^3 FP32 172.5 -> 106 us, with
+// gradients 322 -> 192 us; FP64 129^3 609 -> 384 us.
 #pragma once
 
 #include "cdi_row.cuh"
 
 namespace cdi {
 
-template <typename T, int TY>
+template <typename T, int TY, bool AL>
 struct AdjRowCfg : RowGeo<T, TY> {
     using G = RowGeo<T, TY>;
+    // velocity slots; other rows: two, which leaves L1 32 kB more (255^3 FP32 121 -> 106 us, with
+    // gradients 209 -> 192)
+    static constexpr int NVS = AL ? 4 : 2;
     static constexpr int OLAM = G::NS * G::PHI, OVEL = 2 * G::NS * G::PHI;
-    static constexpr int OGX = OVEL + G::NS * G::VEL, OGY = OGX + 2 * G::SXS;
+    static constexpr int OGX = OVEL + NVS * G::VEL, OGY = OGX + 2 * G::SXS;
     static constexpr size_t bytes = sizeof(T) * (size_t)(OGY + 2 * G::SYS);
     static_assert(G::VEL >= 2 * G::PHI, "the prologue's first planes borrow a velocity slot");
 };
@@ -53,10 +56,10 @@ __device__ __forceinline__ void red_add(double *p, const double *v, int n)
 
 // VEL: the velocity gradients are accumulated (a.gu, a.gv, a.gw not null).
 template <typename T, int TY, bool VEL, bool AL>
-__global__ void __launch_bounds__(AdjRowCfg<T, TY>::NT, 512 / AdjRowCfg<T, TY>::NT)
+__global__ void __launch_bounds__(AdjRowCfg<T, TY, AL>::NT, 512 / AdjRowCfg<T, TY, AL>::NT)
 adj_row_kernel(const AdjArgs<T> a, const int nchunks)
 {
-    using C = AdjRowCfg<T, TY>;
+    using C = AdjRowCfg<T, TY, AL>;
     using VV = V16<T>;
     constexpr int VX = C::VX, W = C::W, H = C::H, PP = C::PP, TX = C::TX, PHI = C::PHI;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -146,15 +149,17 @@ adj_row_kernel(const AdjArgs<T> a, const int nchunks)
             zq = zq + 1 == nz ? 0 : zq + 1;
         };
         // planes z0-2 (in the velocity slot of plane z0+3, free until then), z0-1 .. z0+2
-        constexpr int M2 = C::OVEL + 3 * C::VEL;
+        constexpr int M2 = C::OVEL + (C::NVS - 1) * C::VEL;
         next_planes(IC<M2>{}, IC<M2 + PHI>{});
         next_planes(IC<3 * PHI>{}, IC<C::OLAM + 3 * PHI>{});
         next_planes(IC<0>{}, IC<C::OLAM>{});
         next_planes(IC<PHI>{}, IC<C::OLAM + PHI>{});
         next_planes(IC<2 * PHI>{}, IC<C::OLAM + 2 * PHI>{});
         cp_async_commit();
-        if (z0 + 1 < z1) issue_vel(zo + plane, IC<C::OVEL + C::VEL>{});
-        if (z0 + 2 < z1) issue_vel(zo + 2 * plane, IC<C::OVEL + 2 * C::VEL>{});
+        if constexpr (C::NVS == 4) {
+            if (z0 + 1 < z1) issue_vel(zo + plane, IC<C::OVEL + C::VEL>{});
+            if (z0 + 2 < z1) issue_vel(zo + 2 * plane, IC<C::OVEL + 2 * C::VEL>{});
+        }
         cp_async_commit();
         cp_async_wait<1>();
         __syncthreads();
@@ -218,10 +223,16 @@ adj_row_kernel(const AdjArgs<T> a, const int nchunks)
             // left iteration k-1.
             cp_async_wait<1>();
             __syncthreads();
+            if constexpr (C::NVS == 2) {  // a group of its own: landed at the next barrier
+                if (k + 1 < z1) issue_vel(zo + plane, IC<C::OVEL + b1 * C::VEL>{});
+                cp_async_commit();
+            }
             if (k + 4 <= z1 + 1) next_planes(IC<S * PHI>{}, IC<C::OLAM + S * PHI>{});
-            if (k + 3 < z1) issue_vel(zo + 3 * plane, IC<C::OVEL + ((S + 3) & 3) * C::VEL>{});
+            if constexpr (C::NVS == 4) {
+                if (k + 3 < z1) issue_vel(zo + 3 * plane, IC<C::OVEL + ((S + 3) & 3) * C::VEL>{});
+            }
             cp_async_commit();
-            if (!AL && k + 5 < z1) {
+            if (!AL && !VEL && k + 5 < z1) {
                 const long long zp = zo + 5 * plane;
                 cp.ahead(a.u + zp);
                 cp.ahead(a.v + zp);
@@ -263,7 +274,7 @@ adj_row_kernel(const AdjArgs<T> a, const int nchunks)
                 VV::st(bp + C::OGX + b1 * C::SXS - PP, gxN);
                 // C: lam at plane k.
                 const T *gx = bp + C::OGX + b * C::SXS - PP, *gy = bp + C::OGY + b * C::SYS;
-                const T *vel = bp + C::OVEL + S * C::VEL;
+                const T *vel = bp + C::OVEL + (S & (C::NVS - 1)) * C::VEL;
                 T gyn[VX], gyp[VX], uc[VX], vc[VX], vn[VX], wc[VX];
                 VV::ld(gyn, gy - PP);
                 VV::ld(gyp, gy + PP);

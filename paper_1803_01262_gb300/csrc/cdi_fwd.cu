@@ -445,15 +445,19 @@ void fwd_tile_dims(int tile, int esize, int *bw, int *bh)
 // unless the 6-row one covers ny with less work (each tile row of blocks pays two ring rows),
 // else one cell per thread.  FP64, whose time is FP64 instructions, takes the vector kernel on
 // aligned rows of 48 cells and more, and the row kernel on other rows of 64 and more
-// (129^3: 306 us with the 32x16 tile, 289 us).
-int fwd_default_tile(int esize, int nx, int ny)
+// (129^3: 306 us with the 32x16 tile, 289 us).  Unaligned FP32 rows of boxes whose arrays do not
+// stay in L2 (4 M cells: 80 MB) take the 6-row tile, whose four blocks per SM leave L1 more room
+// than the 14-row tile's two (row_vel_slots): 255^3 90.1 -> 83.9 us, 160x177x190 31.7 -> 31.0;
+// below, the 14-row one is faster (129^3 19.4 against 20.9 us).
+int fwd_default_tile(int esize, int nx, int ny, int nz)
 {
     const int vx = 16 / esize;
     const bool al = nx % vx == 0;
     if (esize == 4 ? nx >= 16 : (al ? nx >= 48 : nx >= 64)) {
         if (esize == 8 && al) return ny >= 12 ? 4 : 5;
         const int w14 = (ny + 13) / 14 * 16, w6 = (ny + 5) / 6 * 8;
-        return (w6 < w14 ? 5 : 4) + (al ? 0 : 3);
+        const bool big = esize == 4 && !al && (long long)nx * ny * nz >= 4000000;
+        return (w6 < w14 || big ? 5 : 4) + (al ? 0 : 3);
     }
     return (nx >= 32 && ny >= 16) ? 1 : 3;
 }
@@ -473,11 +477,19 @@ static cudaError_t occ(K kernel, int threads, size_t smem, int *resident)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, kernel, threads, smem);
 }
 
+// Velocity slots of the row kernel.  Rows staged by elements, plain steps: two, the velocities one
+// plane ahead, for the copies pass through L1, whose lines bound the bytes in flight: what shared
+// memory leaves of it counts for more than the distance (301x257x211 FP32, 6-row tile: 91.0 us
+// with four slots, 84.2 with two; with L1 squeezed by 32 kB more, 126).  Else four.
+template <bool RK, bool ZR, bool AL>
+constexpr int row_vel_slots() { return !AL && !RK && !ZR ? 2 : 4; }
+
 template <typename T, int TY, bool AL, bool RK = false, bool ZR = false>
 static cudaError_t row_occ(int *resident)
 {
-    using C = RowCfg<T, TY, RK>;
-    return occ(fwd_row_kernel<T, TY, RK, ZR, AL>, C::NT, C::bytes, resident);
+    constexpr int NV = row_vel_slots<RK, ZR, AL>();
+    using C = RowCfg<T, TY, RK, NV>;
+    return occ(fwd_row_kernel<T, TY, RK, ZR, AL, NV>, C::NT, C::bytes, resident);
 }
 
 // Runge-Kutta stage kernels exist for tiles 1, 3 (one cell per thread), 4 and 7 (vectors) only.
@@ -554,8 +566,9 @@ static cudaError_t launch_dependent(K kernel, int nblocks, int threads, size_t s
 template <typename T, int TY, bool AL, bool RK = false, bool ZR = false>
 static cudaError_t row_launch(const FwdArgs<T> &a, int nblocks, int nchunks, cudaStream_t s)
 {
-    using C = RowCfg<T, TY, RK>;
-    return launch_dependent(fwd_row_kernel<T, TY, RK, ZR, AL>, nblocks, C::NT, C::bytes, s, a, nchunks);
+    constexpr int NV = row_vel_slots<RK, ZR, AL>();
+    using C = RowCfg<T, TY, RK, NV>;
+    return launch_dependent(fwd_row_kernel<T, TY, RK, ZR, AL, NV>, nblocks, C::NT, C::bytes, s, a, nchunks);
 }
 
 template <typename T>

@@ -22,8 +22,9 @@
 //   AL = true   rows start on 16-byte boundaries (nx % VX == 0): 16-byte cp.async and stores.
 //   AL = false  rows start at any element: a warp copies its rows element by element (a lane
 //               per column: contiguous runs) and stores element by element (through shared
-//               memory, for contiguous stores: 89.1 against 86.4 us at 255^3).  255^3 FP32:
-//               139 us with one cell per thread (32x8 tile) -> 86.4 us; 385^3 501 -> 317 us.
+//               memory, for contiguous stores: 89.1 against 86.4 us at 255^3 with the
+//               14-row tile).  255^3 FP32:
+//               139 us with one cell per thread (32x8 tile) -> 83.6 us; 385^3 501 -> 308 us.
 // The arithmetic is that of every other forward kernel, in the same order: the fields are the
 // same bit for bit.
 #pragma once
@@ -35,21 +36,22 @@
 
 namespace cdi {
 
-template <typename T, int TY, bool RK = false>
+template <typename T, int TY, bool RK, int NV>
 struct RowCfg : RowGeo<T, TY> {
     using G = RowGeo<T, TY>;
-    static constexpr int OVEL = G::NS * G::PHI, OSX = OVEL + G::NS * G::VEL, OSY = OSX + 2 * G::SXS;
+    static constexpr int NVS = NV;            // velocity slots
+    static constexpr int OVEL = G::NS * G::PHI, OSX = OVEL + NVS * G::VEL, OSY = OSX + 2 * G::SXS;
     static constexpr int RKO = G::H * G::W;   // a plane of one Runge-Kutta operand (RK: two operands, two slots)
     static constexpr int ORK = OSY + 2 * G::SYS;
     static constexpr size_t bytes = sizeof(T) * (size_t)(ORK + (RK ? 4 * RKO : 0));
     static_assert(G::VEL >= G::PHI, "the prologue's first phi plane borrows a velocity slot");
 };
 
-template <typename T, int TY, bool RK, bool ZR, bool AL>
-__global__ void __launch_bounds__(RowCfg<T, TY, RK>::NT, 512 / RowCfg<T, TY, RK>::NT)
+template <typename T, int TY, bool RK, bool ZR, bool AL, int NV>
+__global__ void __launch_bounds__(RowCfg<T, TY, RK, NV>::NT, 512 / RowCfg<T, TY, RK, NV>::NT)
 fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
 {
-    using C = RowCfg<T, TY, RK>;
+    using C = RowCfg<T, TY, RK, NV>;
     using VV = V16<T>;
     constexpr int VX = C::VX, W = C::W, H = C::H, PP = C::PP, TX = C::TX;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -159,7 +161,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
             zq = zq + 1 == nz ? 0 : zq + 1;
         };
         // planes z0-2 (in the velocity slot of plane z0+3, free until then), z0-1 .. z0+2
-        constexpr int M2 = C::OVEL + 3 * C::VEL;
+        constexpr int M2 = C::OVEL + (C::NVS - 1) * C::VEL;
         next_phi(IC<M2>{});
         next_phi(IC<3 * C::PHI>{});
         next_phi(IC<0>{});
@@ -167,8 +169,10 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
         next_phi(IC<2 * C::PHI>{});
         if constexpr (RK) issue_rk(zo, IC<0>{});
         cp_async_commit();
-        if (z0 + 1 < z1) issue_vel(zo + plane, IC<C::OVEL + C::VEL>{});
-        if (z0 + 2 < z1) issue_vel(zo + 2 * plane, IC<C::OVEL + 2 * C::VEL>{});
+        if constexpr (C::NVS == 4) {
+            if (z0 + 1 < z1) issue_vel(zo + plane, IC<C::OVEL + C::VEL>{});
+            if (z0 + 2 < z1) issue_vel(zo + 2 * plane, IC<C::OVEL + 2 * C::VEL>{});
+        }
         cp_async_commit();
         cp_async_wait<1>();
         __syncthreads();
@@ -222,12 +226,17 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
             // has left iteration k-1.
             cp_async_wait<1>();
             __syncthreads();
-            if constexpr (RK) {  // a group of its own, before plane k+4's: landed at the next barrier
-                if (k + 1 < z1) issue_rk(zo + plane, IC<b1>{});
+            if constexpr (RK || C::NVS == 2) {  // a group of its own, before plane k+4's: landed at the next barrier
+                if (k + 1 < z1) {
+                    if constexpr (RK) issue_rk(zo + plane, IC<b1>{});
+                    if constexpr (C::NVS == 2) issue_vel(zo + plane, IC<C::OVEL + b1 * C::VEL>{});
+                }
                 cp_async_commit();
             }
             if (k + 4 <= z1 + 1) next_phi(IC<S * C::PHI>{});
-            if (k + 3 < z1) issue_vel(zo + 3 * plane, IC<C::OVEL + ((S + 3) & 3) * C::VEL>{});
+            if constexpr (C::NVS == 4) {
+                if (k + 3 < z1) issue_vel(zo + 3 * plane, IC<C::OVEL + ((S + 3) & 3) * C::VEL>{});
+            }
             cp_async_commit();
 
             // B: sharpening at plane k+1 (every warp).
@@ -257,7 +266,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
                 // C: fluxes and update at plane k (x and y faces telescoped, the z face
                 // below carried).
                 const T *sx = bp + C::OSX + b * C::SXS - PP, *sy = bp + C::OSY + b * C::SYS;
-                T *const vel = bp + C::OVEL + S * C::VEL;
+                T *const vel = bp + C::OVEL + (S & (C::NVS - 1)) * C::VEL;
                 T syn[VX], syp[VX], uc[VX], vc[VX], vn[VX], wc[VX];
                 VV::ld(syn, sy - PP);
                 VV::ld(syp, sy + PP);
@@ -265,7 +274,8 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
                 VV::ld(vc, vel + C::VO);
                 VV::ld(vn, vel + C::VO - PP);
                 VV::ld(wc, vel + C::WO - PP);
-                const T sxL = sx[-1], sxR = sx[VX], uL = vel[-PP - 1];
+                const T sxL = sx[-1], sxR = sx[VX];
+                const T uL = vel[-PP - 1];
                 T o[VX];
 #pragma unroll
                 for (int i = 0; i < VX; ++i) {

@@ -129,8 +129,9 @@ struct RowStage {
     // AL = false: ask for the own warp's two rows of a plane (src its first element) in L2, a
     // line at a time.  The element copies pass through L1, whose lines (what shared memory leaves
     // of it) bound the bytes in flight; with the rows in L2 a copy holds its line for an L2, not a
-    // memory, latency.  For the adjoint, whose rings leave L1 the least: 255^3 FP32 145 -> 130 us.
-    // (The forward kernel gained nothing; cp.async.bulk.prefetch, one per row, took 238 us.)
+    // memory, latency.  For the adjoint without velocity gradients, whose rings leave L1 the least:
+    // 255^3 FP32 109 -> 106 us.  (The others gained nothing; cp.async.bulk.prefetch, one per row,
+    // took twice as long.)
     __device__ __forceinline__ void ahead(const T *src) const
     {
         if constexpr (!AL) {
