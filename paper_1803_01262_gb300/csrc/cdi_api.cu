@@ -291,10 +291,11 @@ static int plane_setup(cdi_grid *g)
     const size_t bytes = g->dtype == CDI_F64 ? cdi::plane_word_bytes<double>(g->nx, g->plane_bands)
                                              : cdi::plane_word_bytes<float>(g->nx, g->plane_bands);
     const unsigned one = 1u;
-    if ((e = cudaMalloc(&g->plane_words, bytes)) != cudaSuccess ||
-        (e = cudaMalloc(&g->plane_tag, sizeof(unsigned))) != cudaSuccess ||
-        (e = cudaMemset(g->plane_words, 0, bytes)) != cudaSuccess ||
-        (e = cudaMemcpy(g->plane_tag, &one, sizeof(one), cudaMemcpyHostToDevice)) != cudaSuccess)
+    if ((e = cudaMalloc(&g->plane_words, bytes + sizeof(unsigned))) != cudaSuccess ||
+        (e = cudaMemset(g->plane_words, 0, bytes)) != cudaSuccess)
+        return cuda_fail(e, "halo words");
+    g->plane_tag = (unsigned *)((char *)g->plane_words + bytes);  // the tag counter, after the words
+    if ((e = cudaMemcpy(g->plane_tag, &one, sizeof(one), cudaMemcpyHostToDevice)) != cudaSuccess)
         return cuda_fail(e, "halo words");
     g->plane_on = true;
     return CDI_OK;
@@ -382,7 +383,6 @@ int cdi_destroy_grid(cdi_grid *g)
     cudaFree(g->rec2);
     cudaFree(g->status);
     cudaFree(g->plane_words);
-    cudaFree(g->plane_tag);
     cudaFree(g->stage_in);
     cudaFree(g->stage_out);
     delete g;

@@ -387,7 +387,7 @@ fwd_vec_kernel(const FwdArgs<T> a, const int nchunks)
     }
     if (!dep_waited) grid_dep_wait();
     grid_dep_launch();  // the next step may start staging its velocities
-    reduce_and_finish<ZR>(acc, a.red);
+    if (!RK || a.red.update_run) reduce_and_finish<ZR>(acc, a.red);  // (the record is the last stage's)
 }
 
 // ===========================================================================
@@ -410,7 +410,7 @@ fwd_kernel(const FwdArgs<T> a, const int nchunks)
         else
             scalar_unit<T, BX, BY, RK, SCALAR_PF, FACE>(a, un, acc, smem_raw);
     }
-    reduce_and_finish(acc, a.red);
+    if (!RK || a.red.update_run) reduce_and_finish(acc, a.red);  // (the record is the last stage's)
 }
 
 // ===========================================================================

@@ -110,6 +110,8 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
 
     Acc<T> acc;
     acc.init();
+    // The record is the last Runge-Kutta stage's, which overwrites the others': they skip it.
+    const bool stats = !RK || a.red.update_run;
     bool dep_waited = false;  // the previous grid on the stream has completed
 
     const int zlo = ZR ? a.z_lo : 0, zr = ZR ? a.z_hi - a.z_lo : nz;
@@ -323,10 +325,10 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
                 if constexpr (AL) {
                     if (nown > 0) {
                         VV::st(op + cp.g[0], o);
-                        acc.template add_group<VX>(o, a.c.tol);
+                        if (stats) acc.template add_group<VX>(o, a.c.tol);
                     }
                 } else {
-                    if (nown > 0) acc.template add_group_n<VX>(o, nown, a.c.tol);
+                    if (stats && nown > 0) acc.template add_group_n<VX>(o, nown, a.c.tol);
 #pragma unroll
                     for (int i = 0; i < VX; ++i)
                         if (i < nown) op[go + i] = o[i];
@@ -360,7 +362,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
     }
     if (!dep_waited) grid_dep_wait();
     grid_dep_launch();  // the next step may start staging its velocities
-    reduce_and_finish<ZR>(acc, a.red);
+    if (stats) reduce_and_finish<ZR>(acc, a.red);
 }
 
 }  // namespace cdi
