@@ -477,17 +477,18 @@ static cudaError_t occ(K kernel, int threads, size_t smem, int *resident)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, kernel, threads, smem);
 }
 
-// Velocity slots of the row kernel.  Rows staged by elements, plain steps: two, the velocities one
-// plane ahead, for the copies pass through L1, whose lines bound the bytes in flight: what shared
-// memory leaves of it counts for more than the distance (301x257x211 FP32, 6-row tile: 91.0 us
-// with four slots, 84.2 with two; with L1 squeezed by 32 kB more, 126).  Else four.
-template <bool RK, bool ZR, bool AL>
-constexpr int row_vel_slots() { return !AL && !RK && !ZR ? 2 : 4; }
+// Velocity slots of the row kernel.  Rows staged by elements: two, the velocities one plane ahead,
+// for the copies pass through L1, whose lines bound the bytes in flight: what shared memory leaves
+// of it counts for more than the distance (301x257x211 FP32, 6-row tile: 91.0 us with four slots,
+// 84.2 with two; RK4 at 255^3, whose stage operands take shared memory too: 568 and 460 us).
+// Aligned rows, and the slabs of the host step (timed so only): four.
+template <bool ZR, bool AL>
+constexpr int row_vel_slots() { return !AL && !ZR ? 2 : 4; }
 
 template <typename T, int TY, bool AL, bool RK = false, bool ZR = false>
 static cudaError_t row_occ(int *resident)
 {
-    constexpr int NV = row_vel_slots<RK, ZR, AL>();
+    constexpr int NV = row_vel_slots<ZR, AL>();
     using C = RowCfg<T, TY, RK, NV>;
     return occ(fwd_row_kernel<T, TY, RK, ZR, AL, NV>, C::NT, C::bytes, resident);
 }
@@ -566,7 +567,7 @@ static cudaError_t launch_dependent(K kernel, int nblocks, int threads, size_t s
 template <typename T, int TY, bool AL, bool RK = false, bool ZR = false>
 static cudaError_t row_launch(const FwdArgs<T> &a, int nblocks, int nchunks, cudaStream_t s)
 {
-    constexpr int NV = row_vel_slots<RK, ZR, AL>();
+    constexpr int NV = row_vel_slots<ZR, AL>();
     using C = RowCfg<T, TY, RK, NV>;
     return launch_dependent(fwd_row_kernel<T, TY, RK, ZR, AL, NV>, nblocks, C::NT, C::bytes, s, a, nchunks);
 }
