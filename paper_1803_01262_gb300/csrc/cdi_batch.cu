@@ -1187,6 +1187,43 @@ int cdi_batch_step(cdi_batch *b, double vel_scale, void *stream)
     return rc;
 }
 
+// Counters of a run's launches: one pair each, the box epochs.
+static int reserve_run(cdi_batch *b, int nsteps)
+{
+    if (nsteps <= b->run_cap) return CDI_OK;
+    cudaError_t e;
+    if ((e = cudaDeviceSynchronize()) != cudaSuccess)  // no graph in flight uses the old counters
+        return cdi::set_error(CDI_ERR_CUDA, "batch run: %s", cudaGetErrorString(e));
+    drop_graphs(b);
+    cudaFree(b->run_queue);
+    b->run_queue = nullptr;
+    b->run_cap = 0;
+    if ((e = cudaMalloc(&b->run_queue, sizeof(unsigned int) * 2 * (size_t)nsteps)) != cudaSuccess) {
+        b->run_queue = nullptr;
+        return cdi::set_error(CDI_ERR_CUDA, "batch run counters: %s", cudaGetErrorString(e));
+    }
+    b->run_cap = nsteps;
+    return CDI_OK;
+}
+
+static int zero_run(cdi_batch *b, int nsteps, cudaStream_t s)
+{
+    cudaError_t e;
+    if ((e = cudaMemsetAsync(b->run_queue, 0, sizeof(unsigned int) * 2 * (size_t)nsteps, s)) != cudaSuccess ||
+        (e = cudaMemsetAsync(b->epoch, 0, sizeof(unsigned int) * b->nbox, s)) != cudaSuccess ||
+        (e = cudaMemsetAsync(b->box_done, 0, sizeof(unsigned int) * b->nbox, s)) != cudaSuccess)
+        return cdi::set_error(CDI_ERR_CUDA, "batch run counters: %s", cudaGetErrorString(e));
+    return CDI_OK;
+}
+
+// Launch i of a run.  A unit waits at most about one step: one second plus 2 ns per cell (a step of
+// the slowest tile takes well under 1 ns per cell).
+static cdi::BatchSync run_sync(const cdi_batch *b, int i)
+{
+    const unsigned long long wait_ns = 1000000000ull + 2ull * (unsigned long long)b->cells;
+    return {b->run_queue + 2 * i, b->epoch, i, 0, wait_ns};
+}
+
 int cdi_batch_run(cdi_batch *b, int nsteps, void *stream)
 {
     cdi::NvtxRange nvtx_("cdi_batch_run");
@@ -1201,36 +1238,17 @@ int cdi_batch_run(cdi_batch *b, int nsteps, void *stream)
     const std::pair<int, int> key(nsteps, b->parity);
     auto it = b->graphs.find(key);
     if (it == b->graphs.end()) {
-        if (nsteps > b->run_cap) {  // one counter pair per launch of the run
-            if ((e = cudaDeviceSynchronize()) != cudaSuccess)  // no graph in flight uses the old counters
-                return cdi::set_error(CDI_ERR_CUDA, "batch run: %s", cudaGetErrorString(e));
-            drop_graphs(b);
-            cudaFree(b->run_queue);
-            b->run_queue = nullptr;
-            b->run_cap = 0;
-            if ((e = cudaMalloc(&b->run_queue, sizeof(unsigned int) * 2 * (size_t)nsteps)) != cudaSuccess) {
-                b->run_queue = nullptr;
-                return cdi::set_error(CDI_ERR_CUDA, "batch run counters: %s", cudaGetErrorString(e));
-            }
-            b->run_cap = nsteps;
-        }
+        if (int rc = reserve_run(b, nsteps)) return rc;
         // Capture nsteps launches (parity alternating) once on the private stream:
         // the run's counters and box epochs zeroed, then the steps, each after the
         // first overlapping the one before (BatchSync).
         cudaGraph_t graph;
         if ((e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
             return cdi::set_error(CDI_ERR_CUDA, "begin capture: %s", cudaGetErrorString(e));
-        int rc = CDI_OK;
-        if ((e = cudaMemsetAsync(b->run_queue, 0, sizeof(unsigned int) * 2 * (size_t)nsteps, b->cap)) != cudaSuccess ||
-            (e = cudaMemsetAsync(b->epoch, 0, sizeof(unsigned int) * b->nbox, b->cap)) != cudaSuccess ||
-            (e = cudaMemsetAsync(b->box_done, 0, sizeof(unsigned int) * b->nbox, b->cap)) != cudaSuccess)
-            rc = cdi::set_error(CDI_ERR_CUDA, "batch run counters: %s", cudaGetErrorString(e));
+        int rc = zero_run(b, nsteps, b->cap);
         if (rc == CDI_OK && b->tile == cdi::BATCH_TILE_VBAND) rc = vband_pack_state(b, b->parity, b->cap);
-        // a unit waits at most about one step: one second plus 2 ns per cell (a step
-        // of the slowest tile takes well under 1 ns per cell)
-        const unsigned long long wait_ns = 1000000000ull + 2ull * (unsigned long long)b->cells;
         for (int i = 0; i < nsteps && rc == CDI_OK; ++i) {
-            const cdi::BatchSync y = {b->run_queue + 2 * i, b->epoch, i, 0, wait_ns};
+            const cdi::BatchSync y = run_sync(b, i);
             rc = launch_any(b, b->parity ^ (i & 1), 1.0, b->cap, i == nsteps - 1, &y);
         }
         e = cudaStreamEndCapture(b->cap, &graph);
@@ -1375,7 +1393,7 @@ int cdi_batch_autotune(cdi_batch *b, int reps, float *best_ms, void *stream)
     const int nz_opts = b->flat ? 1 : (int)(sizeof(zopts) / sizeof(int));
     int best_tile = b->tile, best_z = b->zdepth, rc = CDI_OK;
     float best_t = 1e30f;
-    for (int tile = 0; tile < cdi::BATCH_TILES && rc == CDI_OK; ++tile) {
+    for (int tile = cdi::BATCH_TILES - 1; tile >= 0 && rc == CDI_OK; --tile) {  // the likely ones first
         if (tile == cdi::BATCH_TILE_PLANE && b->plane_bytes == 0) continue;
         if (tile == cdi::BATCH_TILE_BAND && b->band_bytes == 0) continue;
         if (tile == cdi::BATCH_TILE_VBAND && b->vband_bytes == 0) continue;
@@ -1388,21 +1406,35 @@ int cdi_batch_autotune(cdi_batch *b, int reps, float *best_ms, void *stream)
             // not storing the state before the last, so that they too only read the state)
             constexpr int kTrial = 9;
             const bool pr = plane_run_applies(b, kTrial);
-            auto trial = [&]() { return pr ? plane_run(b, kTrial, false, s) : launch_any(b, b->parity, 1.0, s, 0); };
-            if ((rc = trial()) != CDI_OK) break;  // warm-up
-            if ((e = cudaEventRecord(e0, s)) != cudaSuccess) {
-                rc = cdi::set_error(CDI_ERR_CUDA, "event: %s", cudaGetErrorString(e));
-                break;
-            }
-            for (int i = 0; i < reps && rc == CDI_OK; ++i) rc = trial();
-            if (rc != CDI_OK) break;
-            if ((e = cudaEventRecord(e1, s)) != cudaSuccess || (e = cudaEventSynchronize(e1)) != cudaSuccess) {
-                rc = cdi::set_error(CDI_ERR_CUDA, "event: %s", cudaGetErrorString(e));
-                break;
-            }
+            // the others as a run's launches are made, each overlapping the one before, but all from
+            // the current state to the other buffer.  (Timed one after another, 60 boxes of 16..100
+            // cells took 16 planes per unit: 755 us for 8 steps against 673 with 32.)
+            const int n = reps > 6 ? reps : 6;
+            if (!pr && (rc = reserve_run(b, n)) != CDI_OK) break;
+            auto trial = [&](int k) {
+                if (pr) return plane_run(b, kTrial, false, s);
+                int r = zero_run(b, k, s);
+                for (int i = 0; i < k && r == CDI_OK; ++i) {
+                    const cdi::BatchSync y = run_sync(b, i);
+                    r = launch_any(b, b->parity, 1.0, s, 0, &y);
+                }
+                return r;
+            };
+            auto timed = [&](int k, float *ms) {  // of the k launches (tile 4: of reps runs)
+                if ((e = cudaEventRecord(e0, s)) != cudaSuccess)
+                    return cdi::set_error(CDI_ERR_CUDA, "event: %s", cudaGetErrorString(e));
+                for (int i = 0; i < (pr && k > 1 ? reps : 1); ++i)
+                    if (int r = trial(k)) return r;
+                if ((e = cudaEventRecord(e1, s)) != cudaSuccess || (e = cudaEventSynchronize(e1)) != cudaSuccess ||
+                    (e = cudaEventElapsedTime(ms, e0, e1)) != cudaSuccess)
+                    return cdi::set_error(CDI_ERR_CUDA, "event: %s", cudaGetErrorString(e));
+                *ms /= pr ? (k > 1 ? reps : 1) * kTrial : k;
+                return (int)CDI_OK;
+            };
             float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            ms /= pr ? reps * kTrial : reps;
+            if ((rc = timed(1, &ms)) != CDI_OK) break;  // warm-up
+            if (ms > 3.f * best_t) continue;
+            if ((rc = timed(n, &ms)) != CDI_OK) break;
             if (ms < best_t) {
                 best_t = ms;
                 best_tile = tile;
