@@ -22,13 +22,14 @@
 // every array.  Its expressions in its order: the field is the other kernels' bit for
 // bit.
 //
-// What bounds it: latency (16 warps per SM, one barrier per plane; 60% of the issue slots, DRAM
-// and L2 at 60% and 32% of their rates).  Fewer rows per band, so that no thread has a ring group
-// besides its own, took 20% longer.  64 FP32 boxes with edges 32..160 (65 M cells): 143 -> 107
-// instructions per cell, 341 -> 304 us per step of a run (with the ghost cells at both ends of a
-// row kept by the stores, slots at run-time offsets, a condition per thread around the update and
-// its operands loaded after the sharpening).  The output goes to the padded copy of the next state and, on the last step of a
-// call (final_write), also to the caller's array.
+// What bounds it: latency (16 warps per SM, one barrier per plane; 54% of the issue slots, the L1
+// data pipe at 55%, DRAM at 50% of its rate).  Fewer rows per band, so that no thread has a ring
+// group besides its own, took 20% longer; 512 threads, one block per SM, 10%.  64 FP32 boxes with
+// edges 32..160 (65 M cells): 143 -> 107 instructions per cell, 341 -> 304 us per step of a run;
+// before, the stores kept ghost cells at both ends of every row, the slots lay at run-time offsets,
+// a condition per thread stood around the update, and its operands were loaded after the
+// sharpening.  The output goes to the padded copy of the next state and, on the last step of a call
+// (final_write), also to the caller's array.
 #pragma once
 
 #include "cdi_async.cuh"
