@@ -342,31 +342,31 @@ void adj_vec_tile_dims(int esize, int *bw, int *bh)
     *bh = kAdjRows;
 }
 
-template <typename T, bool VEL, bool AL>
+template <typename T, bool VEL, int A>
 static cudaError_t adj_row_occ(int *resident)
 {
-    using C = AdjRowCfg<T, kAdjRows, AL>;
-    auto kernel = adj_row_kernel<T, kAdjRows, VEL, AL>;
+    using C = AdjRowCfg<T, kAdjRows, A>;
+    auto kernel = adj_row_kernel<T, kAdjRows, VEL, A>;
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::bytes);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, kernel, C::NT, C::bytes);
 }
 
 template <typename T>
-cudaError_t adj_vec_resident(int *resident) { return adj_row_occ<T, false, true>(resident); }
+cudaError_t adj_vec_resident(int *resident) { return adj_row_occ<T, false, 16 / (int)sizeof(T)>(resident); }
 template cudaError_t adj_vec_resident<float>(int *);
 template cudaError_t adj_vec_resident<double>(int *);
 
 // Persistent grid of the row kernel: every resident block (*blocks, of the grid's), at most one
 // per unit.
-template <typename T, bool VEL, bool AL>
+template <typename T, bool VEL, int A>
 static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s, int *blocks)
 {
-    using C = AdjRowCfg<T, kAdjRows, AL>;
+    using C = AdjRowCfg<T, kAdjRows, A>;
     if (*blocks == 0) {  // first launch of this grid: kept, for the queries take longer than the launch
         int resident = 0, dev = 0, sms = 0;
         cudaError_t e;
-        if ((e = adj_row_occ<T, VEL, AL>(&resident)) != cudaSuccess) return e;
+        if ((e = adj_row_occ<T, VEL, A>(&resident)) != cudaSuccess) return e;
         if (resident < 1) return cudaErrorInvalidConfiguration;
         if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
             (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
@@ -399,7 +399,7 @@ static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s, int *bloc
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, adj_row_kernel<T, kAdjRows, VEL, AL>, a, nchunks);
+    return cudaLaunchKernelEx(&cfg, adj_row_kernel<T, kAdjRows, VEL, A>, a, nchunks);
 }
 
 template <typename T, int BX, int BY>
@@ -422,14 +422,21 @@ static cudaError_t launch_adj_t(const AdjArgs<T> &a, cudaStream_t s)
 template <typename T>
 cudaError_t launch_adj(const AdjArgs<T> &a, int tile, cudaStream_t s, int *row_blocks)
 {
+    constexpr int VX = 16 / (int)sizeof(T);
     switch (tile) {
     case 0: return launch_adj_t<T, 32, 8>(a, s);
     case 1: return launch_adj_t<T, 32, 16>(a, s);
     case 2: return launch_adj_t<T, 32, 4>(a, s);
-    case 3: return a.gu ? launch_adj_row<T, true, true>(a, s, row_blocks)
-                        : launch_adj_row<T, false, true>(a, s, row_blocks + 1);
-    case 4: return a.gu ? launch_adj_row<T, true, false>(a, s, row_blocks + 2)
-                        : launch_adj_row<T, false, false>(a, s, row_blocks + 3);
+    case 3: return a.gu ? launch_adj_row<T, true, VX>(a, s, row_blocks)
+                        : launch_adj_row<T, false, VX>(a, s, row_blocks + 1);
+    case 4:
+        if constexpr (sizeof(T) == 4) {  // rows on pairs
+            if (a.nx % 2 == 0)
+                return a.gu ? launch_adj_row<T, true, 2>(a, s, row_blocks + 2)
+                            : launch_adj_row<T, false, 2>(a, s, row_blocks + 3);
+        }
+        return a.gu ? launch_adj_row<T, true, 1>(a, s, row_blocks + 2)
+                    : launch_adj_row<T, false, 1>(a, s, row_blocks + 3);
     default: return cudaErrorInvalidValue;
     }
 }

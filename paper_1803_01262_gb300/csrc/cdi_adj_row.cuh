@@ -11,19 +11,19 @@
 // FP32, aligned rows: 148 -> 105 instructions per cell; 256^3 100.5 -> 83.5 us per step (4.0 -> 4.8
 // TB/s), with velocity gradients 156 -> 142 us (5.7 TB/s); FP64 128^3 348 -> 316 us (fewer FP64
 // operations).  Other rows, against one cell per thread: 255^3 FP32 172.5 -> 106 us, with
-// gradients 322 -> 192 us; FP64 129^3 609 -> 384 us.
+// gradients 322 -> 171 us; 254^3 (rows on pairs) 171 -> 100 and 315 -> 139; FP64 129^3 609 -> 384 us.
 #pragma once
 
 #include "cdi_row.cuh"
 
 namespace cdi {
 
-template <typename T, int TY, bool AL>
+template <typename T, int TY, int A>
 struct AdjRowCfg : RowGeo<T, TY> {
     using G = RowGeo<T, TY>;
     // velocity slots; other rows: two, which leaves L1 32 kB more (255^3 FP32 121 -> 106 us, with
     // gradients 209 -> 192)
-    static constexpr int NVS = AL ? 4 : 2;
+    static constexpr int NVS = A == G::VX ? 4 : 2;
     static constexpr int OLAM = G::NS * G::PHI, OVEL = 2 * G::NS * G::PHI;
     static constexpr int OGX = OVEL + NVS * G::VEL, OGY = OGX + 2 * G::SXS;
     static constexpr size_t bytes = sizeof(T) * (size_t)(OGY + 2 * G::SYS);
@@ -32,34 +32,48 @@ struct AdjRowCfg : RowGeo<T, TY> {
 
 // Add the group's n cells to memory by reductions at L2 (no other thread of the launch touches
 // them): the sums come back to no register, so no load's latency sits at the end of a plane.
-// With loads and stores instead, 256^3 FP32 with velocity gradients took 202 us, 142 us so.
-template <bool AL>
+// With loads and stores instead, 256^3 FP32 with velocity gradients took 202 us, 142 us so.  Rows
+// at any element: pairs where the address allows, for fewer reductions (255^3 192 -> 171 us; a
+// neighbour's first cell fetched by a shuffle, so that every lane issues two, 168 but it spills).
+template <int A>
 __device__ __forceinline__ void red_add(float *p, const float *v, int n)
 {
-    if constexpr (AL) {
+    if constexpr (A == 4) {
         asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
                      "f"(v[3])
                      : "memory");
+    } else if constexpr (A == 2) {
+#pragma unroll
+        for (int i = 0; i < 4; i += 2)
+            if (i < n)
+                asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p + i), "f"(v[i]), "f"(v[i + 1]) : "memory");
+    } else if (n == 4) {  // pairs where they lie on 8-byte boundaries
+        const int o = ((size_t)p >> 2) & 1;
+        if (o) atomicAdd(p, v[0]);
+        asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p + o), "f"(o ? v[1] : v[0]), "f"(o ? v[2] : v[1])
+                     : "memory");
+        if (o) atomicAdd(p + 3, v[3]);
+        else asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p + 2), "f"(v[2]), "f"(v[3]) : "memory");
     } else {
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 3; ++i)
             if (i < n) atomicAdd(p + i, v[i]);
     }
 }
-template <bool AL>
+template <int A>
 __device__ __forceinline__ void red_add(double *p, const double *v, int n)
 {
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-        if (AL || i < n) atomicAdd(p + i, v[i]);
+        if (A == 2 || i < n) atomicAdd(p + i, v[i]);
 }
 
 // VEL: the velocity gradients are accumulated (a.gu, a.gv, a.gw not null).
-template <typename T, int TY, bool VEL, bool AL>
-__global__ void __launch_bounds__(AdjRowCfg<T, TY, AL>::NT, 512 / AdjRowCfg<T, TY, AL>::NT)
+template <typename T, int TY, bool VEL, int A>
+__global__ void __launch_bounds__(AdjRowCfg<T, TY, A>::NT, 512 / AdjRowCfg<T, TY, A>::NT)
 adj_row_kernel(const AdjArgs<T> a, const int nchunks)
 {
-    using C = AdjRowCfg<T, TY, AL>;
+    using C = AdjRowCfg<T, TY, A>;
     using VV = V16<T>;
     constexpr int VX = C::VX, W = C::W, H = C::H, PP = C::PP, TX = C::TX, PHI = C::PHI;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -82,7 +96,8 @@ adj_row_kernel(const AdjArgs<T> a, const int nchunks)
     const bool has_xr = (lane & 15) < TY;                     // ring warp: an x-ring cell
     T *const bp = sm + (ty + 1) * PP + VX + tx * VX;
     T *const xb = sm + ((lane & 15) + 1) * PP + VX + (lane < 16 ? -1 : W);
-    RowStage<T, TY, AL> cp(sm, tid, ty, tx);
+    constexpr bool AL = A == VX;
+    RowStage<T, TY, A> cp(sm, tid, ty, tx);
 
     // gbar (b0, b1, b2) and the local term of the group's cells p, from the phi differences g
     // and the lam' differences dl
@@ -306,9 +321,7 @@ adj_row_kernel(const AdjArgs<T> a, const int nchunks)
                     if constexpr (AL) {
                         VV::st(a.out + ko, o);
                     } else {
-#pragma unroll
-                        for (int i = 0; i < VX; ++i)
-                            if (i < nown) a.out[ko + i] = o[i];
+                        store_cells<A, VX>(a.out + ko, o, nown);
                     }
                     if constexpr (VEL) {
                         T *const G3[3] = {a.gu + ko, a.gv + ko, a.gw + ko};
@@ -320,7 +333,7 @@ adj_row_kernel(const AdjArgs<T> a, const int nchunks)
                                 const T pr = q == 0 ? (i + 1 < VX ? cK[i + 1] : RK_) : q == 1 ? ypK[i] : cN[i];
                                 v[i] = (q == 0 ? dx[i] : q == 1 ? dy[i] : dz[i]) * c_vel * (cK[i] + pr);
                             }
-                            red_add<AL>(G3[q], v, nown);
+                            red_add<A>(G3[q], v, nown);
                         }
                     }
                 }

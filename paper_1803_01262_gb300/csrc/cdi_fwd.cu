@@ -482,15 +482,19 @@ static cudaError_t occ(K kernel, int threads, size_t smem, int *resident)
 // of it counts for more than the distance (301x257x211 FP32, 6-row tile: 91.0 us with four slots,
 // 84.2 with two; RK4 at 255^3, whose stage operands take shared memory too: 568 and 460 us).
 // Aligned rows, and the slabs of the host step (timed so only): four.
-template <bool ZR, bool AL>
-constexpr int row_vel_slots() { return !AL && !ZR ? 2 : 4; }
+template <typename T, bool ZR, int A>
+constexpr int row_vel_slots() { return A < 16 / (int)sizeof(T) && !ZR ? 2 : 4; }
 
 template <typename T, int TY, bool AL, bool RK = false, bool ZR = false>
 static cudaError_t row_occ(int *resident)
 {
-    constexpr int NV = row_vel_slots<ZR, AL>();
+    constexpr int A = AL ? 16 / (int)sizeof(T) : 1, NV = row_vel_slots<T, ZR, A>();
     using C = RowCfg<T, TY, RK, NV>;
-    return occ(fwd_row_kernel<T, TY, RK, ZR, AL, NV>, C::NT, C::bytes, resident);
+    if constexpr (!AL && sizeof(T) == 4) {  // row_launch takes this one where nx is even: as many blocks
+        cudaError_t e = occ(fwd_row_kernel<T, TY, RK, ZR, 2, NV>, C::NT, C::bytes, resident);
+        if (e != cudaSuccess) return e;
+    }
+    return occ(fwd_row_kernel<T, TY, RK, ZR, A, NV>, C::NT, C::bytes, resident);
 }
 
 // Runge-Kutta stage kernels exist for tiles 1, 3 (one cell per thread), 4 and 7 (vectors) only.
@@ -567,9 +571,13 @@ static cudaError_t launch_dependent(K kernel, int nblocks, int threads, size_t s
 template <typename T, int TY, bool AL, bool RK = false, bool ZR = false>
 static cudaError_t row_launch(const FwdArgs<T> &a, int nblocks, int nchunks, cudaStream_t s)
 {
-    constexpr int NV = row_vel_slots<ZR, AL>();
+    constexpr int A = AL ? 16 / (int)sizeof(T) : 1, NV = row_vel_slots<T, ZR, A>();
     using C = RowCfg<T, TY, RK, NV>;
-    return launch_dependent(fwd_row_kernel<T, TY, RK, ZR, AL, NV>, nblocks, C::NT, C::bytes, s, a, nchunks);
+    if constexpr (!AL && sizeof(T) == 4) {  // rows on pairs (the arrays' bases are 16-byte aligned)
+        if (a.nx % 2 == 0)
+            return launch_dependent(fwd_row_kernel<T, TY, RK, ZR, 2, NV>, nblocks, C::NT, C::bytes, s, a, nchunks);
+    }
+    return launch_dependent(fwd_row_kernel<T, TY, RK, ZR, A, NV>, nblocks, C::NT, C::bytes, s, a, nchunks);
 }
 
 template <typename T>

@@ -19,12 +19,14 @@
 // FP32, aligned rows: 102.5 -> 80.1 instructions per cell; 256^3 72.4 -> 57.4 us per step of a
 // run (4.63 -> 5.84 TB/s), 512^3 516 -> 420 us (5.20 -> 6.39 TB/s).
 //
-//   AL = true   rows start on 16-byte boundaries (nx % VX == 0): 16-byte cp.async and stores.
-//   AL = false  rows start at any element: a warp copies its rows element by element (a lane
+//   A = VX  (AL) rows start on 16-byte boundaries (nx % VX == 0): 16-byte cp.async and stores.
+//   A = 1, 2    rows start at any element, or on pairs (FP32, nx even): a warp copies its rows
+//               an element or a pair at a time (a lane
 //               per column: contiguous runs) and stores element by element (through shared
 //               memory, for contiguous stores: 89.1 against 86.4 us at 255^3 with the
 //               14-row tile).  255^3 FP32:
-//               139 us with one cell per thread (32x8 tile) -> 83.6 us; 385^3 501 -> 308 us.
+//               139 us with one cell per thread (32x8 tile) -> 83.6 us; 385^3 501 -> 308 us; 254^3 by
+//               pairs 135 -> 76.9 us, RK4 at 254^3 456 (by elements) -> 376 us.
 // The arithmetic is that of every other forward kernel, in the same order: the fields are the
 // same bit for bit.
 #pragma once
@@ -47,7 +49,7 @@ struct RowCfg : RowGeo<T, TY> {
     static_assert(G::VEL >= G::PHI, "the prologue's first phi plane borrows a velocity slot");
 };
 
-template <typename T, int TY, bool RK, bool ZR, bool AL, int NV>
+template <typename T, int TY, bool RK, bool ZR, int A, int NV>
 __global__ void __launch_bounds__(RowCfg<T, TY, RK, NV>::NT, 512 / RowCfg<T, TY, RK, NV>::NT)
 fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
 {
@@ -76,7 +78,8 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
     // bp[.. - PP], s_y row ty at bp[..]; xb: the same for the x-ring cell
     T *const bp = sm + (ty + 1) * PP + VX + tx * VX;
     T *const xb = sm + ((lane & 15) + 1) * PP + VX + (lane < 16 ? -1 : W);
-    RowStage<T, TY, AL> cp(sm, tid, ty, tx);
+    constexpr bool AL = A == VX;
+    RowStage<T, TY, A> cp(sm, tid, ty, tx);
 
     // Sharpening of the group's cells c, from its y neighbours, the planes below (zn) and
     // above (zp) and the x neighbours L, R.
@@ -315,9 +318,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
                             if constexpr (AL) {
                                 VV::st(qout, qo);
                             } else {
-#pragma unroll
-                                for (int i = 0; i < VX; ++i)
-                                    if (i < nown) qout[i] = qo[i];
+                                store_cells<A, VX>(qout, qo, nown);
                             }
                         }
                     }
@@ -329,9 +330,7 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
                     }
                 } else {
                     if (stats && nown > 0) acc.template add_group_n<VX>(o, nown, a.c.tol);
-#pragma unroll
-                    for (int i = 0; i < VX; ++i)
-                        if (i < nown) op[go + i] = o[i];
+                    store_cells<A, VX>(op + go, o, nown);
                 }
             }
 #pragma unroll

@@ -33,16 +33,18 @@ struct RowGeo {
 };
 
 // Copies of one work unit: in-plane offsets planned once, then a plane's copies are a base
-// pointer and immediates.  Own threads, AL: g[0] the own vector; else g[r NJ + j] column
-// lane + 32 j of row r0 + r.  Ring warp, AL: g[0..2] / d[0..2] vectors of a halo-2 plane (rows -1
+// pointer and immediates.  Own threads, AL: g[0] the own vector; else (A elements per copy:
+// 1, or 2 where rows start on pairs) g[r NJ + j] column A (lane + 32 j) of row r0 + r.  Ring warp, AL: g[0..2] / d[0..2] vectors of a halo-2 plane (rows -1
 // and H with their x halos, rows -2 and H+1, the x halos of rows 0..H-1), g[3] / d[3] the x halo
 // of u (lanes < H) and v row -1 (16 lanes).  Else g[r NJ + j] the rows -2, -1, H, H+1, gv[j] v
 // row -1, gh[0..1] / d[0..1] single cells (columns -1 and W of rows -1 and H; columns -2, -1, W,
-// W+1 of rows 0..H-1), gh[2] / d[2] u column -1.
-template <typename T, int TY, bool AL>
+// W+1 of rows 0..H-1; A = 2: pairs left and right of rows -1 .. H), gh[2] / d[2] u column -1.
+template <typename T, int TY, int A>
 struct RowStage {
     using G = RowGeo<T, TY>;
-    static constexpr int VX = G::VX, W = G::W, H = G::H, PP = G::PP, NJ = G::NJ, ES = sizeof(T);
+    static constexpr bool AL = A == G::VX, PR = !AL && A == 2;
+    static constexpr int EB = A * sizeof(T);  // bytes of a copy by elements
+    static constexpr int VX = G::VX, W = G::W, H = G::H, PP = G::PP, NJ = G::W / 32 / (AL ? 1 : A), ES = sizeof(T);
     static constexpr int NG = AL ? 4 : 4 * NJ;
     int g[NG], gh[3], gv[NJ];
     unsigned d[4];     // shared byte addresses of the ring warp's single places
@@ -58,7 +60,7 @@ struct RowStage {
     {
         is_own = tid < G::NOWN;
         lane = tid & 31;
-        cb = smem_addr(AL ? sm + (ty + 1) * PP + VX + tx * VX : sm + (is_own ? (ty & ~1) * PP : 0) + VX + lane);
+        cb = smem_addr(AL ? sm + (ty + 1) * PP + VX + tx * VX : sm + (is_own ? (ty & ~1) * PP : 0) + VX + lane * A);
     }
 
     __device__ __forceinline__ void plan(T *sm, int x0, int y0, int ty, int tx, int nx, int ny, long long plane,
@@ -80,7 +82,7 @@ struct RowStage {
 #pragma unroll
                 for (int r = 0; r < 2; ++r)
 #pragma unroll
-                    for (int j = 0; j < NJ; ++j) g[r * NJ + j] = at(y0 + r0 + r, x0 + lane + 32 * j, 1);
+                    for (int j = 0; j < NJ; ++j) g[r * NJ + j] = at(y0 + r0 + r, x0 + (lane + 32 * j) * A, A);
             }
         } else if constexpr (AL) {
 #pragma unroll
@@ -110,9 +112,14 @@ struct RowStage {
             for (int r = 0; r < 4; ++r)
 #pragma unroll
                 for (int j = 0; j < NJ; ++j)
-                    g[r * NJ + j] = at(y0 + (r < 2 ? r - 2 : H + r - 2), x0 + lane + 32 * j, 1);
+                    g[r * NJ + j] = at(y0 + (r < 2 ? r - 2 : H + r - 2), x0 + (lane + 32 * j) * A, A);
 #pragma unroll
-            for (int j = 0; j < NJ; ++j) gv[j] = at(y0 - 1, x0 + lane + 32 * j, 1);
+            for (int j = 0; j < NJ; ++j) gv[j] = at(y0 - 1, x0 + (lane + 32 * j) * A, A);
+            if constexpr (PR) {  // pairs left and right of rows -1 .. H
+                const int row = lane < 2 * H + 4 ? lane / 2 - 1 : 0, col = lane & 1 ? W : -2;
+                gh[0] = at(y0 + row, x0 + col, 2);
+                d[0] = smem_addr(sm + (row + 2) * PP + VX + col);
+            } else {
 #pragma unroll
             for (int i = 0; i < 2; ++i) {  // 4 H + 4 <= 64 cells
                 const int e = lane + 32 * i - 4;
@@ -120,6 +127,7 @@ struct RowStage {
                 const int col = e < 0 ? (e & 1 ? W : -1) : q < 2 ? q - 2 : W + q - 2;
                 gh[i] = at(y0 + row, x0 + col, 1);
                 d[i] = smem_addr(sm + (e < 4 * H ? (row + 2) * PP + VX + col : 0));
+            }
             }
             gh[2] = at(y0 + (lane < H ? lane : 0), x0 - 1, 1);
             d[2] = smem_addr(sm + (lane < H ? lane : 0) * PP + VX - 1);
@@ -148,11 +156,11 @@ struct RowStage {
             if constexpr (AL) {
                 cp_async_at<16, so + PP * ES>(cb, src + g[0]);
             } else {
-                cp_async_at<ES, so + 2 * PP * ES>(cb, src + g[0]);
-                cp_async_at<ES, so + 3 * PP * ES>(cb, src + g[NJ]);
+                cp_async_at<EB, so + 2 * PP * ES>(cb, src + g[0]);
+                cp_async_at<EB, so + 3 * PP * ES>(cb, src + g[NJ]);
                 if constexpr (NJ == 2) {
-                    cp_async_at<ES, so + (2 * PP + 32) * ES>(cb, src + g[1]);
-                    cp_async_at<ES, so + (3 * PP + 32) * ES>(cb, src + g[NJ + 1]);
+                    cp_async_at<EB, so + (2 * PP + 32) * ES>(cb, src + g[1]);
+                    cp_async_at<EB, so + (3 * PP + 32) * ES>(cb, src + g[NJ + 1]);
                 }
             }
         } else if constexpr (AL) {
@@ -160,18 +168,20 @@ struct RowStage {
             cp_async_at<16, so>(d[1], src + g[1]);
             if (TY == 14 || hx2) cp_async_at<16, so>(d[2], src + g[2]);
         } else {
-            cp_async_at<ES, so>(cb, src + g[0]);
-            cp_async_at<ES, so + PP * ES>(cb, src + g[NJ]);
-            cp_async_at<ES, so + (H + 2) * PP * ES>(cb, src + g[2 * NJ]);
-            cp_async_at<ES, so + (H + 3) * PP * ES>(cb, src + g[3 * NJ]);
+            cp_async_at<EB, so>(cb, src + g[0]);
+            cp_async_at<EB, so + PP * ES>(cb, src + g[NJ]);
+            cp_async_at<EB, so + (H + 2) * PP * ES>(cb, src + g[2 * NJ]);
+            cp_async_at<EB, so + (H + 3) * PP * ES>(cb, src + g[3 * NJ]);
             if constexpr (NJ == 2) {
-                cp_async_at<ES, so + 32 * ES>(cb, src + g[1]);
-                cp_async_at<ES, so + (PP + 32) * ES>(cb, src + g[NJ + 1]);
-                cp_async_at<ES, so + ((H + 2) * PP + 32) * ES>(cb, src + g[2 * NJ + 1]);
-                cp_async_at<ES, so + ((H + 3) * PP + 32) * ES>(cb, src + g[3 * NJ + 1]);
+                cp_async_at<EB, so + 32 * ES>(cb, src + g[1]);
+                cp_async_at<EB, so + (PP + 32) * ES>(cb, src + g[NJ + 1]);
+                cp_async_at<EB, so + ((H + 2) * PP + 32) * ES>(cb, src + g[2 * NJ + 1]);
+                cp_async_at<EB, so + ((H + 3) * PP + 32) * ES>(cb, src + g[3 * NJ + 1]);
             }
-            if (lane < 4 * H + 4) cp_async_at<ES, so>(d[0], src + gh[0]);
-            if (lane + 32 < 4 * H + 4) cp_async_at<ES, so>(d[1], src + gh[1]);
+            if (lane < (PR ? 2 * H + 4 : 4 * H + 4)) cp_async_at<EB, so>(d[0], src + gh[0]);
+            if constexpr (!PR) {
+                if (lane + 32 < 4 * H + 4) cp_async_at<EB, so>(d[1], src + gh[1]);
+            }
         }
     }
 
@@ -186,26 +196,26 @@ struct RowStage {
                 cp_async_at<16, so + G::VO * ES>(cb, pv + g[0]);
                 cp_async_at<16, so + (G::WO - PP) * ES>(cb, pw + g[0]);
             } else {
-                cp_async_at<ES, so>(cb, pu + g[0]);
-                cp_async_at<ES, so + PP * ES>(cb, pu + g[NJ]);
-                cp_async_at<ES, so + (G::VO + PP) * ES>(cb, pv + g[0]);
-                cp_async_at<ES, so + (G::VO + 2 * PP) * ES>(cb, pv + g[NJ]);
-                cp_async_at<ES, so + G::WO * ES>(cb, pw + g[0]);
-                cp_async_at<ES, so + (G::WO + PP) * ES>(cb, pw + g[NJ]);
+                cp_async_at<EB, so>(cb, pu + g[0]);
+                cp_async_at<EB, so + PP * ES>(cb, pu + g[NJ]);
+                cp_async_at<EB, so + (G::VO + PP) * ES>(cb, pv + g[0]);
+                cp_async_at<EB, so + (G::VO + 2 * PP) * ES>(cb, pv + g[NJ]);
+                cp_async_at<EB, so + G::WO * ES>(cb, pw + g[0]);
+                cp_async_at<EB, so + (G::WO + PP) * ES>(cb, pw + g[NJ]);
                 if constexpr (NJ == 2) {
-                    cp_async_at<ES, so + 32 * ES>(cb, pu + g[1]);
-                    cp_async_at<ES, so + (PP + 32) * ES>(cb, pu + g[NJ + 1]);
-                    cp_async_at<ES, so + (G::VO + PP + 32) * ES>(cb, pv + g[1]);
-                    cp_async_at<ES, so + (G::VO + 2 * PP + 32) * ES>(cb, pv + g[NJ + 1]);
-                    cp_async_at<ES, so + (G::WO + 32) * ES>(cb, pw + g[1]);
-                    cp_async_at<ES, so + (G::WO + PP + 32) * ES>(cb, pw + g[NJ + 1]);
+                    cp_async_at<EB, so + 32 * ES>(cb, pu + g[1]);
+                    cp_async_at<EB, so + (PP + 32) * ES>(cb, pu + g[NJ + 1]);
+                    cp_async_at<EB, so + (G::VO + PP + 32) * ES>(cb, pv + g[1]);
+                    cp_async_at<EB, so + (G::VO + 2 * PP + 32) * ES>(cb, pv + g[NJ + 1]);
+                    cp_async_at<EB, so + (G::WO + 32) * ES>(cb, pw + g[1]);
+                    cp_async_at<EB, so + (G::WO + PP + 32) * ES>(cb, pw + g[NJ + 1]);
                 }
             }
         } else if constexpr (AL) {
             if (lane < H + 16) cp_async_at<16, so>(d[3], (lane < H ? pu : pv) + g[3]);
         } else {
-            cp_async_at<ES, so + G::VO * ES>(cb, pv + gv[0]);
-            if constexpr (NJ == 2) cp_async_at<ES, so + (G::VO + 32) * ES>(cb, pv + gv[1]);
+            cp_async_at<EB, so + G::VO * ES>(cb, pv + gv[0]);
+            if constexpr (NJ == 2) cp_async_at<EB, so + (G::VO + 32) * ES>(cb, pv + gv[1]);
             if (lane < H) cp_async_at<ES, so>(d[2], pu + gh[2]);
         }
     }
@@ -214,7 +224,7 @@ struct RowStage {
     // place at base + SO elements (base: own_base), read back by the same warp.
     __device__ __forceinline__ unsigned own_base(T *sm, int ty, int tx) const
     {
-        return smem_addr(sm + (AL ? ty * W + tx * VX : (ty & ~1) * W + lane));
+        return smem_addr(sm + (AL ? ty * W + tx * VX : (ty & ~1) * W + lane * A));
     }
     template <int SO>
     __device__ __forceinline__ void own(unsigned base, const T *src) const
@@ -223,14 +233,26 @@ struct RowStage {
         if constexpr (AL) {
             cp_async_at<16, so>(base, src + g[0]);
         } else {
-            cp_async_at<ES, so>(base, src + g[0]);
-            cp_async_at<ES, so + W * ES>(base, src + g[NJ]);
+            cp_async_at<EB, so>(base, src + g[0]);
+            cp_async_at<EB, so + W * ES>(base, src + g[NJ]);
             if constexpr (NJ == 2) {
-                cp_async_at<ES, so + 32 * ES>(base, src + g[1]);
-                cp_async_at<ES, so + (W + 32) * ES>(base, src + g[NJ + 1]);
+                cp_async_at<EB, so + 32 * ES>(base, src + g[1]);
+                cp_async_at<EB, so + (W + 32) * ES>(base, src + g[NJ + 1]);
             }
         }
     }
 };
+
+// The first n of N cells, A at a time (A = 2: to an address on a pair).
+template <int A, int N, typename T>
+__device__ __forceinline__ void store_cells(T *p, const T *o, int n)
+{
+#pragma unroll
+    for (int i = 0; i < N; i += A) {
+        if (i >= n) continue;
+        if constexpr (A == 2 && sizeof(T) == 4) *reinterpret_cast<float2 *>(p + i) = make_float2(o[i], o[i + 1]);
+        else p[i] = o[i];
+    }
+}
 
 }  // namespace cdi
