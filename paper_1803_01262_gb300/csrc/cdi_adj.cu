@@ -363,15 +363,19 @@ template <typename T, bool VEL, int A>
 static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s, int *blocks)
 {
     using C = AdjRowCfg<T, kAdjRows, A>;
-    if (*blocks == 0) {  // first launch of this grid: kept, for the queries take longer than the launch
-        int resident = 0, dev = 0, sms = 0;
+    // Asked once per grid, for the queries take longer than the launch (threads that ask at the same
+    // time store the same number).
+    int resident = __atomic_load_n(blocks, __ATOMIC_RELAXED);
+    if (resident == 0) {
+        int dev = 0, sms = 0;
         cudaError_t e;
         if ((e = adj_row_occ<T, VEL, A>(&resident)) != cudaSuccess) return e;
         if (resident < 1) return cudaErrorInvalidConfiguration;
         if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
             (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
             return e;
-        *blocks = resident * sms;
+        resident *= sms;
+        __atomic_store_n(blocks, resident, __ATOMIC_RELAXED);
     }
     // zchunk < 0: balanced shares of the tile-planes (UnitIter; -2 rotated); else z chunks
     const long long tiles = (long long)((a.nx + C::W - 1) / C::W) * ((a.ny + C::H - 1) / C::H);
@@ -385,7 +389,7 @@ static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s, int *bloc
         const int zc = (a.nz + nchunks - 1) / nchunks;
         units = tiles * ((a.nz + zc - 1) / zc);
     }
-    long long nb = *blocks;
+    long long nb = resident;
     if (nb > units) nb = units;
     // programmatic stream serialisation: the launch may overlap the previous grid's
     // end (the kernel waits for it before touching anything it may write)
