@@ -360,7 +360,7 @@ template cudaError_t adj_vec_resident<double>(int *);
 // Persistent grid of the row kernel: every resident block (*blocks, of the grid's), at most one
 // per unit.
 template <typename T, bool VEL, int A>
-static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s, int *blocks)
+static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s, int *blocks, bool chained)
 {
     using C = AdjRowCfg<T, kAdjRows, A>;
     // Asked once per grid, for the queries take longer than the launch (threads that ask at the same
@@ -391,8 +391,8 @@ static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s, int *bloc
     }
     long long nb = resident;
     if (nb > units) nb = units;
-    // programmatic stream serialisation: the launch may overlap the previous grid's
-    // end (the kernel waits for it before touching anything it may write)
+    // programmatic stream serialisation: the launch may overlap the previous grid's end (the kernel
+    // waits for it before touching anything it may write; chained, as for launch_fwd)
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)nb);
     cfg.blockDim = dim3(C::NT);
@@ -403,7 +403,7 @@ static cudaError_t launch_adj_row(const AdjArgs<T> &a, cudaStream_t s, int *bloc
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, adj_row_kernel<T, kAdjRows, VEL, A>, a, nchunks);
+    return cudaLaunchKernelEx(&cfg, adj_row_kernel<T, kAdjRows, VEL, A>, a, nchunks, (int)chained);
 }
 
 template <typename T, int BX, int BY>
@@ -424,28 +424,28 @@ static cudaError_t launch_adj_t(const AdjArgs<T> &a, cudaStream_t s)
 }
 
 template <typename T>
-cudaError_t launch_adj(const AdjArgs<T> &a, int tile, cudaStream_t s, int *row_blocks)
+cudaError_t launch_adj(const AdjArgs<T> &a, int tile, cudaStream_t s, int *row_blocks, bool chained)
 {
     constexpr int VX = 16 / (int)sizeof(T);
     switch (tile) {
     case 0: return launch_adj_t<T, 32, 8>(a, s);
     case 1: return launch_adj_t<T, 32, 16>(a, s);
     case 2: return launch_adj_t<T, 32, 4>(a, s);
-    case 3: return a.gu ? launch_adj_row<T, true, VX>(a, s, row_blocks)
-                        : launch_adj_row<T, false, VX>(a, s, row_blocks + 1);
+    case 3: return a.gu ? launch_adj_row<T, true, VX>(a, s, row_blocks, chained)
+                        : launch_adj_row<T, false, VX>(a, s, row_blocks + 1, chained);
     case 4:
         if constexpr (sizeof(T) == 4) {  // rows on pairs
             if (a.nx % 2 == 0)
-                return a.gu ? launch_adj_row<T, true, 2>(a, s, row_blocks + 2)
-                            : launch_adj_row<T, false, 2>(a, s, row_blocks + 3);
+                return a.gu ? launch_adj_row<T, true, 2>(a, s, row_blocks + 2, chained)
+                            : launch_adj_row<T, false, 2>(a, s, row_blocks + 3, chained);
         }
-        return a.gu ? launch_adj_row<T, true, 1>(a, s, row_blocks + 2)
-                    : launch_adj_row<T, false, 1>(a, s, row_blocks + 3);
+        return a.gu ? launch_adj_row<T, true, 1>(a, s, row_blocks + 2, chained)
+                    : launch_adj_row<T, false, 1>(a, s, row_blocks + 3, chained);
     default: return cudaErrorInvalidValue;
     }
 }
 
-template cudaError_t launch_adj<float>(const AdjArgs<float> &, int, cudaStream_t, int *);
-template cudaError_t launch_adj<double>(const AdjArgs<double> &, int, cudaStream_t, int *);
+template cudaError_t launch_adj<float>(const AdjArgs<float> &, int, cudaStream_t, int *, bool);
+template cudaError_t launch_adj<double>(const AdjArgs<double> &, int, cudaStream_t, int *, bool);
 
 }  // namespace cdi

@@ -71,7 +71,7 @@ __device__ __forceinline__ void red_add(double *p, const double *v, int n)
 // VEL: the velocity gradients are accumulated (a.gu, a.gv, a.gw not null).
 template <typename T, int TY, bool VEL, int A>
 __global__ void __launch_bounds__(AdjRowCfg<T, TY, A>::NT, 512 / AdjRowCfg<T, TY, A>::NT)
-adj_row_kernel(const AdjArgs<T> a, const int nchunks)
+adj_row_kernel(const AdjArgs<T> a, const int nchunks, const int chained)
 {
     using C = AdjRowCfg<T, TY, A>;
     using VV = V16<T>;
@@ -127,7 +127,8 @@ adj_row_kernel(const AdjArgs<T> a, const int nchunks)
         return b0;
     };
 
-    bool dep_waited = false;  // the previous grid on the stream has completed
+    bool dep_waited = !chained;  // the previous grid on the stream has completed
+    if (!chained) grid_dep_wait();
     UnitIter<W, H> units(ntiles, nz, nchunks);
     Unit un;
     while (units.next(un, ntiles, tiles_x, nz, nchunks)) {
@@ -138,7 +139,8 @@ adj_row_kernel(const AdjArgs<T> a, const int nchunks)
         };
 
         // Slot of plane z in every ring: (z - z0) mod 4.  The velocities (and w below plane z0)
-        // before waiting for the previous grid on the stream; phi, lam' and the accumulated
+        // before waiting for the previous grid on the stream if that is one of the same call
+        // (chained); phi, lam' and the accumulated
         // velocity gradients, which it may write, only after.
         __syncthreads();  // the previous unit's readers are done with every slot
         long long zo = (long long)CDI_CHK(z0, nz, st) * plane;  // element offset of plane k

@@ -571,11 +571,12 @@ struct DeferCfg {
 };
 
 // One forward step, or (z_hi > 0) its planes [z_lo, z_hi) folded into the record:
-// combine adds to the record's per-step fields, update_run closes the step.
+// combine adds to the record's per-step fields, update_run closes the step.  chained: the launch
+// before it on the stream belongs to the same call (launch_fwd).
 template <typename T>
 static int step_t(cdi_grid *g, const void *in, void *out, double dt, double eps, double gamma,
                   double vs, cudaStream_t s, int z_lo = 0, int z_hi = 0, int combine = 0,
-                  int update_run = 1, const DeferCfg *dfr = nullptr)
+                  int update_run = 1, const DeferCfg *dfr = nullptr, bool chained = false)
 {
     cdi::FwdArgs<T> a;
     a.phi = (const T *)in;
@@ -608,7 +609,7 @@ static int step_t(cdi_grid *g, const void *in, void *out, double dt, double eps,
         }
     }
     cudaError_t e = cdi::launch_fwd<T>(a, c.tile, c.nblocks, c.nchunks, false, s,
-                                       g->sharpen == CDI_SHARPEN_FACE);
+                                       g->sharpen == CDI_SHARPEN_FACE, chained);
     if (e != cudaSuccess) return cuda_fail(e, "forward step launch");
     return CDI_OK;
 }
@@ -763,7 +764,8 @@ struct RkStage {
     const void *in, *base, *q;
     void *out, *qout;
     double alpha, delta, mu, beta, vs;
-    int last;  // fold the result into the run statistics
+    int last;      // fold the result into the run statistics
+    bool chained;  // the launch before it belongs to the same call (launch_fwd)
 };
 
 template <typename T>
@@ -789,7 +791,7 @@ static int rk_stage_t(cdi_grid *g, const RkStage &st, double dt, double eps, dou
     a.rk_delta = (T)st.delta;
     a.rk_mu = (T)st.mu;
     a.rk_beta = (T)st.beta;
-    cudaError_t e = cdi::launch_fwd<T>(a, g->rk.tile, g->rk.nblocks, g->rk.nchunks, true, s);
+    cudaError_t e = cdi::launch_fwd<T>(a, g->rk.tile, g->rk.nblocks, g->rk.nchunks, true, s, false, st.chained);
     if (e != cudaSuccess) return cuda_fail(e, "Runge-Kutta stage launch");
     return CDI_OK;
 }
@@ -802,13 +804,16 @@ static int rk_stage(cdi_grid *g, const RkStage &st, double dt, double eps, doubl
 
 static double vscale(double t, double period) { return period > 0 ? cos(M_PI * t / period) : 1.0; }
 
-// One step of the scheme from phi_in (kept) to phi_out, with work arrays w1, w2.
+// One step of the scheme from phi_in (kept) to phi_out, with work arrays w1, w2 (chained: not the
+// first of its call).
 static int rk_step_impl(cdi_grid *g, const void *pin, void *pout, void *w1, void *w2, double dt,
-                        double eps, double gamma, double t, double period, int scheme, cudaStream_t s)
+                        double eps, double gamma, double t, double period, int scheme, cudaStream_t s,
+                        bool chained)
 {
     auto S = [&](const void *in, void *out, const void *base, const void *q, void *qout, double al,
                  double de, double mu, double be, double tt, int last) {
-        RkStage st{in, base, q, out, qout, al, de, mu, be, vscale(tt, period), last};
+        RkStage st{in, base, q, out, qout, al, de, mu, be, vscale(tt, period), last, chained};
+        chained = true;
         return rk_stage(g, st, dt, eps, gamma, s);
     };
     int rc = CDI_OK;
@@ -868,7 +873,7 @@ int cdi_step_rk(cdi_grid *g, const void *phi_in, void *phi_out, void *work1, voi
     if (g && g->sharpen == CDI_SHARPEN_FACE) return fail(CDI_ERR_ARG, "Runge-Kutta stages use the centre-product sharpening");
     if (int rc = check_rk_args(g, phi_in, phi_out, work1, work2, dt, eps, gamma, scheme, flags)) return rc;
     return rk_step_impl(g, phi_in, phi_out, work1, work2, dt, eps, gamma, t, period, scheme,
-                        (cudaStream_t)stream);
+                        (cudaStream_t)stream, false);
 }
 
 int cdi_run_rk(cdi_grid *g, void *buf_a, void *buf_b, void *work1, void *work2, int nsteps, double t0,
@@ -882,7 +887,7 @@ int cdi_run_rk(cdi_grid *g, void *buf_a, void *buf_b, void *work1, void *work2, 
     void *src = buf_a, *dst = buf_b;
     for (int i = 0; i < nsteps; ++i) {
         if (int rc = rk_step_impl(g, src, dst, work1, work2, dt, eps, gamma, t0 + i * dt, period, scheme,
-                                  (cudaStream_t)stream))
+                                  (cudaStream_t)stream, i > 0))
             return rc;
         void *tmp = src;
         src = dst;
@@ -940,8 +945,8 @@ int cdi_run(cdi_grid *g, void *buf_a, void *buf_b, int nsteps, double t0, double
         } else {
             const DeferCfg d = {i & 1, i + 1 < nsteps, i > 0};
             const DeferCfg *dp = defer ? &d : nullptr;
-            rc = g->dtype == CDI_F64 ? step_t<double>(g, src, dst, dt, eps, gamma, vs, s, 0, 0, 0, 1, dp)
-                                     : step_t<float>(g, src, dst, dt, eps, gamma, vs, s, 0, 0, 0, 1, dp);
+            rc = g->dtype == CDI_F64 ? step_t<double>(g, src, dst, dt, eps, gamma, vs, s, 0, 0, 0, 1, dp, i > 0)
+                                     : step_t<float>(g, src, dst, dt, eps, gamma, vs, s, 0, 0, 0, 1, dp, i > 0);
             i += 1;
         }
         if (rc) return rc;
@@ -1129,8 +1134,8 @@ static int step_host_pipelined(cdi_grid *g, const void *hin, void *hout, double 
     for (int j = 0; j < S; ++j) {
         if ((e = cudaStreamWaitEvent(s, g->ev_in[j], 0)) != cudaSuccess) return cuda_fail(e, "wait");
         int rc = g->dtype == CDI_F64
-                     ? step_t<double>(g, si, so, dt, eps, gamma, vs, s, b[j], b[j + 1], j > 0, j == S - 1)
-                     : step_t<float>(g, si, so, dt, eps, gamma, vs, s, b[j], b[j + 1], j > 0, j == S - 1);
+                     ? step_t<double>(g, si, so, dt, eps, gamma, vs, s, b[j], b[j + 1], j > 0, j == S - 1, nullptr, j > 0)
+                     : step_t<float>(g, si, so, dt, eps, gamma, vs, s, b[j], b[j + 1], j > 0, j == S - 1, nullptr, j > 0);
         if (rc) return rc;
         const size_t off = (size_t)b[j] * pb, len = (size_t)(b[j + 1] - b[j]) * pb;
         if ((e = cudaEventRecord(g->ev_c[j], s)) != cudaSuccess ||
@@ -1181,7 +1186,7 @@ int cdi_step_host(cdi_grid *g, const void *phi_in_host, void *phi_out_host, doub
 
 template <typename T>
 static int adjoint_t(cdi_grid *g, const void *phi, const void *lam, void *out, void *gu, void *gv,
-                     void *gw, double dt, double eps, double gamma, double vs, cudaStream_t s)
+                     void *gw, double dt, double eps, double gamma, double vs, cudaStream_t s, bool chained)
 {
     cdi::AdjArgs<T> a;
     a.phi = (const T *)phi;
@@ -1201,14 +1206,14 @@ static int adjoint_t(cdi_grid *g, const void *phi, const void *lam, void *out, v
     a.status = g->status;
     if (cdi::adj_blocks(g->adj.tile, a.zchunk, g->nx, g->ny, g->nz) > g->capacity)
         return fail(CDI_ERR_STATE, "adjoint launch configuration out of range");
-    cudaError_t e = cdi::launch_adj<T>(a, g->adj.tile, s, g->adj_blocks);
+    cudaError_t e = cdi::launch_adj<T>(a, g->adj.tile, s, g->adj_blocks, chained);
     if (e != cudaSuccess) return cuda_fail(e, "adjoint step launch");
     return CDI_OK;
 }
 
-int cdi_step_adjoint(cdi_grid *g, const void *phi_k, const void *lam_next, void *lam_k, void *gu,
-                     void *gv, void *gw, double dt, double eps, double gamma, double vel_scale,
-                     void *stream)
+// chained: not the first adjoint step of its call
+static int adjoint_step(cdi_grid *g, const void *phi_k, const void *lam_next, void *lam_k, void *gu, void *gv,
+                        void *gw, double dt, double eps, double gamma, double vel_scale, void *stream, bool chained)
 {
     cdi::NvtxRange nvtx_("cdi_step_adjoint");
     if (int rc = check_step_args(g, phi_k, lam_k, dt, eps, gamma, vel_scale)) return rc;
@@ -1224,8 +1229,15 @@ int cdi_step_adjoint(cdi_grid *g, const void *phi_k, const void *lam_next, void 
         return fail(CDI_ERR_ARG, "velocity gradients must be 16-byte aligned");
     cudaStream_t s = (cudaStream_t)stream;
     return g->dtype == CDI_F64
-        ? adjoint_t<double>(g, phi_k, lam_next, lam_k, gu, gv, gw, dt, eps, gamma, vel_scale, s)
-        : adjoint_t<float>(g, phi_k, lam_next, lam_k, gu, gv, gw, dt, eps, gamma, vel_scale, s);
+        ? adjoint_t<double>(g, phi_k, lam_next, lam_k, gu, gv, gw, dt, eps, gamma, vel_scale, s, chained)
+        : adjoint_t<float>(g, phi_k, lam_next, lam_k, gu, gv, gw, dt, eps, gamma, vel_scale, s, chained);
+}
+
+int cdi_step_adjoint(cdi_grid *g, const void *phi_k, const void *lam_next, void *lam_k, void *gu,
+                     void *gv, void *gw, double dt, double eps, double gamma, double vel_scale,
+                     void *stream)
+{
+    return adjoint_step(g, phi_k, lam_next, lam_k, gu, gv, gw, dt, eps, gamma, vel_scale, stream, false);
 }
 
 int cdi_step_path(cdi_grid *g, void *const *phi, int nsteps, double dt, double eps, double gamma,
@@ -1240,8 +1252,8 @@ int cdi_step_path(cdi_grid *g, void *const *phi, int nsteps, double dt, double e
         const DeferCfg d = {i & 1, i + 1 < nsteps, i > 0};
         const DeferCfg *dp = defer ? &d : nullptr;
         const int rc = g->dtype == CDI_F64
-            ? step_t<double>(g, phi[i], phi[i + 1], dt, eps, gamma, vel_scale[i], s, 0, 0, 0, 1, dp)
-            : step_t<float>(g, phi[i], phi[i + 1], dt, eps, gamma, vel_scale[i], s, 0, 0, 0, 1, dp);
+            ? step_t<double>(g, phi[i], phi[i + 1], dt, eps, gamma, vel_scale[i], s, 0, 0, 0, 1, dp, i > 0)
+            : step_t<float>(g, phi[i], phi[i + 1], dt, eps, gamma, vel_scale[i], s, 0, 0, 0, 1, dp, i > 0);
         if (rc) return rc;
     }
     return CDI_OK;
@@ -1254,7 +1266,8 @@ int cdi_adjoint_path(cdi_grid *g, void *const *phi, int nsteps, void *lam_a, voi
     if (nsteps < 0 || (nsteps > 0 && (!phi || !vel_scale))) return fail(CDI_ERR_ARG, "bad adjoint path");
     void *src = lam_a, *dst = lam_b;
     for (int i = nsteps - 1; i >= 0; --i) {
-        if (int rc = cdi_step_adjoint(g, phi[i], src, dst, gu, gv, gw, dt, eps, gamma, vel_scale[i], stream))
+        if (int rc = adjoint_step(g, phi[i], src, dst, gu, gv, gw, dt, eps, gamma, vel_scale[i], stream,
+                                  i + 1 < nsteps))
             return rc;
         std::swap(src, dst);
     }
@@ -1524,8 +1537,9 @@ int cdi_autotune(cdi_grid *g, void *phi_a, void *phi_b, double dt, double eps, d
             for (int i = 0; i <= reps && rc == CDI_OK; ++i) {
                 if (i == 1 && (e = cudaEventRecord(e0, s)) != cudaSuccess) rc = cuda_fail(e, "event");
                 if (rc == CDI_OK)
-                    rc = g->dtype == CDI_F64 ? step_t<double>(g, src, dst, dt, eps, gamma, 1.0, s)
-                                             : step_t<float>(g, src, dst, dt, eps, gamma, 1.0, s);
+                    rc = g->dtype == CDI_F64
+                        ? step_t<double>(g, src, dst, dt, eps, gamma, 1.0, s, 0, 0, 0, 1, nullptr, i > 0)
+                        : step_t<float>(g, src, dst, dt, eps, gamma, 1.0, s, 0, 0, 0, 1, nullptr, i > 0);
                 void *t = src; src = dst; dst = t;
             }
             if (rc != CDI_OK) break;

@@ -69,7 +69,7 @@ struct VecCfg {
 // step); the full-box instantiations keep no range.
 template <typename T, int TX, int TY, bool RK, bool ZR = false>
 __global__ void __launch_bounds__(VecCfg<T, TX, TY>::NT, 2)
-fwd_vec_kernel(const FwdArgs<T> a, const int nchunks)
+fwd_vec_kernel(const FwdArgs<T> a, const int nchunks, const int chained)
 {
     using C = VecCfg<T, TX, TY>;
     using VV = V16<T>;
@@ -138,7 +138,8 @@ fwd_vec_kernel(const FwdArgs<T> a, const int nchunks)
 
     Acc<T> acc;
     acc.init();
-    bool dep_waited = false;  // the previous grid on the stream has completed
+    bool dep_waited = !chained;  // the previous grid on the stream has completed
+    if (!chained) grid_dep_wait();
 
     // planes [z_lo, z_hi) with ZR, else all of them
     const int zlo = ZR ? a.z_lo : 0, zr = ZR ? a.z_hi - a.z_lo : nz;
@@ -214,9 +215,9 @@ fwd_vec_kernel(const FwdArgs<T> a, const int nchunks)
         // phi slot of plane z: (z - z0 + 2) mod 5; velocity slot: (z - z0) mod 3.
         __syncthreads();  // the previous unit's readers are done with every slot
         // The face velocities are never written by a step: staged (and the w below
-        // plane z0 loaded) before waiting for the previous grid on the stream,
-        // whose outputs -- phi, the Runge-Kutta operands, the reduction scratch --
-        // are touched only after it.
+        // plane z0 loaded) before waiting for the previous grid on the stream if that is
+        // one of the same call (chained), whose outputs -- phi, the Runge-Kutta operands,
+        // the reduction scratch -- are touched only after it.
         issue_vel(z0, 0);
         const int own_x = x0 + tx * VX, own_y = y0 + ty;
         const bool writes = is_own && own_x < nx && own_y < ny;
@@ -549,11 +550,16 @@ cudaError_t fwd_occupancy(int tile, bool rk, int *resident, bool face, bool slab
 template cudaError_t fwd_occupancy<float>(int, bool, int *, bool, bool);
 template cudaError_t fwd_occupancy<double>(int, bool, int *, bool, bool);
 
-// Launch with programmatic stream serialisation: the kernel may start while
-// the previous grid on the stream finishes (it waits in grid_dep_wait before
-// touching anything that grid may write).
+// Launch with programmatic stream serialisation: the kernel may start while the previous grid on the
+// stream finishes (it waits in grid_dep_wait before touching anything that grid may write).
+// chained: that grid is a launch of the same call, which writes no face velocities, and the kernel
+// reads them before it waits.  A call's first launch follows whatever the caller queued, often the
+// kernel that wrote the velocities: it waits before it reads anything.  (An ordinary launch there
+// cost 3-4 us per call: RK4 at 192^3 157.2 -> 162.1 us, one adjoint step at 256^3 82.4 -> 85.3; so,
+// 158.5 and 82.7.)
 template <typename K, typename... Args>
-static cudaError_t launch_dependent(K kernel, int nblocks, int threads, size_t smem, cudaStream_t s, Args... args)
+static cudaError_t launch_dependent(K kernel, int nblocks, int threads, size_t smem, cudaStream_t s, bool chained,
+                                    Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nblocks);
@@ -565,34 +571,35 @@ static cudaError_t launch_dependent(K kernel, int nblocks, int threads, size_t s
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
+    return cudaLaunchKernelEx(&cfg, kernel, args..., (int)chained);
 }
 
 template <typename T, int TY, bool AL, bool RK = false, bool ZR = false>
-static cudaError_t row_launch(const FwdArgs<T> &a, int nblocks, int nchunks, cudaStream_t s)
+static cudaError_t row_launch(const FwdArgs<T> &a, int nblocks, int nchunks, cudaStream_t s, bool chained)
 {
     constexpr int A = AL ? 16 / (int)sizeof(T) : 1, NV = row_vel_slots<T, ZR, A>();
     using C = RowCfg<T, TY, RK, NV>;
     if constexpr (!AL && sizeof(T) == 4) {  // rows on pairs (the arrays' bases are 16-byte aligned)
         if (a.nx % 2 == 0)
-            return launch_dependent(fwd_row_kernel<T, TY, RK, ZR, 2, NV>, nblocks, C::NT, C::bytes, s, a, nchunks);
+            return launch_dependent(fwd_row_kernel<T, TY, RK, ZR, 2, NV>, nblocks, C::NT, C::bytes, s, chained, a,
+                                    nchunks);
     }
-    return launch_dependent(fwd_row_kernel<T, TY, RK, ZR, A, NV>, nblocks, C::NT, C::bytes, s, a, nchunks);
+    return launch_dependent(fwd_row_kernel<T, TY, RK, ZR, A, NV>, nblocks, C::NT, C::bytes, s, chained, a, nchunks);
 }
 
 template <typename T>
 cudaError_t launch_fwd(const FwdArgs<T> &a, int tile, int nblocks, int nchunks, bool rk, cudaStream_t s,
-                       bool face)
+                       bool face, bool chained)
 {
     if (a.z_hi > 0) {  // a z slab: tile 4 (aligned rows) or 7 (any), centre form, Euler
         if (rk || face) return cudaErrorInvalidValue;
         if (tile == 4) {
-            if constexpr (sizeof(T) == 4) return row_launch<T, 14, true, false, true>(a, nblocks, nchunks, s);
+            if constexpr (sizeof(T) == 4) return row_launch<T, 14, true, false, true>(a, nblocks, nchunks, s, chained);
             else
                 return launch_dependent(fwd_vec_kernel<T, 16, 16, false, true>, nblocks, VecCfg<T, 16, 16>::NT,
-                                        VecCfg<T, 16, 16>::bytes, s, a, nchunks);
+                                        VecCfg<T, 16, 16>::bytes, s, chained, a, nchunks);
         }
-        if (tile == 7) return row_launch<T, 14, false, false, true>(a, nblocks, nchunks, s);
+        if (tile == 7) return row_launch<T, 14, false, false, true>(a, nblocks, nchunks, s, chained);
         return cudaErrorInvalidValue;
     }
     if (face) {  // face-product sharpening: tile 0 only, Euler only
@@ -605,11 +612,11 @@ cudaError_t launch_fwd(const FwdArgs<T> &a, int tile, int nblocks, int nchunks, 
         case 1: fwd_kernel<T, 32, 16, true><<<nblocks, dim3(32, 16), FwdSmem<T, 32, 16>::bytes, s>>>(a, nchunks); break;
         case 3: fwd_kernel<T, 32, 4, true><<<nblocks, dim3(32, 4), FwdSmem<T, 32, 4>::bytes, s>>>(a, nchunks); break;
         case 4:
-            if constexpr (sizeof(T) == 4) return row_launch<T, 14, true, true>(a, nblocks, nchunks, s);
+            if constexpr (sizeof(T) == 4) return row_launch<T, 14, true, true>(a, nblocks, nchunks, s, chained);
             else
                 return launch_dependent(fwd_vec_kernel<T, 16, 16, true>, nblocks, VecCfg<T, 16, 16>::NT,
-                                        VecCfg<T, 16, 16>::bytes, s, a, nchunks);
-        case 7: return row_launch<T, 14, false, true>(a, nblocks, nchunks, s);
+                                        VecCfg<T, 16, 16>::bytes, s, chained, a, nchunks);
+        case 7: return row_launch<T, 14, false, true>(a, nblocks, nchunks, s, chained);
         default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
@@ -620,25 +627,25 @@ cudaError_t launch_fwd(const FwdArgs<T> &a, int tile, int nblocks, int nchunks, 
     case 2: fwd_kernel<T, 64, 8, false><<<nblocks, dim3(64, 8), FwdSmem<T, 64, 8>::bytes, s>>>(a, nchunks); break;
     case 3: fwd_kernel<T, 32, 4, false><<<nblocks, dim3(32, 4), FwdSmem<T, 32, 4>::bytes, s>>>(a, nchunks); break;
     case 4:
-        if constexpr (sizeof(T) == 4) return row_launch<T, 14, true>(a, nblocks, nchunks, s);
+        if constexpr (sizeof(T) == 4) return row_launch<T, 14, true>(a, nblocks, nchunks, s, chained);
         else
             return launch_dependent(fwd_vec_kernel<T, 16, 16, false>, nblocks, VecCfg<T, 16, 16>::NT,
-                                    VecCfg<T, 16, 16>::bytes, s, a, nchunks);
+                                    VecCfg<T, 16, 16>::bytes, s, chained, a, nchunks);
     case 5:
-        if constexpr (sizeof(T) == 4) return row_launch<T, 6, true>(a, nblocks, nchunks, s);
+        if constexpr (sizeof(T) == 4) return row_launch<T, 6, true>(a, nblocks, nchunks, s, chained);
         else
             return launch_dependent(fwd_vec_kernel<T, 16, 8, false>, nblocks, VecCfg<T, 16, 8>::NT,
-                                    VecCfg<T, 16, 8>::bytes, s, a, nchunks);
+                                    VecCfg<T, 16, 8>::bytes, s, chained, a, nchunks);
     case 6: return launch_fwd_tma<T>(a, nblocks, nchunks, s);
-    case 7: return row_launch<T, 14, false>(a, nblocks, nchunks, s);
-    case 8: return row_launch<T, 6, false>(a, nblocks, nchunks, s);
+    case 7: return row_launch<T, 14, false>(a, nblocks, nchunks, s, chained);
+    case 8: return row_launch<T, 6, false>(a, nblocks, nchunks, s, chained);
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
 
-template cudaError_t launch_fwd<float>(const FwdArgs<float> &, int, int, int, bool, cudaStream_t, bool);
-template cudaError_t launch_fwd<double>(const FwdArgs<double> &, int, int, int, bool, cudaStream_t, bool);
+template cudaError_t launch_fwd<float>(const FwdArgs<float> &, int, int, int, bool, cudaStream_t, bool, bool);
+template cudaError_t launch_fwd<double>(const FwdArgs<double> &, int, int, int, bool, cudaStream_t, bool, bool);
 
 // ---------------------------------------------------------------------------
 // Stand-alone reductions: statistics of any field, and max |component| of

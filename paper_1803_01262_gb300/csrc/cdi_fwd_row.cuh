@@ -51,7 +51,7 @@ struct RowCfg : RowGeo<T, TY> {
 
 template <typename T, int TY, bool RK, bool ZR, int A, int NV>
 __global__ void __launch_bounds__(RowCfg<T, TY, RK, NV>::NT, 512 / RowCfg<T, TY, RK, NV>::NT)
-fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
+fwd_row_kernel(const FwdArgs<T> a, const int nchunks, const int chained)
 {
     using C = RowCfg<T, TY, RK, NV>;
     using VV = V16<T>;
@@ -115,7 +115,8 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
     acc.init();
     // The record is the last Runge-Kutta stage's, which overwrites the others': they skip it.
     const bool stats = !RK || a.red.update_run;
-    bool dep_waited = false;  // the previous grid on the stream has completed
+    bool dep_waited = !chained;  // the previous grid on the stream has completed
+    if (!chained) grid_dep_wait();
 
     const int zlo = ZR ? a.z_lo : 0, zr = ZR ? a.z_hi - a.z_lo : nz;
     UnitIter<W, H> units(ntiles, zr, nchunks);
@@ -139,7 +140,8 @@ fwd_row_kernel(const FwdArgs<T> a, const int nchunks)
         // Slot of plane z, phi and velocities: (z - z0) mod 4.
         __syncthreads();  // the previous unit's readers are done with every slot
         // The face velocities are never written by a step: staged (and the w below
-        // plane z0 loaded) before waiting for the previous grid on the stream.
+        // plane z0 loaded) before waiting for the previous grid on the stream if that is one
+        // of the same call (chained).
         long long zo = (long long)CDI_CHK(z0, nz, st) * plane;  // element offset of plane k
         issue_vel(zo, IC<C::OVEL>{});
         const int own_x = x0 + tx * VX, own_y = y0 + ty;

@@ -147,12 +147,14 @@ cudaError_t launch_fwd_plane(const FwdArgs<T> &a, T *prev, int n, const T *c_adv
                              unsigned long long *words, unsigned *tag, cudaStream_t s);
 
 // rk selects the Runge-Kutta stage variant (tiles with fwd_tile_has_rk only);
-// face the face-product sharpening (tile 0, Euler only).
+// face the face-product sharpening (tile 0, Euler only); chained: the launch before it on the
+// stream belongs to the same call of the library, so it wrote no face velocities, which the
+// vector and row kernels then read before it has ended.
 bool fwd_tile_has_rk(int tile);
 
 template <typename T>
 cudaError_t launch_fwd(const FwdArgs<T> &a, int tile, int nblocks, int nchunks, bool rk, cudaStream_t s,
-                       bool face = false);
+                       bool face = false, bool chained = false);
 
 template <typename T>
 cudaError_t launch_stats(const T *phi, long long n, T tol, RedScratch red, int nblocks,
@@ -163,8 +165,9 @@ cudaError_t launch_absmax(const T *u, const T *v, const T *w, long long n, RedSc
                           int nblocks, cudaStream_t s);
 
 // row_blocks[4]: resident blocks of the row kernel's instantiations (0: not asked yet), kept by the grid.
+// chained: as for launch_fwd.
 template <typename T>
-cudaError_t launch_adj(const AdjArgs<T> &a, int tile, cudaStream_t s, int *row_blocks);
+cudaError_t launch_adj(const AdjArgs<T> &a, int tile, cudaStream_t s, int *row_blocks, bool chained = false);
 
 int adj_num_tiles();
 int adj_blocks(int tile, int zchunk, int nx, int ny, int nz);
