@@ -332,7 +332,8 @@ CDI_API int cdi_batch_reset_run_stats(cdi_batch *b, void *stream);
 
 /* Test of the run's bounded wait: one launch whose work units wait for a step
  * their boxes never reach, the first wait for limit_s seconds (0 < limit_s <=
- * 2), the others giving up when they see it has.  No unit is stepped: fields,
+ * 2), the others giving up when they see it has (with tile 4 also a run's launch,
+ * where it holds whole boxes on chip and hands them on between blocks).  No unit is stepped: fields,
  * statistics and parity are unchanged.  Returns CDI_ERR_TIMEOUT (the expected
  * result; the status words are cleared) or CDI_OK if no wait ran out (the
  * time-out path is broken).  Synchronises. */

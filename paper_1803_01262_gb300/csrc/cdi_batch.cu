@@ -286,9 +286,10 @@ batch_kernel(const BoxDev<T> *__restrict__ boxes, const int *__restrict__ unit_b
 // cdi_plane.cuh): one launch for the whole run.  A step per launch left a third of the FP64 pipe
 // idle (two boxes on 104 of 152 SMs, the loads, reductions and waits of every step): 256 boxes of
 // 50^2 FP64 58 -> 41.8 us per step, which is the FP64 pipe of every SM; FP32 11.2 -> 3.8 us.  A unit is m steps of one box (chunk-major: chunk
-// c of every box, then chunk c + 1), handed out from a counter; a unit after its box's first waits,
-// bounded, for the box's epoch, which the unit before it releases with the state stored.  The
-// unit before was handed out earlier, to a block that is running: no deadlock.
+// c of every box, then chunk c + 1), every one handed out from a counter; a unit after its box's
+// first waits, bounded, for the box's epoch, which the unit before it releases with the state
+// stored.  The unit before was handed out earlier, to a block that is running, also where some
+// blocks start late (SMs taken by another stream's kernel): no deadlock.
 // sync: [0] units handed out, [1] blocks finished, [2 + box] the box's epoch; the last block
 // zeroes them.
 template <typename T, int NT, bool FACE>
@@ -301,7 +302,9 @@ plane_batch_kernel(const BoxDev<T> *__restrict__ boxes, const int *__restrict__ 
     __shared__ int next_u, ready;
     const int tid = threadIdx.x;
     unsigned int *const status = boxes[0].a.red.status;
-    for (int u = blockIdx.x; u < nbox * nchunks; u = next_u) {
+    if (tid == 0) next_u = (int)atomicAdd(sync, 1u);
+    __syncthreads();
+    for (int u = next_u; u < nbox * nchunks; u = next_u) {
         const int c = u / nbox, bi = order[u - c * nbox];
         if (c > 0) {  // the box's earlier steps: complete and visible
             if (tid == 0) {
@@ -328,7 +331,7 @@ plane_batch_kernel(const BoxDev<T> *__restrict__ boxes, const int *__restrict__ 
         plane_steps<T, NT, FACE, false>(a, keep_prev && fin && n > 1 ? buf[fp ^ 1] : nullptr, 0, a.ny, steps,
                                         [&](int) { return c_adv; }, h, run, last, reinterpret_cast<T *>(smem_raw));
         int claim = 0;
-        if (tid == 0) claim = (int)atomicAdd(sync, 1u) + (int)gridDim.x;
+        if (tid == 0) claim = (int)atomicAdd(sync, 1u);
         const Partial pr = block_partial(run), pl = block_partial(last);
         if (tid == 0) {
             next_u = claim;
@@ -706,9 +709,11 @@ static cudaError_t plane_bands_launch(cdi_batch *b, int n, bool keep_prev, cudaS
 // One launch for the run of a batch of 2D boxes (plane_batch_kernel) with blocks of NT threads, at
 // most qmax per SM.  More boxes than slots: a box's run is cut into about 20 slots' worth of units
 // per box, so that the SMs end together.  keep_prev: also store the state before the last (as
-// single steps do); without it and for odd n the current state is only read.
+// single steps do); without it and for odd n the current state is only read.  probe_ns > 0: two
+// units per box, whose waits last that long at most.
 template <typename T, int NT, bool FACE>
-static cudaError_t plane_run_launch(cdi_batch *b, int n, bool keep_prev, int qmax, cudaStream_t s)
+static cudaError_t plane_run_launch(cdi_batch *b, int n, bool keep_prev, int qmax, cudaStream_t s,
+                                    unsigned long long probe_ns)
 {
     auto kernel = cdi::plane_batch_kernel<T, NT, FACE>;
     const size_t smem = b->plane_run_bytes;
@@ -722,7 +727,11 @@ static cudaError_t plane_run_launch(cdi_batch *b, int n, bool keep_prev, int qma
     if (b->nbox > slots) nchunks = std::min(n, (20 * slots + b->nbox - 1) / b->nbox);
     const int grid = (int)std::min<long long>(slots, (long long)b->nbox * nchunks);
     // a unit waits at most for the units before it of every box on its block
-    const unsigned long long wait_ns = 1000000000ull + 4ull * (unsigned long long)b->cells * (unsigned long long)n;
+    unsigned long long wait_ns = 1000000000ull + 4ull * (unsigned long long)b->cells * (unsigned long long)n;
+    if (probe_ns) {
+        nchunks = 2;
+        wait_ns = probe_ns;
+    }
     kernel<<<grid, NT, smem, s>>>((const BoxDev<T> *)b->boxes_dev, b->unit_box, b->nbox, b->parity, n, nchunks,
                                   keep_prev, b->recs, b->plane_sync, wait_ns);
     return cudaGetLastError();
@@ -734,16 +743,17 @@ static cudaError_t plane_run_launch(cdi_batch *b, int n, bool keep_prev, int qma
 // against 46.5 us per step), until every SM has several boxes anyway and two blocks (of 256
 // threads) fill each other's barriers (1024 boxes: 159 against 165 us).
 template <typename T, bool FACE>
-static cudaError_t plane_run_t(cdi_batch *b, int n, bool keep_prev, cudaStream_t s)
+static cudaError_t plane_run_t(cdi_batch *b, int n, bool keep_prev, cudaStream_t s, unsigned long long probe_ns)
 {
-    if (b->plane_nb) {
+    if (b->plane_nb && !probe_ns) {
         const cudaError_t e = plane_bands_launch<T, FACE>(b, n, keep_prev, s);
         if (e != cudaErrorCooperativeLaunchTooLarge) return e;
         (void)cudaGetLastError();  // a context with fewer SMs: whole boxes
         b->plane_nb = 0;
     }
-    if (sizeof(T) == 8 && b->nbox >= 4 * b->sms) return plane_run_launch<T, 256, FACE>(b, n, keep_prev, 2, s);
-    return plane_run_launch<T, 512, FACE>(b, n, keep_prev, sizeof(T) == 4 ? 2 : 1, s);
+    if (sizeof(T) == 8 && b->nbox >= 4 * b->sms)
+        return plane_run_launch<T, 256, FACE>(b, n, keep_prev, 2, s, probe_ns);
+    return plane_run_launch<T, 512, FACE>(b, n, keep_prev, sizeof(T) == 4 ? 2 : 1, s, probe_ns);
 }
 
 static bool plane_run_applies(const cdi_batch *b, int n)
@@ -751,14 +761,16 @@ static bool plane_run_applies(const cdi_batch *b, int n)
     return b->tile == cdi::BATCH_TILE_PLANE && b->plane_run_bytes && n > 1;
 }
 
-static int plane_run(cdi_batch *b, int n, bool keep_prev, cudaStream_t s)
+static int plane_run(cdi_batch *b, int n, bool keep_prev, cudaStream_t s, unsigned long long probe_ns = 0)
 {
     const bool face = b->sharpen == CDI_SHARPEN_FACE;
     cudaError_t e;
     if (b->dtype == CDI_F64)
-        e = face ? plane_run_t<double, true>(b, n, keep_prev, s) : plane_run_t<double, false>(b, n, keep_prev, s);
+        e = face ? plane_run_t<double, true>(b, n, keep_prev, s, probe_ns)
+                 : plane_run_t<double, false>(b, n, keep_prev, s, probe_ns);
     else
-        e = face ? plane_run_t<float, true>(b, n, keep_prev, s) : plane_run_t<float, false>(b, n, keep_prev, s);
+        e = face ? plane_run_t<float, true>(b, n, keep_prev, s, probe_ns)
+                 : plane_run_t<float, false>(b, n, keep_prev, s, probe_ns);
     if (e != cudaSuccess) return cdi::set_error(CDI_ERR_CUDA, "batch plane run: %s", cudaGetErrorString(e));
     return CDI_OK;
 }
@@ -1291,16 +1303,9 @@ int cdi_batch_stats(cdi_batch *b, cdi_stats *out, void *stream)
     return CDI_OK;
 }
 
-// One launch whose units wait for a step their boxes never reach: the first wait
-// runs out after limit_s, the others give up on seeing its status bit, and no
-// unit is stepped (fields, records and counters are left as they were).
-int cdi_batch_probe_box_wait(cdi_batch *b, double limit_s, void *stream)
+// Whether a wait of the probe launched on s ran out (the status words are cleared).
+static int probe_result(cdi_batch *b, cudaStream_t s)
 {
-    if (!b) return cdi::set_error(CDI_ERR_ARG, "batch is NULL");
-    if (!(limit_s > 0.0 && limit_s <= 2.0)) return cdi::set_error(CDI_ERR_ARG, "limit_s must be in (0, 2]");
-    cudaStream_t s = (cudaStream_t)stream;
-    const cdi::BatchSync y = {b->queue, b->epoch, 1 << 30, 1, (unsigned long long)(limit_s * 1e9)};
-    if (int rc = launch_any(b, b->parity, 1.0, s, 0, &y)) return rc;
     unsigned int st = 0;
     cudaError_t e;
     if ((e = cudaMemcpyAsync(&st, b->status, sizeof(st), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
@@ -1311,6 +1316,30 @@ int cdi_batch_probe_box_wait(cdi_batch *b, double limit_s, void *stream)
         (e = cudaStreamSynchronize(s)) != cudaSuccess)
         return cdi::set_error(CDI_ERR_CUDA, "probe status reset: %s", cudaGetErrorString(e));
     return cdi::set_error(CDI_ERR_TIMEOUT, "bounded wait for a box's previous step ran out (probe)");
+}
+
+// One launch whose units wait for a step their boxes never reach: the first wait
+// runs out after limit_s, the others give up on seeing its status bit, and no
+// unit is stepped (fields, records and counters are left as they were).  Tile 4 where
+// a run holds whole boxes on chip: then such a run of two units per box whose counter
+// hands out the second ones only, which wait for the first.
+int cdi_batch_probe_box_wait(cdi_batch *b, double limit_s, void *stream)
+{
+    if (!b) return cdi::set_error(CDI_ERR_ARG, "batch is NULL");
+    if (!(limit_s > 0.0 && limit_s <= 2.0)) return cdi::set_error(CDI_ERR_ARG, "limit_s must be in (0, 2]");
+    cudaStream_t s = (cudaStream_t)stream;
+    const cdi::BatchSync y = {b->queue, b->epoch, 1 << 30, 1, (unsigned long long)(limit_s * 1e9)};
+    if (int rc = launch_any(b, b->parity, 1.0, s, 0, &y)) return rc;
+    const int rc = probe_result(b, s);
+    if (rc != CDI_ERR_TIMEOUT || b->plane_nb || !plane_run_applies(b, 2)) return rc;
+    const unsigned int first = (unsigned)b->nbox;
+    const cudaError_t e = cudaMemcpyAsync(b->plane_sync, &first, sizeof(first), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return cdi::set_error(CDI_ERR_CUDA, "probe setup: %s", cudaGetErrorString(e));
+    if (int r = plane_run(b, 2, true, s, y.wait_ns)) {
+        cudaMemsetAsync(b->plane_sync, 0, sizeof(first), s);
+        return r;
+    }
+    return probe_result(b, s);
 }
 
 int cdi_batch_reset_run_stats(cdi_batch *b, void *stream)

@@ -132,3 +132,46 @@ def test_batch_autotune_leaves_state_and_records():
     ref, st = [bt.current(i).clone() for i in range(3)], bt.stats()
     bt.autotune(reps=2)
     assert all(torch.equal(bt.current(i), r) for i, r in enumerate(ref)) and bt.stats() == st
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("nbox", [90, 700])
+def test_units_wait_bounded_and_are_claimed_in_order(dtype, nbox):
+    """A unit after its box's first waits for the one before it, which must have been claimed earlier:
+    with the first units withheld every block's claim is a waiting one, no box is stepped, the wait
+    runs out and is reported, and the next run is that of an untouched twin."""
+    b0 = boxes(dtype, [(5 + i % 7, 4 + i % 11) for i in range(nbox)], 21)
+    twin = [dict(x, phi_a=x["phi_a"].clone(), phi_b=x["phi_b"].clone()) for x in b0]
+    bt = [cdi.Batch(x) for x in (b0, twin)]
+    for b in bt:
+        b.set_launch(4, 0)
+        b.run(4)
+    ref = [bt[0].current(i).clone() for i in range(nbox)]
+    with pytest.raises(cdi.CDIError) as e:
+        bt[0].probe_box_wait(0.02)
+    assert e.value.code == cdi.CDI_ERR_TIMEOUT
+    assert all(torch.equal(bt[0].current(i), ref[i]) for i in range(nbox))
+    for b in bt:
+        b.run(5)
+    assert all(torch.equal(bt[0].current(i), bt[1].current(i)) for i in range(nbox))
+    assert bt[0].stats() == bt[1].stats()
+
+
+def test_run_beside_another_streams_kernels():
+    """A chunked run whose blocks start late, because another stream's kernels hold the SMs."""
+    b0 = boxes(torch.float32, [(20, 30)] * 700, 5)
+    twin = [dict(x, phi_a=x["phi_a"].clone(), phi_b=x["phi_b"].clone()) for x in b0]
+    bt = [cdi.Batch(x) for x in (b0, twin)]
+    for b in bt:
+        b.set_launch(4, 0)
+    bt[1].run(64)
+    m = torch.rand(4096, 4096, device="cuda")
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        for _ in range(8):
+            m = (m @ m).clamp_(0, 1)
+    bt[0].run(64)
+    torch.cuda.synchronize()
+    assert all(torch.equal(bt[0].current(i), bt[1].current(i)) for i in range(700))
+    assert bt[0].stats() == bt[1].stats()
