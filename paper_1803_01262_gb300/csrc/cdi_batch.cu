@@ -761,17 +761,28 @@ static bool plane_run_applies(const cdi_batch *b, int n)
     return b->tile == cdi::BATCH_TILE_PLANE && b->plane_run_bytes && n > 1;
 }
 
+// n steps from the current state, the batch's parity following.  A block counts the violations of
+// its unit, every step's, in 32 bits (the records take the sums in 64): a launch is cut where a box
+// could have 2^31 of them, so a count never wraps.
 static int plane_run(cdi_batch *b, int n, bool keep_prev, cudaStream_t s, unsigned long long probe_ns = 0)
 {
     const bool face = b->sharpen == CDI_SHARPEN_FACE;
-    cudaError_t e;
-    if (b->dtype == CDI_F64)
-        e = face ? plane_run_t<double, true>(b, n, keep_prev, s, probe_ns)
-                 : plane_run_t<double, false>(b, n, keep_prev, s, probe_ns);
-    else
-        e = face ? plane_run_t<float, true>(b, n, keep_prev, s, probe_ns)
-                 : plane_run_t<float, false>(b, n, keep_prev, s, probe_ns);
-    if (e != cudaSuccess) return cdi::set_error(CDI_ERR_CUDA, "batch plane run: %s", cudaGetErrorString(e));
+    long long cells = 1;
+    for (const cdi_box_desc &x : b->desc) cells = std::max(cells, (long long)x.nx * x.ny);
+    const long long most = ((1LL << 31) - 1) / cells;  // steps of a launch (a box held on chip: < 2^15 cells)
+    const int launches = (int)((n + most - 1) / most);
+    for (int l = 0, i0 = 0; l < launches; ++l) {
+        const int i1 = (int)((long long)(l + 1) * n / launches), m = i1 - i0;
+        const bool kp = keep_prev && l == launches - 1;
+        cudaError_t e;
+        if (b->dtype == CDI_F64)
+            e = face ? plane_run_t<double, true>(b, m, kp, s, probe_ns) : plane_run_t<double, false>(b, m, kp, s, probe_ns);
+        else
+            e = face ? plane_run_t<float, true>(b, m, kp, s, probe_ns) : plane_run_t<float, false>(b, m, kp, s, probe_ns);
+        if (e != cudaSuccess) return cdi::set_error(CDI_ERR_CUDA, "batch plane run: %s", cudaGetErrorString(e));
+        b->parity ^= m & 1;
+        i0 = i1;
+    }
     return CDI_OK;
 }
 
@@ -1242,11 +1253,7 @@ int cdi_batch_run(cdi_batch *b, int nsteps, void *stream)
     if (!b) return cdi::set_error(CDI_ERR_ARG, "batch is NULL");
     if (nsteps < 1) return cdi::set_error(CDI_ERR_ARG, "nsteps must be >= 1");
     cudaError_t e;
-    if (plane_run_applies(b, nsteps)) {
-        if (int rc = plane_run(b, nsteps, true, (cudaStream_t)stream)) return rc;
-        b->parity ^= (nsteps & 1);
-        return CDI_OK;
-    }
+    if (plane_run_applies(b, nsteps)) return plane_run(b, nsteps, true, (cudaStream_t)stream);
     const std::pair<int, int> key(nsteps, b->parity);
     auto it = b->graphs.find(key);
     if (it == b->graphs.end()) {
@@ -1441,7 +1448,11 @@ int cdi_batch_autotune(cdi_batch *b, int reps, float *best_ms, void *stream)
             const int n = reps > 6 ? reps : 6;
             if (!pr && (rc = reserve_run(b, n)) != CDI_OK) break;
             auto trial = [&](int k) {
-                if (pr) return plane_run(b, kTrial, false, s);
+                if (pr) {
+                    const int parity = b->parity, r = plane_run(b, kTrial, false, s);
+                    b->parity = parity;
+                    return r;
+                }
                 int r = zero_run(b, k, s);
                 for (int i = 0; i < k && r == CDI_OK; ++i) {
                     const cdi::BatchSync y = run_sync(b, i);

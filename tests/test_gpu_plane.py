@@ -175,3 +175,18 @@ def test_run_beside_another_streams_kernels():
     torch.cuda.synchronize()
     assert all(torch.equal(bt[0].current(i), bt[1].current(i)) for i in range(700))
     assert bt[0].stats() == bt[1].stats()
+
+
+def test_violation_counts_of_a_long_run():
+    """More than 2^32 violations of one box in one run: every cell of 118^2 is one in each of 310000
+    steps (dt = 0 keeps the field)."""
+    n, steps = 118, 310000
+    z = torch.zeros((1, n, n), device="cuda")
+    b = cdi.Batch([dict(dx=1.0, dt=0.0, eps=1.0, gamma=1.0, u=z, v=z, w=z, phi_a=torch.full_like(z, 2.0),
+                        phi_b=torch.empty_like(z)) for _ in range(90)])
+    b.set_launch(4, 0)
+    b.run(steps)
+    for s in b.stats():
+        assert s["n_strict_run"] == s["n_tol_run"] == n * n * steps and s["steps_run"] == steps
+        assert s["n_strict"] == s["n_tol"] == n * n and s["min_run"] == s["max_run"] == 2.0
+    assert b.info()["parity"] == 0 and all(torch.equal(b.current(i), z + 2) for i in range(90))
