@@ -246,7 +246,8 @@ CDI_API int cdi_step_adjoint(cdi_grid *g, const void *phi_k, const void *lam_nex
  * statistics record is the last step's, as after cdi_run.  cdi_adjoint_path: for i = nsteps - 1
  * .. 0 the adjoint step at phi[i] with vel_scale[i], from lam_a to lam_b and back; *final_in_b is
  * 1 if the result is in lam_b.  Arguments are otherwise those of cdi_step and cdi_step_adjoint;
- * the arrays of pointers and scales are host memory, read during the call.  On an error, steps
+ * the arrays of pointers and scales are host memory, read during the call.  cdi_step_path enqueues
+ * nothing if it refuses any step's arguments; on other errors, and in cdi_adjoint_path, steps
  * before the failing one may have been enqueued. */
 CDI_API int cdi_step_path(cdi_grid *g, void *const *phi, int nsteps, double dt, double eps, double gamma,
                           const double *vel_scale, void *stream);

@@ -1244,11 +1244,15 @@ int cdi_step_path(cdi_grid *g, void *const *phi, int nsteps, double dt, double e
                   const double *vel_scale, void *stream)
 {
     cdi::NvtxRange nvtx_("cdi_step_path");
+    if (int rc = check_grid(g)) return rc;
     if (nsteps < 0 || (nsteps > 0 && (!phi || !vel_scale))) return fail(CDI_ERR_ARG, "bad step path");
-    cudaStream_t s = (cudaStream_t)stream;
-    const bool defer = nsteps > 1 && 2 * (g ? g->fwd.nblocks : 0) <= (g ? g->capacity : 0);  // as in cdi_run
-    for (int i = 0; i < nsteps; ++i) {
+    // every step's arguments before the first launch: a step's statistics are folded into the
+    // record by the step after it, which must not be refused
+    for (int i = 0; i < nsteps; ++i)
         if (int rc = check_step_args(g, phi[i], phi[i + 1], dt, eps, gamma, vel_scale[i])) return rc;
+    cudaStream_t s = (cudaStream_t)stream;
+    const bool defer = nsteps > 1 && 2 * g->fwd.nblocks <= g->capacity;  // as in cdi_run
+    for (int i = 0; i < nsteps; ++i) {
         const DeferCfg d = {i & 1, i + 1 < nsteps, i > 0};
         const DeferCfg *dp = defer ? &d : nullptr;
         const int rc = g->dtype == CDI_F64

@@ -71,3 +71,20 @@ def test_overridden_step_is_called():
     out = AG.rollout(phi, *vel, g, 3, *prm)
     g2, _, _, _ = setup((5, 9, 16), torch.float32)
     assert Counting.n == 3 and torch.equal(out, AG.rollout(phi, *vel, g2, 3, *prm))
+
+
+@pytest.mark.parametrize("bad", ["in place", "scale"])
+def test_a_refused_path_enqueues_nothing(bad):
+    """A path refused for a later step leaves the states and the run statistics as they were."""
+    g, phi, vel, prm = setup((6, 16, 64), torch.float32)
+    g.step(phi, torch.empty_like(phi), *prm)
+    st = g.stats()
+    out = torch.full_like(phi, 7.0)
+    states, scales = ([phi, out, out], [1.0, 1.0]) if bad == "in place" else (
+        [phi, out, phi.clone()], [1.0, float("inf")])
+    with pytest.raises(cdi.CDIError) as e:
+        g.step_path(states, *prm, scales)
+    assert e.value.code == cdi.CDI_ERR_ARG
+    assert (out == 7.0).all() and g.stats() == st
+    with pytest.raises(cdi.CDIError):       # no grid, no steps
+        cdi._ck(cdi.lib().cdi_step_path(None, None, 0, *prm, None, None))
