@@ -211,7 +211,7 @@ static int fwd_cfg_rk(const cdi_grid *g, int tile, LaunchCfg *c) { return fwd_cf
 
 static int default_fwd_tile(const cdi_grid *g)
 {
-    return g->sharpen == CDI_SHARPEN_FACE ? 0 : cdi::fwd_default_tile((int)esize(g), g->nx, g->ny, g->nz);
+    return g->sharpen == CDI_SHARPEN_FACE ? 0 : cdi::fwd_default_tile((int)esize(g), g->nx, g->ny, g->nz, g->sm_count);
 }
 
 // Vector adjoint: z chunking from the forward cost model (rounds of the

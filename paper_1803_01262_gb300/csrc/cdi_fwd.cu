@@ -440,27 +440,49 @@ void fwd_tile_dims(int tile, int esize, int *bw, int *bh)
     *bh = tile == 5 || tile == 8 ? (row ? 6 : 8) : (row ? 14 : 16);
 }
 
+// Work of the busiest SM in FP64, where the FP64 pipe bounds a kernel and staging does not: tiles of
+// 32 x bh cells whose plane costs its rows and `ring` rows more (the tile's sharpening ring), columns
+// shared out evenly, `pro` planes of prologue for each column a share touches.
+double fp64_tile_cost(int bh, double ring, double pro, int nx, int ny, int nz, int sms)
+{
+    const long long tiles = (long long)((nx + 31) / 32) * ((ny + bh - 1) / bh);
+    const long long share = (tiles * nz + sms - 1) / sms;
+    return ((double)share + pro * (double)((share + nz - 1) / nz)) * (bh + ring);
+}
+
 // Default tile of an Euler step (centre form): a vector kernel where the box is wide enough to
 // use its 16 vectors per row (FP32 rows of 16 cells and more: one-cell-per-thread tiles cost
 // three times the instructions per lane, and waste half as many lanes at most), the 14-row tile
 // unless the 6-row one covers ny with less work (each tile row of blocks pays two ring rows),
-// else one cell per thread.  FP64, whose time is FP64 instructions, takes the vector kernel on
-// aligned rows of 48 cells and more, and the row kernel on other rows of 64 and more
-// (129^3: 306 us with the 32x16 tile, 289 us).  Unaligned FP32 rows of boxes whose arrays do not
-// stay in L2 (4 M cells: 80 MB) take the 6-row tile, whose four blocks per SM leave L1 more room
-// than the 14-row tile's two (row_vel_slots): 255^3 90.1 -> 83.9 us, 160x177x190 31.7 -> 31.0;
-// below, the 14-row one is faster (129^3 19.4 against 20.9 us).
-int fwd_default_tile(int esize, int nx, int ny, int nz)
+// else one cell per thread.  Unaligned FP32 rows of 3D boxes of 4 M cells and more take the 6-row
+// tile (row_vel_slots): 255^3 90.1 -> 83.9 us, 160x177x190 31.7 -> 31.0; below, the 14-row one is
+// faster (129^3 19.4 against 20.9 us), and in 2D (2049^2 54.4 against 58.2 us).  That line was
+// measured on odd rows; rows on pairs lie on either side of it (6 rows against 14: 130x256x256
+// 55.6 and 60.4 us, 162x177x190 32.3 and 33.3, 254^3 78.8 and 76.7, 514x256x128 90.0 and 87.0).
+// FP64, whose time is FP64 instructions, takes the vector kernel on aligned rows of 48 cells and
+// more.  Its other rows cost the same per cell in either kernel, so the one whose rows cover ny
+// with less work is taken, by fp64_tile_cost with the ring and prologue that fit 336 boxes of 65..201
+// by 2..150 by 4..150 cells (the choice is 1.5% off the better of the two on average; the row kernel
+// throughout 5%, up to 44%; one cell per thread throughout 12%): 129^3 row kernel, 289 against 306 us,
+// 129x64x64 one cell per thread, 81 against 91 us, 129x7x300 62 against 78.  A 2D box stays on the
+// one-cell-per-thread tiles, whose single-plane body evaluates the sharpening of one plane and no z
+// flux: 129^2 17.5 against 18.0 us, 513^2 39 against 66, 1001^2 110 against 193, 2049^2 425 against 757.
+// (FP32, whose planes move through memory, gains in 2D too: 129^2 8.3 -> 5.1 us, 513^2 12.4 -> 9.2,
+// 1001^2 27.7 -> 15.8, 2049^2 94.4 -> 54.4.)
+int fwd_default_tile(int esize, int nx, int ny, int nz, int sms)
 {
     const int vx = 16 / esize;
     const bool al = nx % vx == 0;
-    if (esize == 4 ? nx >= 16 : (al ? nx >= 48 : nx >= 64)) {
-        if (esize == 8 && al) return ny >= 12 ? 4 : 5;
-        const int w14 = (ny + 13) / 14 * 16, w6 = (ny + 5) / 6 * 8;
-        const bool big = esize == 4 && !al && (long long)nx * ny * nz >= 4000000;
-        return (w6 < w14 || big ? 5 : 4) + (al ? 0 : 3);
-    }
-    return (nx >= 32 && ny >= 16) ? 1 : 3;
+    const int scalar = (nx >= 32 && ny >= 16) ? 1 : 3;
+    if (esize == 8 && al) return nx >= 48 ? (ny >= 12 ? 4 : 5) : scalar;
+    if (nx < (esize == 4 ? 16 : 64)) return scalar;
+    const int w14 = (ny + 13) / 14 * 16, w6 = (ny + 5) / 6 * 8;
+    const bool big = esize == 4 && !al && nz > 1 && (long long)nx * ny * nz >= 4000000;
+    const int row = (w6 < w14 || big ? 5 : 4) + (al ? 0 : 3);
+    if (esize == 4) return row;
+    if (nz == 1) return scalar;
+    const double crow = fp64_tile_cost(row == 7 ? 14 : 6, 4, 1, nx, ny, nz, sms);
+    return crow < fp64_tile_cost(scalar == 1 ? 16 : 4, 4, 1, nx, ny, nz, sms) ? row : scalar;
 }
 
 long long fwd_tiles_xy(int tile, int esize, int nx, int ny)

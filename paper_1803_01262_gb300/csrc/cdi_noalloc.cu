@@ -97,7 +97,7 @@ static int noalloc_t(int nx, int ny, int nz, double dx, const void *in, void *ou
                      void *stats_dev, NoAllocScratch *scr, int sms, cudaStream_t s)
 {
     const int es = (int)sizeof(T);
-    const int tile = cdi::fwd_default_tile(es, nx, ny, nz);
+    const int tile = cdi::fwd_default_tile(es, nx, ny, nz, sms);
     int resident = 0;
     cudaError_t e = cdi::fwd_occupancy<T>(tile, false, &resident);
     if (e != cudaSuccess) return na_fail(CDI_ERR_CUDA, "occupancy query", e);
