@@ -68,6 +68,7 @@ struct cdi_grid {
     // launch configuration of the forward and adjoint kernels
     LaunchCfg fwd, adj;
     int adj_blocks[4];         // launch_adj's resident blocks (0: not asked yet)
+    bool fwd_dflt;  // fwd is the default launch, not a chosen or an autotuned one
     LaunchCfg rk;  // Runge-Kutta stage kernels (set on first use; nblocks 0 = unset)
     LaunchCfg slab;  // z slabs of the pipelined host step (set on first use; nblocks 0 = unset)
     LaunchCfg tb;    // two steps per pass (cdi_run with depth 2; nblocks 0 = unset)
@@ -355,6 +356,7 @@ int cdi_create_grid(cdi_grid **out, int nx, int ny, int nz, double dx, int dtype
         cdi_destroy_grid(g);
         return rc;
     }
+    g->fwd_dflt = true;
     g->adj = adj_default(g);
     if (int rc = plane_setup(g)) {
         cdi_destroy_grid(g);
@@ -758,8 +760,8 @@ static int step2_t(cdi_grid *g, const void *in, void *out, double dt, double eps
 
 // One Runge-Kutta stage: evaluates r = dt * RHS(in) and writes
 //   out = (base ? base : in) + alpha r + (q ? delta q : 0),  qout = mu (q ? q : in) + beta r.
-// Uses the RK variant of the configured tile's kernel family (vectors, aligned rows
-// or any; or the one-cell-per-thread 32x16 / 32x4 tile).
+// Uses the default stage tile, or the RK variant of the configured tile's kernel family
+// (vectors, aligned rows or any; or the one-cell-per-thread 32x16 / 32x4 tile).
 struct RkStage {
     const void *in, *base, *q;
     void *out, *qout;
@@ -772,7 +774,10 @@ template <typename T>
 static int rk_stage_t(cdi_grid *g, const RkStage &st, double dt, double eps, double gamma, cudaStream_t s)
 {
     if (g->rk.nblocks == 0) {  // first use: RK launch configuration for this grid
-        const int tile = g->fwd.tile >= 7 ? 7 : g->fwd.tile >= 4 ? 4 : (g->nx >= 32 && g->ny >= 16) ? 1 : 3;
+        const int tile = g->fwd_dflt      ? cdi::fwd_default_rk_tile((int)esize(g), g->nx, g->ny, g->nz, g->sm_count)
+                         : g->fwd.tile >= 7 ? 7
+                         : g->fwd.tile >= 4 ? 4
+                                            : (g->nx >= 32 && g->ny >= 16) ? 1 : 3;
         if (int rc = fwd_cfg_rk(g, tile, &g->rk)) return rc;
     }
     cdi::FwdArgs<T> a;
@@ -1289,6 +1294,7 @@ int cdi_set_launch(cdi_grid *g, int which, int tile, int blocks_per_sm, int nchu
         if (int rc = fwd_cfg(g, tile, blocks_per_sm, nchunks, &c)) return rc;
         g->plane_on = dflt && g->plane_bands > 0;
         g->fwd = c;
+        g->fwd_dflt = dflt;
         g->rk.nblocks = 0;  // the Runge-Kutta configuration follows on next use
         return CDI_OK;
     }
@@ -1457,6 +1463,7 @@ int cdi_set_sharpening(cdi_grid *g, int mode)
         return rc;
     }
     g->fwd = c;
+    g->fwd_dflt = true;
     g->rk.nblocks = 0;
     if (mode != CDI_SHARPEN_CENTRE) g->run_depth = 1;  // two steps per pass: centre form only
     return CDI_OK;
@@ -1595,6 +1602,7 @@ int cdi_autotune(cdi_grid *g, void *phi_a, void *phi_b, double dt, double eps, d
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     g->fwd = rc == CDI_OK ? best : saved;
+    if (rc == CDI_OK) g->fwd_dflt = false;
     g->rk.nblocks = 0;
     if (rc == CDI_OK) {
         g->plane_on = g->plane_bands > 0;

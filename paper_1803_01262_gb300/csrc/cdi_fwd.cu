@@ -485,6 +485,29 @@ int fwd_default_tile(int esize, int nx, int ny, int nz, int sms)
     return crow < fp64_tile_cost(scalar == 1 ? 16 : 4, 4, 1, nx, ny, nz, sms) ? row : scalar;
 }
 
+// Default tile of a Runge-Kutta stage: vectors as for the Euler step (14 rows), but
+//   - FP64 on other rows by fp64_tile_cost with the ring and prologue that fit the stages (421
+//     boxes, 2D ones included: the choice is 1% off the better kernel on average and 14% at most; the
+//     row kernel throughout 13% and up to two times): RK2 steps of 129x64x64 168 us with one cell per
+//     thread, 192 with the row kernel, 129x28x150 181 and 166; 2D, where a stage has no single-plane
+//     body, 129^2 45 and 34 us, 2049^2 1742 and 1577, but a row of 10^6 cells 1639 and 4864;
+//   - FP32 boxes of at most four rows and 250 k cells and more, one 14-row tile of which is mostly
+//     empty (RK2: 300001x1 98 us with one cell per thread, 110 with vectors, 1000003x1 283 and 349;
+//     100003x1 43 and 41).
+int fwd_default_rk_tile(int esize, int nx, int ny, int nz, int sms)
+{
+    const int scalar = (nx >= 32 && ny >= 16) ? 1 : 3;
+    const bool al = nx % (16 / esize) == 0;
+    if (esize == 4) {
+        if (nx < 16 || (ny <= 4 && (long long)nx * ny * nz >= 250000)) return scalar;
+        return al ? 4 : 7;
+    }
+    if (al) return nx >= 48 ? 4 : scalar;
+    if (nx < 64) return scalar;
+    const double crow = fp64_tile_cost(14, 4, 0.5, nx, ny, nz, sms);
+    return crow < fp64_tile_cost(scalar == 1 ? 16 : 4, 2, 1, nx, ny, nz, sms) ? 7 : scalar;
+}
+
 long long fwd_tiles_xy(int tile, int esize, int nx, int ny)
 {
     int bw, bh;

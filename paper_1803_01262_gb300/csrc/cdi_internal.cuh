@@ -110,6 +110,7 @@ struct LaunchCfg {
 int fwd_num_tiles();
 bool fwd_tile_is_vec(int tile);  // tiles that need rows on 16-byte boundaries
 int fwd_default_tile(int esize, int nx, int ny, int nz, int sms);
+int fwd_default_rk_tile(int esize, int nx, int ny, int nz, int sms);
 double fp64_tile_cost(int bh, double ring, double pro, int nx, int ny, int nz, int sms);
 void fwd_tile_dims(int tile, int esize, int *bw, int *bh);
 long long fwd_tiles_xy(int tile, int esize, int nx, int ny);
