@@ -250,9 +250,16 @@ static int adj_vec_zchunk(const cdi_grid *g)
 static bool adj_vec_eligible(const cdi_grid *g) { return g->nx % (16 / (int)esize(g)) == 0; }
 
 // Adjoint launch: the row kernel (tile 3 where rows start on 16-byte boundaries, else 4) for
-// rows of 16 cells and more, as the forward step (fwd_default_tile; FP64 too: its formulas take
-// fewer FP64 operations); else a one-cell-per-thread tile with a z chunk giving about eight
-// blocks per SM.
+// rows of 16 cells and more, as the forward step; else a one-cell-per-thread tile with a z chunk
+// giving about eight blocks per SM, also where a 14-row tile is mostly empty:
+//   - FP32 boxes of at most four rows (1001x1 5.1 us with one cell per thread, 5.3 with the row
+//     kernel, 201x2x300 9.2 and 11.5, 30001x1 9.2 and 11.4, 1000003x1 127 and 237; 10001x1 7.35 and
+//     7.0);
+//   - FP64, bound by its FP64 operations, of which the row kernel's formulas take fewer, by
+//     fp64_tile_cost against the busiest SM's blocks at 1.6 times the cost per cell (fits 595 boxes
+//     of 16..201 by 2..150 by 4..150 cells and rows of up to 10^6: the choice is 0.1% off the better
+//     kernel on average, the row kernel throughout 6%): 129x129x150 742 us with one cell per thread,
+//     435 with the row kernel, 16x64x64 47 and 54, 129x5x64 47 and 54, 1000003x1 1664 and 3690.
 static LaunchCfg adj_scalar_default(const cdi_grid *g)
 {
     LaunchCfg c;
@@ -271,7 +278,14 @@ static LaunchCfg adj_scalar_default(const cdi_grid *g)
 
 static LaunchCfg adj_default(const cdi_grid *g)
 {
-    if (g->nx < 16) return adj_scalar_default(g);
+    const LaunchCfg sc = adj_scalar_default(g);
+    if (g->nx < 16 || (g->dtype == CDI_F32 && g->ny <= 4)) return sc;
+    if (g->dtype == CDI_F64) {
+        const int bh = sc.tile == 1 ? 16 : 4;
+        const long long blocks = cdi::adj_blocks(sc.tile, sc.zchunk, g->nx, g->ny, g->nz);
+        const double cs = (double)((blocks + g->sm_count - 1) / g->sm_count) * (sc.zchunk + 2) * (bh + 1);
+        if (8 * cs <= 5 * cdi::fp64_tile_cost(14, 2, 2, g->nx, g->ny, g->nz, g->sm_count)) return sc;
+    }
     LaunchCfg c;
     c.tile = adj_vec_eligible(g) ? 3 : 4;
     c.zchunk = adj_vec_zchunk(g);

@@ -60,3 +60,16 @@ def stage_kernels(shape, dtype):
 def test_runge_kutta_stage(dtype, shape, row):
     for name in stage_kernels(shape, dtype):
         assert ("fwd_row_kernel" in name) == row, name
+
+
+@pytest.mark.parametrize("dtype,shape,row", [
+    (torch.float32, (1, 1, 1001), False), (torch.float32, (300, 2, 201), False), (torch.float32, (1, 4, 1000003), False),
+    (torch.float32, (1, 5, 1000003), True), (torch.float32, (64, 64, 67), True), (torch.float64, (1, 1, 1001), False),
+    (torch.float64, (64, 64, 16), False), (torch.float64, (64, 5, 129), False), (torch.float64, (1, 17, 17), False),
+    (torch.float64, (16, 16, 16), True), (torch.float64, (1, 129, 129), True), (torch.float64, (64, 64, 33), True),
+    (torch.float64, (150, 7, 129), True), (torch.float64, (129, 129, 129), True)])
+def test_adjoint(dtype, shape, row):
+    g = cdi.Grid(*shape[::-1], 0.01, dtype)
+    t = g.get_launch(cdi.CDI_KERNEL_ADJOINT)["tile"]
+    aligned = shape[2] % (4 if dtype == torch.float32 else 2) == 0
+    assert t == ((3 if aligned else 4) if row else (1 if shape[2] >= 32 and shape[1] >= 16 else 2))
