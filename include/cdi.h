@@ -384,9 +384,10 @@ CDI_API int cdi_batch_get_launch(const cdi_batch *b, int *tile, int *zdepth, int
 /* Time every tile x zdepth in {8, 16, 32, 64, whole} (a batch of 2D boxes: every
  * tile once, tile 4 where it applies; tile 5 where it applies) with max(reps, 6) launches
  * each, overlapping as in a run (after one warm-up, which alone rules out what takes three times
- * the best), and keep the fastest; *best_ms (nullable) gets its time per launch.  The trial launches read the current state and write the other
- * buffer only, and the statistics records are restored, so the batch's state
- * and records are as before the call.  Synchronises. */
+ * the best and 20 us more; a run that holds 2D boxes on chip is timed as runs of several steps),
+ * and keep the fastest; *best_ms (nullable) gets its time per step.  The trial launches read
+ * the current state and write the other buffer only, and the statistics records are restored,
+ * so the batch's state and records are as before the call.  Synchronises. */
 CDI_API int cdi_batch_autotune(cdi_batch *b, int reps, float *best_ms, void *stream);
 
 /* Sharpening form of the forward step.  CDI_SHARPEN_CENTRE (the default) is

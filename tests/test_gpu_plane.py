@@ -2,12 +2,17 @@
 the same buffers, extrema and counts as one launch per step on the one-cell-per-thread tile, bit
 for bit (the sums to rounding), for one band (no neighbour), bands of two rows and of uneven
 heights, odd rows, every buffer parity, runs of several launches and time-dependent velocities."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
 from paper_1803_01262_gb300 import cdi
 
 pytestmark = pytest.mark.gpu
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def setup(ny, nx, dtype, seed):
@@ -190,3 +195,20 @@ def test_violation_counts_of_a_long_run():
         assert s["n_strict_run"] == s["n_tol_run"] == n * n * steps and s["steps_run"] == steps
         assert s["n_strict"] == s["n_tol"] == n * n and s["min_run"] == s["max_run"] == 2.0
     assert b.info()["parity"] == 0 and all(torch.equal(b.current(i), z + 2) for i in range(90))
+
+
+def test_autotune_takes_the_run_on_chip_in_a_new_process():
+    """256 boxes of 50^2 in FP32: a run on chip takes a third of any other tile's time, also where the
+    autotuner's first trial of it loads its kernel."""
+    code = """
+import torch
+from paper_1803_01262_gb300 import cdi
+z = torch.rand((1, 50, 50), device="cuda")
+b = cdi.Batch([dict(dx=0.02, dt=1e-4, eps=0.02, gamma=1.0, u=z, v=z, w=z, phi_a=z.clone(), phi_b=z.clone())
+               for _ in range(256)])
+b.autotune(reps=2)
+print(b.get_launch()["tile"])
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=240, cwd=ROOT)
+    assert r.returncode == 0, r.stderr
+    assert r.stdout.split()[-1] == "4"
