@@ -180,9 +180,6 @@ batch_kernel(const BoxDev<T> *__restrict__ boxes, const int *__restrict__ unit_b
     __shared__ int fold, next_u, ready;
     const int tid = threadIdx.x + BX * threadIdx.y;
     unsigned int *const status = boxes[0].a.red.status;
-    // The next launch of a run may start once every block of this one has
-    // started; it takes the SMs as this launch's blocks finish.
-    grid_dep_launch();
     // Units are handed out in list order from a counter (queue[0]; every block
     // starts with unit blockIdx.x): a block takes the next unit when it is done
     // with one, so blocks that run faster take more.  The fields do not depend
@@ -199,6 +196,12 @@ batch_kernel(const BoxDev<T> *__restrict__ boxes, const int *__restrict__ unit_b
             __syncthreads();
             if (!ready) break;  // a wait gave up (reported); the remaining units are skipped
         }
+        // The next launch of a run may start once every block of this one has begun its first
+        // unit; it takes the SMs as this launch's blocks finish.  (Once every block had started,
+        // waiting or not, the launches of a small batch piled up and left the working one few SMs:
+        // one FP64 box of 64^3, 16 planes per unit, 52 us per step in runs of 4 and 144 in runs of
+        // 256; 50 so.)
+        if (u == (int)blockIdx.x) grid_dep_launch();
         FwdArgs<T> a = boxes[bi].a;
         if (parity) {
             T *t = a.out;

@@ -425,3 +425,27 @@ def test_run_wait_times_out_and_the_batch_stays_usable():
             assert a[k] == c[k], k
     with pytest.raises(cdi.CDIError):
         b1.probe_box_wait(5.0)          # limit out of range
+
+
+def test_long_runs_step_as_fast_as_short_ones():
+    """A run's launches overlap, but do not pile up: a batch whose launches leave most of the GPU
+    free takes no longer per step in a long run than in a short one (twice: the waiting launches'
+    blocks held the SMs' slots)."""
+    z = torch.rand((64, 64, 64), device="cuda", dtype=torch.float64)
+    b = cdi.Batch([dict(dx=0.01, dt=1e-6, eps=0.01, gamma=1.0, u=z, v=z, w=z, phi_a=z.clone(), phi_b=z.clone())])
+    b.set_launch(3, 16)
+
+    def per_step(n):
+        b.run(n)
+        best = float("inf")
+        for _ in range(5):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            e0.record()
+            b.run(n)
+            e1.record()
+            e1.synchronize()
+            best = min(best, e0.elapsed_time(e1) / n)
+        return best
+
+    assert per_step(128) <= 1.5 * per_step(4)
