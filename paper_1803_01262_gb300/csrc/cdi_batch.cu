@@ -710,8 +710,12 @@ static cudaError_t plane_bands_launch(cdi_batch *b, int n, bool keep_prev, cudaS
 }
 
 // One launch for the run of a batch of 2D boxes (plane_batch_kernel) with blocks of NT threads, at
-// most qmax per SM.  More boxes than slots: a box's run is cut into about 20 slots' worth of units
-// per box, so that the SMs end together.  keep_prev: also store the state before the last (as
+// most qmax per SM.  More boxes than slots: a box's run is cut into units so that the SMs end
+// together, at most about 20 slots' worth of them, by the rounds of units a slot gets and what a
+// unit costs besides its steps (load, reductions, hand-over: as much as a step of 6000 cells in FP32,
+// of 2000 in FP64).  With one unit per step where the run has few, 8 steps of 1000 boxes of 16^2
+// FP32 took 165 us, against 110 of single steps; so 44 (256 of 50^2 FP64 497 -> 404, 518; 64 steps
+// of 256 of 16^2 FP64 513 -> 374).  keep_prev: also store the state before the last (as
 // single steps do); without it and for odd n the current state is only read.  probe_ns > 0: two
 // units per box, whose waits last that long at most.
 template <typename T, int NT, bool FACE>
@@ -727,7 +731,17 @@ static cudaError_t plane_run_launch(cdi_batch *b, int n, bool keep_prev, int qma
     if (q < 1) return cudaErrorInvalidConfiguration;
     const int slots = std::min(q, qmax) * b->sms;
     int nchunks = 1;
-    if (b->nbox > slots) nchunks = std::min(n, (20 * slots + b->nbox - 1) / b->nbox);
+    if (b->nbox > slots) {
+        const double unit = (sizeof(T) == 4 ? 6000.0 : 2000.0) * b->nbox / (double)b->cells;  // in steps
+        double best = 1e300;
+        for (int c = 1; c <= std::min(n, (20 * slots + b->nbox - 1) / b->nbox); ++c) {
+            const double cost = (double)(((long long)b->nbox * c + slots - 1) / slots) * ((double)n / c + unit);
+            if (cost < best) {
+                best = cost;
+                nchunks = c;
+            }
+        }
+    }
     const int grid = (int)std::min<long long>(slots, (long long)b->nbox * nchunks);
     // a unit waits at most for the units before it of every box on its block
     unsigned long long wait_ns = 1000000000ull + 4ull * (unsigned long long)b->cells * (unsigned long long)n;

@@ -212,3 +212,27 @@ print(b.get_launch()["tile"])
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=240, cwd=ROOT)
     assert r.returncode == 0, r.stderr
     assert r.stdout.split()[-1] == "4"
+
+
+@pytest.mark.parametrize("dtype,nbox,n", [(torch.float32, 1000, 16), (torch.float64, 256, 16)])
+def test_short_runs_of_many_boxes(dtype, nbox, n):
+    """A run of eight steps takes no longer than eight single steps, also with more boxes than slots."""
+    z = torch.rand((1, n, n), device="cuda", dtype=dtype)
+    b = cdi.Batch([dict(dx=0.02, dt=1e-6, eps=0.02, gamma=1.0, u=z, v=z, w=z, phi_a=z.clone(), phi_b=z.clone())
+                   for _ in range(nbox)])
+    b.set_launch(4, 0)
+
+    def timed(f):
+        f()
+        best = float("inf")
+        for _ in range(5):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            e0.record()
+            f()
+            e1.record()
+            e1.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        return best
+
+    assert timed(lambda: b.run(8)) <= timed(lambda: [b.step(1.0) for _ in range(8)])
