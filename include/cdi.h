@@ -501,8 +501,10 @@ CDI_API int cdi_get_run_depth(const cdi_grid *g, int *depth, int *nblocks, int *
  * overwritten) with CUDA events on the stream (one warm-up + reps launches
  * each) and keep the fastest for cdi_step; then time the two-steps-per-pass
  * kernel (where it applies) and set the run depth of cdi_run to 2 if it is
- * faster per step than that, else to 1.  *best_ms (may be NULL) gets the time
- * per step of what cdi_run will use.  Synchronises the stream. */
+ * faster per step than that, else to 1; then, on a 2D grid whose state fits in
+ * shared memory, runs held there (cdi_run), which cdi_run uses (at depth 1) if they
+ * are faster per step than either.  *best_ms (may be NULL) gets the time per step of
+ * what cdi_run will use.  Synchronises the stream. */
 CDI_API int cdi_autotune(cdi_grid *g, void *phi_a, void *phi_b, double dt, double eps,
                          double gamma, int reps, double *best_ms, void *stream);
 

@@ -2,6 +2,7 @@
 the same buffers, extrema and counts as one launch per step on the one-cell-per-thread tile, bit
 for bit (the sums to rounding), for one band (no neighbour), bands of two rows and of uneven
 heights, odd rows, every buffer parity, runs of several launches and time-dependent velocities."""
+import ctypes
 import os
 import subprocess
 import sys
@@ -236,3 +237,36 @@ def test_short_runs_of_many_boxes(dtype, nbox, n):
         return best
 
     assert timed(lambda: b.run(8)) <= timed(lambda: [b.step(1.0) for _ in range(8)])
+
+
+def nodes(call):
+    """Number of nodes that ``call`` captures."""
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g, capture_error_mode="thread_local"):
+        call()
+    n = ctypes.c_size_t(0)
+    assert ctypes.CDLL("libcuda.so.1").cuGraphGetNodes(ctypes.c_void_p(g.raw_cuda_graph()), None, ctypes.byref(n)) == 0
+    return n.value
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("n", [64, 128, 300])
+def test_autotune_times_the_run_on_chip(dtype, n):
+    """The autotuner's choice for a run is the fastest it timed: one launch for all steps, at depth 1,
+    its time per step that of the run."""
+    g, phi, prm = setup(n, n, dtype, 3)
+    phi.clamp_(0, 1)
+    a, b = phi.clone(), torch.empty_like(phi)
+    ms = g.autotune(a, b, *prm, reps=3)
+    assert g.get_run_depth()["depth"] == 1
+    assert nodes(lambda: g.run(a, b, 32, *prm)) == 1
+    best = float("inf")
+    for _ in range(5):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda.synchronize()
+        e0.record()
+        g.run(a, b, 33, *prm)
+        e1.record()
+        e1.synchronize()
+        best = min(best, e0.elapsed_time(e1) / 33)
+    assert 0.5 * best <= ms <= 1.5 * best
