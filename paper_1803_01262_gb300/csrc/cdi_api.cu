@@ -1478,6 +1478,7 @@ int cdi_set_sharpening(cdi_grid *g, int mode)
     }
     g->fwd = c;
     g->fwd_dflt = true;
+    g->plane_on = g->plane_bands > 0;  // (runs on chip take the centre form only)
     g->rk.nblocks = 0;
     if (mode != CDI_SHARPEN_CENTRE) g->run_depth = 1;  // two steps per pass: centre form only
     return CDI_OK;

@@ -270,3 +270,16 @@ def test_autotune_times_the_run_on_chip(dtype, n):
         e1.synchronize()
         best = min(best, e0.elapsed_time(e1) / 33)
     assert 0.5 * best <= ms <= 1.5 * best
+
+
+def test_setting_the_sharpening_restores_the_default_run():
+    g, phi, prm = setup(64, 64, torch.float32, 4)
+    a, b = phi.clone(), torch.empty_like(phi)
+    run = lambda: g.run(a, b, 8, *prm)
+    assert nodes(run) == 1
+    g.set_launch(cdi.CDI_KERNEL_FORWARD, 0)
+    assert nodes(run) == 8
+    g.set_sharpening("face")
+    assert nodes(run) == 8
+    g.set_sharpening("centre")
+    assert nodes(run) == 1
