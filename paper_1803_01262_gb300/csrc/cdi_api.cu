@@ -637,13 +637,12 @@ template <typename T>
 static int plane_run_t(cdi_grid *g, void *buf_a, void *buf_b, int nsteps, double t0, double dt, double eps,
                        double gamma, double period, cudaStream_t s)
 {
-    cdi::FwdArgs<T> a = {};
+    cdi::PlaneArgs<T> a = {};
     a.u = (const T *)g->u;
     a.v = (const T *)(g->v ? g->v : g->u);
-    a.w = a.u;
-    a.nx = g->nx; a.ny = g->ny; a.nz = g->nz;
+    a.nx = g->nx; a.ny = g->ny;
     a.c = coefs<T>(g, dt, eps, gamma, 1.0);
-    a.red = scratch(g, g->rec, 1);
+    const RedScratch red = scratch(g, g->rec, 1);
     const int launches = (nsteps + cdi::kPlaneSteps - 1) / cdi::kPlaneSteps;
     void *src = buf_a, *dst = buf_b;  // the state, the other buffer
     int i0 = 0;
@@ -663,8 +662,8 @@ static int plane_run_t(cdi_grid *g, void *buf_a, void *buf_b, int nsteps, double
             a.out = (T *)src;
         }
         T *const prev = n == 1 ? nullptr : (T *)((n & 1) ? src : dst);
-        cudaError_t e = cdi::launch_fwd_plane<T>(a, prev, n, ca, g->plane_bands, g->plane_smem, g->plane_words,
-                                                 g->plane_tag, s);
+        cudaError_t e = cdi::launch_fwd_plane<T>(a, red, prev, n, ca, g->plane_bands, g->plane_smem,
+                                                 g->plane_words, g->plane_tag, s);
         if (e == cudaErrorCooperativeLaunchTooLarge && l == 0) {
             (void)cudaGetLastError();
             g->plane_on = false;

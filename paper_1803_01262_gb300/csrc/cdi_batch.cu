@@ -285,6 +285,12 @@ batch_kernel(const BoxDev<T> *__restrict__ boxes, const int *__restrict__ unit_b
     }
 }
 
+template <typename T>
+__device__ __forceinline__ PlaneArgs<T> plane_args(const FwdArgs<T> &a)
+{
+    return {a.phi, a.out, a.u, a.v, a.nx, a.ny, a.c};
+}
+
 // A run of a batch of 2D boxes, each held in shared memory while it is stepped (plane_steps,
 // cdi_plane.cuh): one launch for the whole run.  A step per launch left a third of the FP64 pipe
 // idle (two boxes on 104 of 152 SMs, the loads, reductions and waits of every step): 256 boxes of
@@ -319,7 +325,7 @@ plane_batch_kernel(const BoxDev<T> *__restrict__ boxes, const int *__restrict__ 
         }
         // the last state goes to the buffer of the run's final parity, the one before it to the
         // other, as single steps leave them; between units the state waits in the former
-        FwdArgs<T> a = boxes[bi].a;
+        PlaneArgs<T> a = plane_args(boxes[bi].a);
         T *const buf[2] = {const_cast<T *>(a.phi), a.out};
         const int fp = parity ^ (n & 1), s0 = (int)((long long)c * n / nchunks);
         const int steps = (int)((long long)(c + 1) * n / nchunks) - s0;
@@ -384,7 +390,7 @@ plane_bands_kernel(const BoxDev<T> *__restrict__ boxes, const int nb, const int 
     __shared__ int is_last;
     const int tid = threadIdx.x, bi = blockIdx.x / nb, band = blockIdx.x - bi * nb;
     const unsigned base = *tag;  // (moved on by the last block of the launch, below)
-    FwdArgs<T> a = boxes[bi].a;
+    PlaneArgs<T> a = plane_args(boxes[bi].a);
     const int B = min(nb, a.ny / 2);
     if (band < B) {
         T *const buf[2] = {const_cast<T *>(a.phi), a.out};
@@ -395,7 +401,7 @@ plane_bands_kernel(const BoxDev<T> *__restrict__ boxes, const int nb, const int 
         run.init();
         last.init();
         const int yb = (int)((long long)band * a.ny / B), R = (int)((long long)(band + 1) * a.ny / B) - yb;
-        const PlaneHalo h = {words + bi * word_stride, B, band, base, wait_ns, a.red.status};
+        const PlaneHalo h = {words + bi * word_stride, B, band, base, wait_ns, boxes[bi].a.red.status};
         const T c_adv = a.c.c_adv;
         plane_steps<T, NT, FACE, true>(a, keep_prev && n > 1 ? buf[fp ^ 1] : nullptr, yb, R, n,
                                        [&](int) { return c_adv; }, h, run, last, reinterpret_cast<T *>(smem_raw));

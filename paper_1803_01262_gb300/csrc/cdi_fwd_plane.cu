@@ -18,7 +18,7 @@ struct PlaneCoefs {
 
 template <typename T, int NT, bool MULTI>
 __global__ void __launch_bounds__(NT)
-fwd_plane_kernel(const FwdArgs<T> a, T *prev, const int n, const __grid_constant__ PlaneCoefs<T> cs,
+fwd_plane_kernel(const PlaneArgs<T> a, const RedScratch red, T *prev, const int n, const __grid_constant__ PlaneCoefs<T> cs,
                  unsigned long long *words, unsigned *tag, const unsigned long long wait_ns)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -29,11 +29,10 @@ fwd_plane_kernel(const FwdArgs<T> a, T *prev, const int n, const __grid_constant
     Acc<T> run, last;
     run.init();
     last.init();
-    const PlaneHalo h = {words, B, b, base, wait_ns, a.red.status};
+    const PlaneHalo h = {words, B, b, base, wait_ns, red.status};
     plane_steps<T, NT, false, MULTI>(a, prev, yb, R, n, [&](int s) { return cs.c_adv[s]; }, h, run, last,
                                      reinterpret_cast<T *>(smem_raw));
     // the last step's statistics into the record, every step's bounds into the run's
-    const RedScratch &red = a.red;
     const Partial pl = block_partial(last), pr = block_partial(run);
     if (tid == 0) {
         red.partials[b] = pl;
@@ -122,8 +121,8 @@ size_t plane_word_bytes(int nx, int bands)
 }
 
 template <typename T>
-cudaError_t launch_fwd_plane(const FwdArgs<T> &a, T *prev, int n, const T *c_adv, int bands, size_t smem,
-                             unsigned long long *words, unsigned *tag, cudaStream_t s)
+cudaError_t launch_fwd_plane(const PlaneArgs<T> &a, const RedScratch &red, T *prev, int n, const T *c_adv, int bands,
+                             size_t smem, unsigned long long *words, unsigned *tag, cudaStream_t s)
 {
     PlaneCoefs<T> cs;
     for (int i = 0; i < n; ++i) cs.c_adv[i] = c_adv[i];
@@ -139,17 +138,18 @@ cudaError_t launch_fwd_plane(const FwdArgs<T> &a, T *prev, int n, const T *c_adv
     cfg.numAttrs = bands > 1 ? 1 : 0;
     const unsigned long long wait_ns = 1000000000ull;  // a step takes microseconds
     if (bands > 1)
-        return cudaLaunchKernelEx(&cfg, fwd_plane_kernel<T, kPlaneNT, true>, a, prev, n, cs, words, tag, wait_ns);
-    return cudaLaunchKernelEx(&cfg, fwd_plane_kernel<T, kPlaneNT, false>, a, prev, n, cs, words, tag, wait_ns);
+        return cudaLaunchKernelEx(&cfg, fwd_plane_kernel<T, kPlaneNT, true>, a, red, prev, n, cs, words, tag, wait_ns);
+    return cudaLaunchKernelEx(&cfg, fwd_plane_kernel<T, kPlaneNT, false>, a, red, prev, n, cs, words, tag, wait_ns);
 }
 
 template cudaError_t plane_bands<float>(int, int, int, int *, size_t *);
 template cudaError_t plane_bands<double>(int, int, int, int *, size_t *);
 template size_t plane_word_bytes<float>(int, int);
 template size_t plane_word_bytes<double>(int, int);
-template cudaError_t launch_fwd_plane<float>(const FwdArgs<float> &, float *, int, const float *, int, size_t,
-                                             unsigned long long *, unsigned *, cudaStream_t);
-template cudaError_t launch_fwd_plane<double>(const FwdArgs<double> &, double *, int, const double *, int, size_t,
-                                              unsigned long long *, unsigned *, cudaStream_t);
+template cudaError_t launch_fwd_plane<float>(const PlaneArgs<float> &, const RedScratch &, float *, int, const float *,
+                                             int, size_t, unsigned long long *, unsigned *, cudaStream_t);
+template cudaError_t launch_fwd_plane<double>(const PlaneArgs<double> &, const RedScratch &, double *, int,
+                                              const double *, int, size_t, unsigned long long *, unsigned *,
+                                              cudaStream_t);
 
 }  // namespace cdi

@@ -140,13 +140,23 @@ cudaError_t launch_fwd_tma(const FwdArgs<T> &a, int nblocks, int nchunks, cudaSt
 // `bands` blocks that wait on one another (plane_bands: 0 where the box does not fit), halo words
 // (plane_word_bytes, zeroed) and a tag counter of the grid (starting at 1).
 constexpr int kPlaneSteps = 512;
+// The box of such a run.  phi and out may be one array (an even number of steps ends where it began;
+// every read of phi comes before the first write), so unlike FwdArgs' they are not restrict.
+template <typename T>
+struct PlaneArgs {
+    const T *phi;
+    T *out;
+    const T *u, *v;
+    int nx, ny;
+    StepCoef<T> c;
+};
 template <typename T>
 cudaError_t plane_bands(int nx, int ny, int sms, int *bands, size_t *smem);
 template <typename T>
 size_t plane_word_bytes(int nx, int bands);
 template <typename T>
-cudaError_t launch_fwd_plane(const FwdArgs<T> &a, T *prev, int n, const T *c_adv, int bands, size_t smem,
-                             unsigned long long *words, unsigned *tag, cudaStream_t s);
+cudaError_t launch_fwd_plane(const PlaneArgs<T> &a, const RedScratch &red, T *prev, int n, const T *c_adv, int bands,
+                             size_t smem, unsigned long long *words, unsigned *tag, cudaStream_t s);
 
 // rk selects the Runge-Kutta stage variant (tiles with fwd_tile_has_rk only);
 // face the face-product sharpening (tile 0, Euler only); chained: the launch before it on the

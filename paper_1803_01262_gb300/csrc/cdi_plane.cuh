@@ -110,7 +110,7 @@ __device__ __forceinline__ double halo_get(const unsigned long long *w, unsigned
 // step before the last; with n == 1, phi itself).  c_adv(s): the advective coefficient of step s.
 // run collects the bounds of every step, last the statistics of the last one.
 template <typename T, int NT, bool FACE, bool MULTI, typename CA>
-__device__ __forceinline__ void plane_steps(const FwdArgs<T> &a, T *prev, int yb, int R, int n, CA c_adv_of,
+__device__ __forceinline__ void plane_steps(const PlaneArgs<T> &a, T *prev, int yb, int R, int n, CA c_adv_of,
                                             const PlaneHalo &h, Acc<T> &run, Acc<T> &last, T *sm)
 {
     constexpr int HL = MULTI ? 2 : 0, RL = MULTI ? 1 : 0;  // halo rows of phi, ring rows of s_y
