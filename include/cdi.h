@@ -410,7 +410,9 @@ CDI_API int cdi_get_sharpening(const cdi_grid *g, int *mode);
  * wait must run out after limit_s seconds (0 < limit_s <= 2), record the time-
  * out in the grid's status word and let the kernel end; the call then reads
  * and clears that word and returns CDI_ERR_TIMEOUT -- the expected result.
- * CDI_OK would mean a time-out went unreported.  Synchronises the stream. */
+ * CDI_OK would mean a time-out went unreported.  A 2D grid whose runs are held
+ * on chip in several bands: then the same for a band's wait for a halo that no
+ * neighbour writes.  Synchronises the stream. */
 CDI_API int cdi_probe_bounded_wait(cdi_grid *g, double limit_s, void *stream);
 
 /* Checked builds.  A library compiled with -DCDI_CHECKED (build.py

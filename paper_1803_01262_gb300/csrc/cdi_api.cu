@@ -80,7 +80,7 @@ struct cdi_grid {
     bool plane_on;
     size_t plane_smem;
     unsigned long long *plane_words;
-    unsigned *plane_tag;
+    unsigned *plane_tag;  // [2]
     int sharpen;   // CDI_SHARPEN_CENTRE (Section 2.2) or CDI_SHARPEN_FACE
     // staging for cdi_step_host (owned, allocated on first use), and the copy
     // streams and events of its slab pipeline (created on first use)
@@ -305,12 +305,12 @@ static int plane_setup(cdi_grid *g)
     if (g->plane_bands == 0) return CDI_OK;
     const size_t bytes = g->dtype == CDI_F64 ? cdi::plane_word_bytes<double>(g->nx, g->plane_bands)
                                              : cdi::plane_word_bytes<float>(g->nx, g->plane_bands);
-    const unsigned one = 1u;
-    if ((e = cudaMalloc(&g->plane_words, bytes + sizeof(unsigned))) != cudaSuccess ||
+    const unsigned tag[2] = {1u, 0u};
+    if ((e = cudaMalloc(&g->plane_words, bytes + sizeof(tag))) != cudaSuccess ||
         (e = cudaMemset(g->plane_words, 0, bytes)) != cudaSuccess)
         return cuda_fail(e, "halo words");
-    g->plane_tag = (unsigned *)((char *)g->plane_words + bytes);  // the tag counter, after the words
-    if ((e = cudaMemcpy(g->plane_tag, &one, sizeof(one), cudaMemcpyHostToDevice)) != cudaSuccess)
+    g->plane_tag = (unsigned *)((char *)g->plane_words + bytes);  // after the words
+    if ((e = cudaMemcpy(g->plane_tag, tag, sizeof(tag), cudaMemcpyHostToDevice)) != cudaSuccess)
         return cuda_fail(e, "halo words");
     g->plane_on = true;
     return CDI_OK;
@@ -1356,13 +1356,8 @@ __global__ void probe_wait_kernel(unsigned int *status, unsigned long long limit
     __syncthreads();
 }
 
-int cdi_probe_bounded_wait(cdi_grid *g, double limit_s, void *stream)
+static int probe_result(cdi_grid *g, cudaError_t e, cudaStream_t s)
 {
-    if (int rc = check_grid(g)) return rc;
-    if (!(limit_s > 0.0 && limit_s <= 2.0)) return fail(CDI_ERR_ARG, "limit_s must be in (0, 2]");
-    cudaStream_t s = (cudaStream_t)stream;
-    probe_wait_kernel<<<1, 32, 0, s>>>(g->status, (unsigned long long)(limit_s * 1e9));
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "probe launch");
     unsigned int st = 0;
     if ((e = cudaMemcpyAsync(&st, g->status, sizeof(st), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||
@@ -1372,6 +1367,18 @@ int cdi_probe_bounded_wait(cdi_grid *g, double limit_s, void *stream)
     cudaMemsetAsync(g->status, 0, sizeof(unsigned int) * cdi::kStatusWords, s);
     if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_fail(e, "probe status reset");
     return fail(CDI_ERR_TIMEOUT, "bounded device wait ran out (probe)");
+}
+
+int cdi_probe_bounded_wait(cdi_grid *g, double limit_s, void *stream)
+{
+    if (int rc = check_grid(g)) return rc;
+    if (!(limit_s > 0.0 && limit_s <= 2.0)) return fail(CDI_ERR_ARG, "limit_s must be in (0, 2]");
+    cudaStream_t s = (cudaStream_t)stream;
+    const unsigned long long limit_ns = (unsigned long long)(limit_s * 1e9);
+    probe_wait_kernel<<<1, 32, 0, s>>>(g->status, limit_ns);
+    const int rc = probe_result(g, cudaGetLastError(), s);
+    if (rc != CDI_ERR_TIMEOUT || g->plane_bands < 2) return rc;
+    return probe_result(g, cdi::launch_halo_probe(g->plane_words, g->plane_tag, g->status, limit_ns, s), s);
 }
 
 // FP64 FMA throughput: every thread runs CHAINS independent fused multiply-add

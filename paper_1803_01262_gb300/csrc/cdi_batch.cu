@@ -401,7 +401,7 @@ plane_bands_kernel(const BoxDev<T> *__restrict__ boxes, const int nb, const int 
         run.init();
         last.init();
         const int yb = (int)((long long)band * a.ny / B), R = (int)((long long)(band + 1) * a.ny / B) - yb;
-        const PlaneHalo h = {words + bi * word_stride, B, band, base, wait_ns, boxes[bi].a.red.status};
+        const PlaneHalo h = {words + bi * word_stride, B, band, base, wait_ns, boxes[bi].a.red.status, tag + 1};
         const T c_adv = a.c.c_adv;
         plane_steps<T, NT, FACE, true>(a, keep_prev && n > 1 ? buf[fp ^ 1] : nullptr, yb, R, n,
                                        [&](int) { return c_adv; }, h, run, last, reinterpret_cast<T *>(smem_raw));
@@ -502,7 +502,8 @@ struct cdi_batch {
     bool flat;                 // every box has nz == 1: the single-plane kernel
     size_t plane_bytes;        // shared memory of the whole-plane body: 3 nx ny values of the largest box
     size_t plane_run_bytes;    // ... of a run held there (4 nx ny values; 0: it does not fit)
-    unsigned int *plane_sync;  // [2 + nbox] its hand-out counters and the boxes' epochs, [+ 1] halo tag
+    unsigned int *plane_sync;  // [2 + nbox] its hand-out counters and the boxes' epochs, [+ 2] halo tag
+                               // and the tag of the last launch in which a halo wait gave up
     int plane_nb;              // bands per box of a run of few boxes (0: whole boxes)
     size_t plane_band_bytes, plane_word_stride;
     unsigned long long *plane_words;  // [nbox][plane_word_stride] halo words
@@ -1168,16 +1169,16 @@ int cdi_batch_create(cdi_batch **out, const cdi_box_desc *boxes, int nbox, int d
     b->vband_bytes = vband_bytes(b);
     cudaError_t e;
     int dev = 0;
-    const unsigned int one = 1u;
+    const unsigned int tag[2] = {1u, 0u};
     std::vector<StatsRec> hrec(nbox);
     reset_recs(hrec);
     if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
         (e = cudaMalloc(&b->box_done, sizeof(unsigned int) * nbox)) != cudaSuccess ||
         (e = cudaMalloc(&b->queue, sizeof(unsigned int) * 2)) != cudaSuccess ||
-        (e = cudaMalloc(&b->plane_sync, sizeof(unsigned int) * (3 + (size_t)nbox))) != cudaSuccess ||
+        (e = cudaMalloc(&b->plane_sync, sizeof(unsigned int) * (4 + (size_t)nbox))) != cudaSuccess ||
         (e = cudaMemset(b->plane_sync, 0, sizeof(unsigned int) * (2 + (size_t)nbox))) != cudaSuccess ||
-        (e = cudaMemcpy(b->plane_sync + 2 + nbox, &one, sizeof(one), cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(b->plane_sync + 2 + nbox, tag, sizeof(tag), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemset(b->queue, 0, sizeof(unsigned int) * 2)) != cudaSuccess ||
         (e = cudaMalloc(&b->epoch, sizeof(unsigned int) * nbox)) != cudaSuccess ||
         (e = cudaMemset(b->epoch, 0, sizeof(unsigned int) * nbox)) != cudaSuccess ||

@@ -29,7 +29,7 @@ fwd_plane_kernel(const PlaneArgs<T> a, const RedScratch red, T *prev, const int 
     Acc<T> run, last;
     run.init();
     last.init();
-    const PlaneHalo h = {words, B, b, base, wait_ns, red.status};
+    const PlaneHalo h = {words, B, b, base, wait_ns, red.status, tag + 1};
     plane_steps<T, NT, false, MULTI>(a, prev, yb, R, n, [&](int s) { return cs.c_adv[s]; }, h, run, last,
                                      reinterpret_cast<T *>(smem_raw));
     // the last step's statistics into the record, every step's bounds into the run's
@@ -69,6 +69,24 @@ fwd_plane_kernel(const PlaneArgs<T> a, const RedScratch red, T *prev, const int 
         *red.counter = 0u;
         *tag = base + (unsigned)n;
     }
+}
+
+// A wait for words that no block writes: it must run out after wait_ns.  The tag moves on, as after a run.
+__global__ void halo_probe_kernel(const unsigned long long *words, unsigned *tag, unsigned *status,
+                                  const unsigned long long wait_ns)
+{
+    const PlaneHalo h = {nullptr, 1, 0, *tag, wait_ns, status, tag + 1};
+    bool ok = true;
+    (void)halo_word(words, h.tag + 0x40000000u, h, ok);
+    __syncthreads();
+    if (threadIdx.x == 0) *tag = h.tag + 1u;
+}
+
+cudaError_t launch_halo_probe(const unsigned long long *words, unsigned *tag, unsigned *status,
+                              unsigned long long wait_ns, cudaStream_t s)
+{
+    halo_probe_kernel<<<1, 32, 0, s>>>(words, tag, status, wait_ns);
+    return cudaGetLastError();
 }
 
 // 512 threads per band (256: 1.75, 1024: 1.77 against 1.60 us per step at 128^2 FP32).

@@ -138,7 +138,8 @@ cudaError_t launch_fwd_tma(const FwdArgs<T> &a, int nblocks, int nchunks, cudaSt
 
 // Runs of a 2D grid in shared memory (cdi_fwd_plane.cu): at most kPlaneSteps steps per launch,
 // `bands` blocks that wait on one another (plane_bands: 0 where the box does not fit), halo words
-// (plane_word_bytes, zeroed) and a tag counter of the grid (starting at 1).
+// (plane_word_bytes, zeroed) and tag[2] of the grid: a counter (starting at 1), and the tag of the
+// last launch in which a wait gave up (0: none).
 constexpr int kPlaneSteps = 512;
 // The box of such a run.  phi and out may be one array (an even number of steps ends where it began;
 // every read of phi comes before the first write), so unlike FwdArgs' they are not restrict.
@@ -157,6 +158,10 @@ size_t plane_word_bytes(int nx, int bands);
 template <typename T>
 cudaError_t launch_fwd_plane(const PlaneArgs<T> &a, const RedScratch &red, T *prev, int n, const T *c_adv, int bands,
                              size_t smem, unsigned long long *words, unsigned *tag, cudaStream_t s);
+
+// One block that waits, at most wait_ns, for halo words that nothing writes.
+cudaError_t launch_halo_probe(const unsigned long long *words, unsigned *tag, unsigned *status,
+                              unsigned long long wait_ns, cudaStream_t s);
 
 // rk selects the Runge-Kutta stage variant (tiles with fwd_tile_has_rk only);
 // face the face-product sharpening (tile 0, Euler only); chained: the launch before it on the

@@ -61,6 +61,7 @@ struct PlaneHalo {
     unsigned tag;               // tag of this launch's first exchanged step
     unsigned long long wait_ns;
     unsigned *status;
+    unsigned *gave_up;          // tag of the last launch in which a wait gave up
 };
 
 __device__ __forceinline__ void halo_put(unsigned long long *w, unsigned tag, float v)
@@ -75,8 +76,9 @@ __device__ __forceinline__ void halo_put(unsigned long long *w, unsigned tag, do
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(w + 1), "l"(t | (b >> 32)) : "memory");
 }
 
-// Wait for the word with this tag, for at most limit_ns (read from the global timer every few
-// polls); gives up at once if a wait of the grid has (status bit 0), else records that bit.
+// Wait for the word with this tag, for at most h.wait_ns (read from the global timer every few
+// polls); gives up at once if a wait of this launch has, else records that and status bit 0 (which
+// stays set until the host reads it: a later launch waits for its own words all the same).
 __device__ __forceinline__ unsigned halo_word(const unsigned long long *w, unsigned tag, const PlaneHalo &h, bool &ok)
 {
     unsigned long long v, t0 = 0;
@@ -85,11 +87,14 @@ __device__ __forceinline__ unsigned halo_word(const unsigned long long *w, unsig
         if ((unsigned)(v >> 32) == tag || !ok) return (unsigned)v;
         if ((i & 63u) == 63u) {
             const unsigned long long t = global_ns();
-            unsigned st;
-            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(st) : "l"(h.status) : "memory");
+            unsigned gu;
+            asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(gu) : "l"(h.gave_up) : "memory");
             if (t0 == 0) t0 = t;
-            if (t - t0 > h.wait_ns || (st & 1u)) {
+            if (t - t0 > h.wait_ns) {
                 atomicOr(h.status, 1u);
+                atomicExch(h.gave_up, h.tag);
+                ok = false;
+            } else if (gu == h.tag) {
                 ok = false;
             }
         }

@@ -6,6 +6,7 @@ import ctypes
 import os
 import subprocess
 import sys
+import time
 
 import pytest
 import torch
@@ -283,3 +284,19 @@ def test_setting_the_sharpening_restores_the_default_run():
     assert nodes(run) == 8
     g.set_sharpening("centre")
     assert nodes(run) == 1
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+def test_halo_wait_is_bounded_and_the_grid_stays_usable(dtype):
+    """A wait for a halo that nobody writes ends at its limit and is reported; the next run waits for
+    its own halos and equals tile 0's."""
+    g, phi, prm = setup(96, 70, dtype, 6)
+    ref = ran(g, phi, 12, prm, 0)
+    ran(g, phi, 5, prm, -1)
+    t0 = time.perf_counter()
+    with pytest.raises(cdi.CDIError) as e:
+        g.probe_bounded_wait(0.05)
+    assert e.value.code == cdi.CDI_ERR_TIMEOUT and 0.1 <= time.perf_counter() - t0 < 5.0   # both waits
+    out = ran(g, phi, 12, prm, -1)
+    assert torch.equal(out[0], ref[0]) and torch.equal(out[1], ref[1])
+    assert all(out[2][k] == ref[2][k] for k in ref[2] if k not in ("mass", "sum"))
