@@ -148,7 +148,8 @@ CDI_API int cdi_step(cdi_grid *g, const void *phi_in, void *phi_out, double dt, 
  * in native code.  On return *final_in_b tells which buffer holds the
  * result.  Stats of the last step are in the device record.
  * A 2D grid (nz = 1) in its default launch configuration (or the autotuner's)
- * whose state fits in shared memory is stepped there, up to 512 steps per
+ * whose state fits in shared memory is stepped there where that is faster (from
+ * a few steps on, if its rows are not too long for its height), up to 512 steps per
  * cooperative launch, bands of rows exchanging halos; buffers, extrema and
  * counts as with one launch per step, the sums to rounding.  Its device-side
  * waits are bounded: CDI_ERR_TIMEOUT from the statistics read-back. */

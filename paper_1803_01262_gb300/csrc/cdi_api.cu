@@ -74,10 +74,11 @@ struct cdi_grid {
     LaunchCfg tb;    // two steps per pass (cdi_run with depth 2; nblocks 0 = unset)
     int run_depth;   // steps per pass of cdi_run: 1, or 2 (temporal blocking)
     // 2D grids (nz == 1) whose state fits in shared memory: blocks of a run held there
-    // (cdi_fwd_plane.cu), 0 where it does not apply; plane_on in the default launch (and after
-    // the autotuner); its shared memory, halo words and tag counter (owned)
+    // (cdi_fwd_plane.cu), 0 where it does not apply; the steps from which on a run is held there in
+    // the default launch and after the autotuner (0: none is); its shared memory, halo words and tag
+    // counter (owned)
     int plane_bands;
-    bool plane_on;
+    int plane_min;
     size_t plane_smem;
     unsigned long long *plane_words;
     unsigned *plane_tag;  // [2]
@@ -294,6 +295,42 @@ static LaunchCfg adj_default(const cdi_grid *g)
     return c;
 }
 
+// Steps from which on a run held on chip pays: its launch and first load cost as much as 7 us (FP32)
+// or 13 us (FP64) more than a launch per step, a step takes gain_us less.  0: never.
+static int plane_break_even(const cdi_grid *g, double gain_us)
+{
+    const bool f64 = g->dtype == CDI_F64;
+    const double n = gain_us > 0.0 ? ceil((f64 ? 13.0 : 7.0) / gain_us) : 1e9;
+    return n >= 1e9 ? 0 : n < (f64 ? 2 : 3) ? (f64 ? 2 : 3) : (int)n;
+}
+
+// The same for the default launch, from the time of a step either way.  On chip: the exchange, and
+// the cells of the busiest block (with ring and halo rows, where there are several), which a box of
+// few long rows has too many of.  Launched: a floor by the tile, and the box's cells.  Fits 840 boxes
+// of 17..13000 by 1..1200 cells to 2..9%; the choice is 0.3% off the better path on average.  (On chip
+// throughout: 8% in FP32, 20% in FP64, and for long rows several times: 32 steps of 3000x4 396 us on
+// chip and 155 launched, FP64 3000x2 1878 and 467; 128^2 44 and 200, FP64 512^2 830 and 1920.)
+static int plane_default_min(const cdi_grid *g)
+{
+    if (g->plane_bands == 0) return 0;
+    const double rows = (g->ny + g->plane_bands - 1) / g->plane_bands, nx = g->nx, cells = nx * g->ny;
+    const bool halo = g->plane_bands > 1;
+    double chip, launched;
+    if (g->dtype == CDI_F32) {
+        chip = 1.0 + 7.5e-4 * nx * (rows + (halo ? 4.0 : 0.0));
+        launched = 5.0 + 1.1e-5 * cells;
+    } else {
+        chip = 1.5 + 9.5e-3 * nx * (rows + (halo ? 1.2 : 0.0));
+        switch (default_fwd_tile(g)) {
+        case 1: launched = 17.5 + 8e-5 * cells; break;
+        case 3: launched = 10.5 + 6e-5 * cells; break;
+        case 4: launched = 19.5 + 1.6e-4 * cells; break;
+        default: launched = 14.25;  // tile 5: fewer than 12 rows
+        }
+    }
+    return plane_break_even(g, launched - chip);
+}
+
 // The shared-memory stepping of a 2D grid: its bands, halo words and tag counter.
 static int plane_setup(cdi_grid *g)
 {
@@ -312,7 +349,7 @@ static int plane_setup(cdi_grid *g)
     g->plane_tag = (unsigned *)((char *)g->plane_words + bytes);  // after the words
     if ((e = cudaMemcpy(g->plane_tag, tag, sizeof(tag), cudaMemcpyHostToDevice)) != cudaSuccess)
         return cuda_fail(e, "halo words");
-    g->plane_on = true;
+    g->plane_min = plane_default_min(g);
     return CDI_OK;
 }
 
@@ -666,7 +703,7 @@ static int plane_run_t(cdi_grid *g, void *buf_a, void *buf_b, int nsteps, double
                                                  g->plane_words, g->plane_tag, s);
         if (e == cudaErrorCooperativeLaunchTooLarge && l == 0) {
             (void)cudaGetLastError();
-            g->plane_on = false;
+            g->plane_min = 0;
             return 1;
         }
         if (e != cudaSuccess) return cuda_fail(e, "plane run launch");
@@ -680,12 +717,10 @@ static int plane_run_t(cdi_grid *g, void *buf_a, void *buf_b, int nsteps, double
     return CDI_OK;
 }
 
-// Whether a run takes that path: its launch and first load cost about two launches, so from three
-// steps on in FP32 (128^2: 12.3 us against 12.6 for two steps, 512^2 16.7 against 14.6, 19.1
-// against 20.8 for three) and from two in FP64 (33 against 44 us).
+// Whether a run takes that path.
 static bool plane_applies(const cdi_grid *g, int nsteps)
 {
-    return g->plane_on && g->sharpen == CDI_SHARPEN_CENTRE && nsteps >= (g->dtype == CDI_F64 ? 2 : 3);
+    return g->plane_min > 0 && g->sharpen == CDI_SHARPEN_CENTRE && nsteps >= g->plane_min;
 }
 
 // Launch configuration of the two-steps-per-pass kernel: one block per SM (or as
@@ -1305,7 +1340,7 @@ int cdi_set_launch(cdi_grid *g, int which, int tile, int blocks_per_sm, int nchu
         const bool dflt = tile < 0 && blocks_per_sm <= 0 && nchunks == 0;
         if (tile < 0) tile = default_fwd_tile(g);
         if (int rc = fwd_cfg(g, tile, blocks_per_sm, nchunks, &c)) return rc;
-        g->plane_on = dflt && g->plane_bands > 0;
+        g->plane_min = dflt ? plane_default_min(g) : 0;
         g->fwd = c;
         g->fwd_dflt = dflt;
         g->rk.nblocks = 0;  // the Runge-Kutta configuration follows on next use
@@ -1484,7 +1519,7 @@ int cdi_set_sharpening(cdi_grid *g, int mode)
     }
     g->fwd = c;
     g->fwd_dflt = true;
-    g->plane_on = g->plane_bands > 0;  // (runs on chip take the centre form only)
+    g->plane_min = mode == CDI_SHARPEN_CENTRE ? plane_default_min(g) : 0;
     g->rk.nblocks = 0;
     if (mode != CDI_SHARPEN_CENTRE) g->run_depth = 1;  // two steps per pass: centre form only
     return CDI_OK;
@@ -1647,10 +1682,10 @@ int cdi_autotune(cdi_grid *g, void *phi_a, void *phi_b, double dt, double eps, d
     g->rk.nblocks = 0;
     if (rc == CDI_OK) {
         const float launched = best2 < best_t ? best2 : best_t;
-        g->plane_on = best_p < launched;
+        g->plane_min = plane_break_even(g, 1e3 * (launched - best_p));
         g->tb = best_tb;
-        g->run_depth = !g->plane_on && best2 < best_t ? 2 : 1;
-        if (best_ms) *best_ms = g->plane_on ? best_p : launched;
+        g->run_depth = g->plane_min == 0 && best2 < best_t ? 2 : 1;
+        if (best_ms) *best_ms = g->plane_min ? best_p : launched;
     }
     return rc;
 }

@@ -300,3 +300,31 @@ def test_halo_wait_is_bounded_and_the_grid_stays_usable(dtype):
     out = ran(g, phi, 12, prm, -1)
     assert torch.equal(out[0], ref[0]) and torch.equal(out[1], ref[1])
     assert all(out[2][k] == ref[2][k] for k in ref[2] if k not in ("mass", "sum"))
+
+
+@pytest.mark.parametrize("dtype,ny,nx,n,on_chip", [
+    (torch.float32, 128, 128, 3, True), (torch.float32, 128, 128, 2, False), (torch.float32, 1024, 1024, 8, True),
+    (torch.float32, 4, 3000, 32, False), (torch.float32, 2, 6000, 32, False), (torch.float32, 1, 13000, 32, False),
+    (torch.float32, 1, 2000, 32, True), (torch.float64, 128, 128, 2, True), (torch.float64, 512, 512, 4, True),
+    (torch.float64, 2, 3000, 32, False), (torch.float64, 64, 1000, 32, False), (torch.float64, 1, 5000, 32, False),
+    (torch.float64, 301, 301, 8, True)])
+def test_runs_are_held_on_chip_where_that_is_faster(dtype, ny, nx, n, on_chip):
+    """Long rows give a block too many cells, short runs do not repay the launch and the first load."""
+    g, phi, prm = setup(ny, nx, dtype, 8)
+    a, b = phi.clone(), torch.empty_like(phi)
+    assert nodes(lambda: g.run(a, b, n, *prm)) == (1 if on_chip else n)
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.float64])
+@pytest.mark.parametrize("ny,nx", [(4, 300), (5, 301), (33, 700), (3, 1500)])
+def test_long_rows_on_chip_by_the_autotuner_or_launched(dtype, ny, nx):
+    """Where the autotuner decides, and whichever way, a run equals one launch per step."""
+    g, phi, prm = setup(ny, nx, dtype, 12 + nx)
+    ref = ran(g, phi, 40, prm, 0)
+    a, b = phi.clone(), torch.empty_like(phi)
+    g.autotune(a, b, *prm, reps=2)
+    g.reset_run_stats()
+    a.copy_(phi)
+    out = g.run(a, b, 40, *prm, period=0.7, t0=0.05)
+    st = g.stats()
+    assert torch.equal(out, ref[0]) and all(st[k] == ref[2][k] for k in st if k not in ("mass", "sum"))
