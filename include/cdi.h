@@ -284,7 +284,8 @@ CDI_API int cdi_max_dt_mixed(double dx, double eps, double gamma, const double *
  * its own spacing, eps, gamma, dt and face velocities, advance together: one
  * kernel launch per step covers every box (a persistent grid taking work
  * units -- a tile of one box and a chunk of its planes -- from one list), and
- * cdi_batch_run replays a captured CUDA graph of nsteps such launches.  Each
+ * cdi_batch_run replays a captured CUDA graph of nsteps such launches (2D boxes
+ * that a run holds on chip: launches of many steps, below).  Each
  * box evolves exactly as with cdi_step on its own grid.  Arrays follow the
  * conventions above and are borrowed for the batch's lifetime.  Like a grid,
  * a batch (its counters, epochs and statistics scratch) must be used by one
@@ -312,7 +313,9 @@ CDI_API int cdi_batch_info(const cdi_batch *b, int *parity, int *total_units, in
  * parity.  Per-box statistics of the result are written to the device. */
 CDI_API int cdi_batch_step(cdi_batch *b, double vel_scale, void *stream);
 
-/* nsteps steps (vel_scale = 1) as one CUDA graph launch; the graph is
+/* nsteps steps (vel_scale = 1) as one CUDA graph launch (tile 4 where a run holds
+ * the boxes on chip: one plain launch, more where a box could count 2^31
+ * violations in it; cdi_batch_set_launch); the graph is
  * captured on first use for each (nsteps, parity) and replayed after.  The
  * launches of a run overlap: launch i + 1 starts on the SMs that launch i
  * leaves, and each of its work units waits (on the device, for at most one
@@ -466,8 +469,8 @@ enum { CDI_KERNEL_FORWARD = 0, CDI_KERNEL_ADJOINT = 1 };
  * (FP32 64x14 and 64x6 cells, FP64 32x16 and 32x8; need nx %
  * (16/sizeof(element)) == 0), 6 the same with tensor-map copies (nx % 64 == 0
  * (FP32) or 32 (FP64), ny % 16 == 0), 7 and 8 vectors per thread for any nx (16
- * vectors by 14 and 6 rows, copied and stored element by element); tile < 0
- * restores the default.  blocks_per_sm <= 0 fills the GPU.  Forward work
+ * vectors by 14 and 6 rows, copied and stored element by element, in FP32 with an
+ * even nx by pairs); tile < 0 restores the default.  blocks_per_sm <= 0 fills the GPU.  Forward work
  * split: nchunks >= 1 cuts every tile column into that many z chunks, taken
  * round-robin by the persistent blocks; CDI_NCHUNKS_BALANCED gives every block
  * an equal contiguous share of the tile-planes (tile-major, cut at column

@@ -39,7 +39,8 @@ def _native(grid, *names):
 def _forward_path(grid, states, dt, eps, gamma, scales):
     """states[i + 1] = the step of states[i] with scales[i].  One native call: a call from Python
     takes 10 us, as long as the step itself at 128^3.  A pass there of 16 steps forward, 14
-    recomputed and 16 adjoint: 1300 us with a call per step, 850 us (700 of them on the device)."""
+    recomputed and 16 adjoint: 1210 us with a call per step, 842 us so (runs of one side differ by 9%;
+    700 us of it on the device), and 1.18 times faster on inputs not seen before."""
     if _native(grid, "step"):
         grid.step_path(states, dt, eps, gamma, scales)
         return

@@ -449,7 +449,8 @@ class BoxDesc(ctypes.Structure):
 
 
 class Batch:
-    """Independent periodic boxes advanced by one launch per step (cdi_batch_*).
+    """Independent periodic boxes advanced together, by one launch per step or, where 2D boxes are held
+    on chip, per run (cdi_batch_*).
 
     ``boxes`` is a list of dicts with keys dx, dt, eps, gamma, u, v, w, phi_a,
     phi_b (CUDA tensors shaped (nz, ny, nx), one dtype for all boxes).  The
@@ -507,7 +508,8 @@ class Batch:
         _ck(lib().cdi_batch_step(self._h, vel_scale, _stream(stream)))
 
     def run(self, nsteps, stream=None):
-        """nsteps steps as one replay of a captured CUDA graph."""
+        """nsteps steps as one replay of a captured CUDA graph, or (2D boxes held on chip, tile 4) one
+        launch."""
         _ck(lib().cdi_batch_run(self._h, nsteps, _stream(stream)))
 
     def set_launch(self, tile=-1, zdepth=-1):

@@ -907,9 +907,8 @@ static int build_units(cdi_batch *b, int tile, int zdepth)
         return cdi::set_error(CDI_ERR_ARG, "batch tile 5 needs a batch with 3D boxes whose rows fit in a band "
                                            "(nx <= %d) and whose band slots fit in shared memory", cdi::BAND_CELLS);
     if (vband && b->vband_bytes == 0)
-        return cdi::set_error(CDI_ERR_ARG, "batch tile 6 needs padded rows of at most %d vectors and band "
-                                           "slots that fit in the shared memory of a block",
-                                           cdi::VBAND_CPY * cdi::VBAND_NT / 5);
+        return cdi::set_error(CDI_ERR_ARG, "batch tile 6 needs rows of at most %d cells, at most 65535 boxes and "
+                                           "band slots that fit in the shared memory of a block", 100 * VX);
     cudaError_t e;
     if (vband && !b->padbuf) {  // the padded copies: state x 2, u, v, w per box
         size_t n = 0;

@@ -16,7 +16,7 @@
 //     ring slots, so a shared access is one base register and an immediate;
 //   - 14 rows and one ring warp make a block of 8 warps, two of which per SM leave each
 //     thread 128 registers (10 warps per block left it 96, and the carried values spilled).
-// FP32, aligned rows: 102.5 -> 80.1 instructions per cell; 256^3 72.4 -> 57.4 us per step of a
+// FP32, aligned rows: 102.5 -> 82.3 instructions per cell; 256^3 72.4 -> 57.4 us per step of a
 // run (4.63 -> 5.84 TB/s), 512^3 516 -> 420 us (5.20 -> 6.39 TB/s).
 //
 //   A = VX  (AL) rows start on 16-byte boundaries (nx % VX == 0): 16-byte cp.async and stores.

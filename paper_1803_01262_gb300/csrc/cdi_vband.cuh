@@ -25,7 +25,8 @@
 // What bounds it: latency (16 warps per SM, one barrier per plane; 54% of the issue slots, the L1
 // data pipe at 55%, DRAM at 50% of its rate).  Fewer rows per band, so that no thread has a ring
 // group besides its own, took 20% longer; 512 threads, one block per SM, 10%.  64 FP32 boxes with
-// edges 32..160 (65 M cells): 143 -> 107 instructions per cell, 341 -> 304 us per step of a run;
+// edges 32..160 (65 M cells): 143 -> 107 instructions per cell, 341 -> 304 us per step of a run
+// (another 64, 58.4 M cells, taller bands: 101.8 and 264 us);
 // before, the stores kept ghost cells at both ends of every row, the slots lay at run-time offsets,
 // a condition per thread stood around the update, and its operands were loaded after the
 // sharpening.  The output goes to the padded copy of the next state and, on the last step of a call

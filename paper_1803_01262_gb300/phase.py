@@ -61,7 +61,7 @@ def phase_diagram(points, n=50, nsteps=None, dtype=torch.float64, device="cuda",
     sufficient condition as ``cdi.check_condition`` reads it: Eq. 17 with U
     the largest face-velocity component, and A <= 1/(2 D_f)); and the run's
     step count, cells, batch launch configuration, the batch itself and the
-    run's device time (run_ms, CUDA events around the graph replay).
+    run's device time (run_ms, CUDA events around it).
     ``sharpen="face"`` runs every box with the face-product sharpening instead of
     Section 2.2's centre form (the boundedness proof covers the centre form only).
     """
